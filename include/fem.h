@@ -21,7 +21,7 @@
  *    fem_integrate_laplacian_host). No entry point allocates device memory for data or
  *    synchronises the stream: work is enqueued on `stream` (0 = the legacy default
  *    stream) and the call returns after the launch. The one exception is
- *    fem_pcg_laplacian, which waits for its result and runs its loop as a CUDA graph.
+ *    the fem_pcg_* solves, which wait for their result.
  *  - Outside stream capture the integration, adjoint, geometry and assembly kernels are
  *    launched with programmatic stream serialisation (programmatic dependent launch):
  *    a kernel may be scheduled onto the GPU while the kernel before it on `stream`
@@ -262,8 +262,8 @@ fem_status fem_integrate_laplacian_transposed(int dim, int64_t n_cells, const vo
                                               fem_precision prec, fem_stream stream);
 
 /* ---------------------------------------------------------------------------------
- * fem_pcg_laplacian -- solve A x = b with a matrix-free Jacobi-preconditioned conjugate
- * gradient, A the assembled operator of Eq. 2 for the variable-coefficient Laplacian
+ * fem_pcg_laplacian -- solve A x = b with a Jacobi-preconditioned conjugate gradient, A the
+ * assembled operator of Eq. 2 for the variable-coefficient Laplacian
  * (element residuals of fem_integrate_laplacian summed per vertex, E^T r_e(x)), not in
  * the paper. Vertices with fixed[v] != 0 are Dirichlet vertices: they keep the value
  * that x holds on entry, and the system is solved on the other vertices.
@@ -275,17 +275,24 @@ fem_status fem_integrate_laplacian_transposed(int dim, int64_t n_cells, const vo
  *   max_iter, rtol       stop when ||r||_2 <= rtol ||r_0||_2 or after max_iter iterations
  *   work       caller-owned device workspace of fem_pcg_work_bytes() bytes, 256-byte aligned
  *   iters_out, resid_out (host, may be NULL) iterations taken and ||r|| / ||r_0||
- * Value arrays are float64 for FEM_FP64 and FEM_FP64_DF (the residual then runs in the
- * double-float form: float64-class accuracy at float32-pipe speed) and float32 otherwise;
- * dot products accumulate in float64 in a fixed order (reproducible). The iteration is CG
- * in Chronopoulos and Gear's form (both inner products of an iteration from one reduction:
- * 3 kernels per iteration). The iterations run on the device as a CUDA graph with a WHILE
- * node (one iteration captured as its body, the condition set by the body's last kernel),
- * so the host does not wait per iteration;
- * unlike the other entry points this one returns only after the solve: it synchronises
- * `stream` twice (initial residual norm, final iteration count). The loop body is
- * captured on a library-owned stream per device, one capture at a time (a lock), so
- * calls from several host threads are safe.
+ * Value arrays are float64 for FEM_FP64 and FEM_FP64_DF and float32 otherwise; dot products
+ * accumulate in float64 (float32 vectors: in float32 pairs) in a fixed order (reproducible on
+ * one device). The iteration is CG in Chronopoulos and Gear's form.
+ * With fem_pcg_work_bytes() of workspace the operator's rows are assembled on the device at
+ * the start of the solve, from element matrices in prec's geometry (FEM_FP64_DF: float64), and
+ * the whole loop runs in one kernel, which occupies the device until the solve ends; other
+ * streams' kernels run before or after it. A smaller workspace is accepted down to what the
+ * element form needs ((dim+1) n_cells values, six vectors of n_verts values, 24 KiB and 256
+ * bytes, each rounded up to 256 bytes); the element residuals are then computed and summed in
+ * every iteration, as three kernels in a CUDA graph with a WHILE node, at several times the
+ * cost (FEM_FP64_DF: in the double-float form). So are meshes with a vertex of more than 64
+ * neighbours or more vertex pairs than the workspace provides for (half as many again as a
+ * conforming mesh of this size has), and matrices past 32 GiB.
+ * Unlike the other entry points this one returns only after the solve: it synchronises
+ * `stream` (once; in element form twice). The element form's loop body is captured on a
+ * library-owned stream per device, one capture at a time (a lock), so calls from several host
+ * threads are safe. FEM_ERR_TIMEOUT: the loop kernel's bounded waits gave up (x is then
+ * unspecified).
  * ------------------------------------------------------------------------------- */
 int64_t fem_pcg_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec);
 fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -325,8 +332,10 @@ fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_verts, const d
  *              aligned (holds the float32 solve's workspace, K in float32, the float64 residual)
  *   outer_out, inner_out, resid_out (host, may be NULL): corrections made, float32 PCG
  *              iterations in all, ||r|| / ||r_0|| of the returned x
- * Synchronises `stream` once per outer step (the residual norm) and as fem_pcg_laplacian
- * does inside each correction; returns when the solve has finished.
+ * The corrections take fem_pcg_laplacian's assembled form with fem_pcg_refined_work_bytes() of
+ * workspace (the matrix is formed once for all of them), its element form with less (down to
+ * the same without the matrix). Synchronises `stream` once per outer step (the residual norm)
+ * and as fem_pcg_laplacian does inside each correction; returns when the solve has finished.
  * ------------------------------------------------------------------------------- */
 int64_t fem_pcg_refined_work_bytes(int dim, int64_t n_cells, int64_t n_verts, int n_q);
 int64_t fem_pcg_elasticity_refined_work_bytes(int dim, int64_t n_cells, int64_t n_verts, int n_q);

@@ -1,21 +1,24 @@
-// fem_solver.cu -- matrix-free Jacobi-preconditioned conjugate-gradient solves with the
-// assembled operators of Eq. 2: A v = E^T r_e(v), the element residuals of the
-// variable-coefficient Laplacian or of linear elasticity summed into the vertices through
-// the vertex-to-cell lists (fem_build_node2cell). Dirichlet vertices keep their value from
-// the initial x. Also: mixed-precision iterative refinement around the FP32-mixed solve.
+// fem_solver.cu -- Jacobi-preconditioned conjugate-gradient solves with the assembled
+// operators of Eq. 2: A v = E^T r_e(v), the element residuals of the variable-coefficient
+// Laplacian or of linear elasticity summed into the vertices through the vertex-to-cell lists
+// (fem_build_node2cell). Dirichlet vertices keep their value from the initial x. Also:
+// mixed-precision iterative refinement around the FP32-mixed solve.
 //
-// Kernels here: the assembled diagonals (element stiffness diagonals summed per vertex), a
-// deterministic two-level dot product, and the CG iteration in Chronopoulos and Gear's form
-// with its scalars kept in device memory. The iteration loop runs on the device: one CG
-// iteration is captured once into the body of a CUDA graph WHILE node, and the last kernel
-// of the body counts the iteration and sets the loop condition (not converged and fewer
-// than max_iter iterations). The host synchronises twice per solve (the initial residual
-// norm, the final count) instead of once per iteration.
+// The iteration is CG in Chronopoulos and Gear's form. A solve takes one of two forms:
+//   * assembled: the operator's rows are formed once on the device (fem_sell.cuh) and the
+//     whole loop runs in one cooperative kernel (sell_cg_kernel). Taken whenever the caller's
+//     workspace has room for the matrix.
+//   * element form: each application is the residual kernel and the vertex sum; one iteration
+//     is captured into the body of a CUDA graph WHILE node. For workspaces without room for
+//     the matrix, meshes whose rows do not fit it, and device partitions that refuse the
+//     cooperative launch.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
 #include "fem_cell.cuh"
+#include "fem_sell.cuh"
 
 namespace fem {
 
@@ -142,9 +145,11 @@ __global__ void __launch_bounds__(256) dot_final_kernel(const double *partial, d
 
 // scalars[] layout: 0 gamma = r.u, 1 delta = w.u, 2 alpha, 3 beta, 4 rr = r.r,
 // 5 (rtol ||r_0||)^2, 6 iterations done, 7 the 32-bit block counter of the reduction
-// (last_block), 8 alpha and beta rounded to float32 once (read by the float32 update)
+// (last_block), 8 alpha and beta rounded to float32 once (read by the float32 update), 9 r.r
+// before the first iteration, 10 the assembled matrix' two 32-bit state words
+// (SellMatrix::state), 11 the grid barrier's counter and its timeout flag
 enum { S_GAMMA = 0, S_DELTA = 1, S_ALPHA = 2, S_BETA = 3, S_RR = 4, S_TOL2 = 5, S_ITER = 6, S_TICKETS = 7,
-       S_AB32 = 8, S_COUNT = 9 };
+       S_AB32 = 8, S_RR0 = 9, S_MATRIX = 10, S_BARRIER = 11, S_COUNT = 12 };
 
 __device__ __forceinline__ unsigned *tickets(double *sc) { return reinterpret_cast<unsigned *>(sc + S_TICKETS); }
 
@@ -166,14 +171,14 @@ __device__ __forceinline__ void block_sum256x3(double (&v)[3], double *sh) {
 }
 
 // True in the block that finishes last: each block's thread 0 publishes the block's partial
-// sums (fence), then takes a ticket; the block holding ticket kDotBlocks - 1 sees every
+// sums (fence), then takes a ticket; the block holding the last of `blocks` tickets sees every
 // partial and reduces them in place of a separate one-block kernel (the order of the sum
 // does not depend on which block that is), then resets the counter for the next iteration.
-__device__ __forceinline__ bool last_block(unsigned *ticket) {
+__device__ __forceinline__ bool last_block(unsigned *ticket, unsigned blocks) {
     __shared__ bool s_last;
     if (threadIdx.x == 0) {
         __threadfence();
-        s_last = atomicAdd(ticket, 1u) == unsigned(kDotBlocks - 1);
+        s_last = atomicAdd(ticket, 1u) == blocks - 1u;
     }
     __syncthreads();
     return s_last;
@@ -233,6 +238,7 @@ struct PairSum {
         hi = s;
         lo += t + l;
     }
+    __device__ __forceinline__ void merge(const PairSum &o) { merge(o.hi, o.lo); }
     __device__ __forceinline__ double value() const { return static_cast<double>(hi) + static_cast<double>(lo); }
 };
 
@@ -292,6 +298,33 @@ __global__ void cg_update_kernel(int64_t N, const double *sc, const T *w, const 
         r[i] = ri;
         u[i] = ri * Dinv[i];
     }
+}
+
+// The end of an iteration, by one thread: gamma, delta and rr, the next alpha and beta, the
+// iteration count and the loop condition (INIT, before the loop: alpha and beta only).
+template <bool INIT>
+__device__ __forceinline__ void cg_scalars(double *sc, double gamma, double delta, double rrs, int max_iter,
+                                           cudaGraphConditionalHandle loop) {
+    if constexpr (INIT) {
+        sc[S_ALPHA] = delta != 0.0 ? gamma / delta : 0.0;
+        sc[S_BETA] = 0.0;
+    } else {
+        const double g0 = sc[S_GAMMA], a_old = sc[S_ALPHA];
+        const double beta = g0 != 0.0 ? gamma / g0 : 0.0;
+        const double den = a_old != 0.0 ? delta - beta * gamma / a_old : delta;
+        sc[S_BETA] = beta;
+        sc[S_ALPHA] = den != 0.0 ? gamma / den : 0.0;
+        const double it = sc[S_ITER] + 1.0;
+        sc[S_ITER] = it;
+        const bool more = it < static_cast<double>(max_iter) && rrs > sc[S_TOL2] && rrs > 0.0;
+        cudaGraphSetConditional(loop, more ? 1u : 0u);
+    }
+    *reinterpret_cast<float2 *>(sc + S_AB32) =
+        make_float2(static_cast<float>(sc[S_ALPHA]), static_cast<float>(sc[S_BETA]));
+    sc[S_GAMMA] = gamma;
+    sc[S_DELTA] = delta;
+    sc[S_RR] = rrs;
+    tickets(sc)[0] = 0u;
 }
 
 // w = A u: the element vectors of u summed per vertex in list order (as the nodal gather
@@ -364,7 +397,7 @@ __global__ void __launch_bounds__(256) cg_apply_dots_kernel(int64_t C, int64_t V
         block_merge256x3(pd, sh2);
         if (threadIdx.x == 0)
             for (int m = 0; m < 3; ++m) pp[m * kDotBlocks + blockIdx.x] = make_float2(pd[m].hi, pd[m].lo);
-        if (!last_block(tickets(sc))) return;
+        if (!last_block(tickets(sc), kDotBlocks)) return;
         PairSum at[3];
         for (int i = threadIdx.x; i < kDotBlocks; i += 256)
 #pragma unroll
@@ -379,7 +412,7 @@ __global__ void __launch_bounds__(256) cg_apply_dots_kernel(int64_t C, int64_t V
         block_sum256x3(t, sh);
         if (threadIdx.x == 0)
             for (int m = 0; m < 3; ++m) partial[m * kDotBlocks + blockIdx.x] = t[m];
-        if (!last_block(tickets(sc))) return;
+        if (!last_block(tickets(sc), kDotBlocks)) return;
         double at[3] = {0.0, 0.0, 0.0};
         for (int i = threadIdx.x; i < kDotBlocks; i += 256)
 #pragma unroll
@@ -387,28 +420,458 @@ __global__ void __launch_bounds__(256) cg_apply_dots_kernel(int64_t C, int64_t V
         block_sum256x3(at, sh);
         gamma = at[0], delta = at[1], rrs = at[2];
     }
-    if (threadIdx.x == 0) {
-        if constexpr (INIT) {
-            sc[S_ALPHA] = delta != 0.0 ? gamma / delta : 0.0;
-            sc[S_BETA] = 0.0;
-        } else {
-            const double g0 = sc[S_GAMMA], a_old = sc[S_ALPHA];
-            const double beta = g0 != 0.0 ? gamma / g0 : 0.0;
-            const double den = a_old != 0.0 ? delta - beta * gamma / a_old : delta;
-            sc[S_BETA] = beta;
-            sc[S_ALPHA] = den != 0.0 ? gamma / den : 0.0;
-            const double it = sc[S_ITER] + 1.0;
-            sc[S_ITER] = it;
-            const bool more = it < static_cast<double>(max_iter) && rrs > sc[S_TOL2] && rrs > 0.0;
-            cudaGraphSetConditional(loop, more ? 1u : 0u);
+    if (threadIdx.x == 0) cg_scalars<INIT>(sc, gamma, delta, rrs, max_iter, loop);
+}
+
+// ------------------------------------------------------------------ the whole loop from the assembled matrix
+//
+// One cooperative launch per solve, one CTA per SM: every CTA owns a contiguous range of
+// slices, a warp takes one slice at a time, and the thread that computes a row's entries of w
+// also updates these entries of the vectors. An iteration is the vector update, a grid barrier
+// (u is read by other CTAs' rows), the rows of w = A u with the sum w.u, and a second barrier
+// for the CTAs' partial sums, which every CTA then adds up in the same order, so that all hold
+// the same alpha, beta and stopping decision. Nothing returns to the host before the end.
+// While they fit, a CTA's part of the matrix stays in its shared memory and a thread's entries
+// of the vectors in its registers for the whole solve; then only u and the partial sums move.
+//
+// Measured per iteration (64^3 x 6 tets, 274,625 rows; elasticity on 511,104 tets, 273,375
+// unknowns): float32 Laplacian 11.1 us against 52 us in element form, float64 27 against 255
+// us, float32 elasticity 15.3 against 38 us, float64 41 us. As two kernels per iteration in a
+// graph the same rows took 19, 37, 27 and 79 us: the launches' drain and the loop node cost
+// more than the barriers. What bounds it: float64, the float64 pipe (a subtraction and an FMA
+// per entry: 14 of the 27 us, the sums and updates 5); float32, latency: two barriers of about
+// 2 us, the gathers of u through L2 after each (5 us), the scalars (1 us). The rows' threads
+// handle all components of a block (a thread per component read every column and nodal value
+// NC times: 21 us), 512 threads with four slices a warp hold the vectors without spills (1024
+// threads at 64 registers spilled, and a spill is reloaded from L2, because each barrier
+// invalidates L1).
+//
+// The kernel occupies the device until the solve ends. The sums' order is fixed by the row
+// count and the device's SM count.
+
+constexpr int kCgMaxBlocks = 1024;  // partial sums provided for
+constexpr int kCgTable = 1024;      // slices per CTA whose place is kept in shared memory
+// threads of a CTA, and the slices per warp whose vector entries stay in registers: the row
+// product wants some 60 registers beside 7 NC values per slice
+template <int NC>
+constexpr int cg_threads() { return NC == 1 ? 512 : 640; }
+template <int NC>
+constexpr int cg_units() { return NC == 1 ? 4 : 1; }
+constexpr int kCgThreads = 640;  // the most of them
+
+template <class T>
+struct CgArgs {
+    int64_t V;
+    const int32_t *cols;
+    const T *vals;
+    const int2 *slice;
+    const T *b, *Dinv;  // b: nullptr for zero
+    const uint8_t *fixed;
+    T *x, *r, *u, *p, *s, *w;
+    double *partial;  // [3][kCgMaxBlocks] sums (float32: pairs)
+    double *sc;
+    double rtol;
+    int max_iter;
+    int cache_slots;  // matrix slots that fit in the launch's dynamic shared memory
+    unsigned *err;
+};
+
+// A bounded wait of one thread until the barrier's counter *p has reached `target`; what the
+// other CTAs wrote before they arrived is visible afterwards. CTAs that wait for one another
+// are resident together (cooperative launch), so the wait ends unless a CTA is lost; after
+// kCgWaitNs it records a timeout and returns false, as the other CTAs' then do.
+constexpr uint64_t kCgWaitNs = 4000000000ull;
+__device__ __forceinline__ bool wait_reached(const unsigned *p, unsigned target, unsigned *gave_up, unsigned *err) {
+    uint64_t t0 = 0, t = 0;
+    unsigned spins = 0;
+    for (;;) {
+        unsigned seen;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(p) : "memory");
+        if (static_cast<int>(seen - target) >= 0) return true;
+        if ((++spins & 255u) == 0u) {
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            if (t - t0 > kCgWaitNs) {
+                atomicExch(gave_up, 1u);
+                record_device_error(err, FEM_DEVERR_TIMEOUT);
+                return false;
+            }
         }
-        *reinterpret_cast<float2 *>(sc + S_AB32) =
-            make_float2(static_cast<float>(sc[S_ALPHA]), static_cast<float>(sc[S_BETA]));
-        sc[S_GAMMA] = gamma;
-        sc[S_DELTA] = delta;
-        sc[S_RR] = rrs;
-        tickets(sc)[0] = 0u;
     }
+}
+
+// The totals of M values per thread over the block (any multiple of 32 threads), in thread 0.
+// float64: a shared-memory tree over the warps, lane by lane, then one over the lanes of warp 0
+// (the float64 pipe does two lanes a clock, and a tree in every warp would cost it five times
+// the additions); float32 pairs: warp trees, then one over the warps.
+template <int M>
+struct BlockSums {
+    double d[M][kCgThreads];
+};
+template <int M>
+__device__ __forceinline__ void block_totals(double (&v)[M], BlockSums<M> &sh) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) sh.d[m][threadIdx.x] = v[m];
+    __syncthreads();
+    int n = blockDim.x;
+    for (; n > 32;) {
+        const int half = (n / 32 + 1) / 2 * 32;
+        if (threadIdx.x + half < n)
+#pragma unroll
+            for (int m = 0; m < M; ++m) sh.d[m][threadIdx.x] += sh.d[m][threadIdx.x + half];
+        n = half;
+        __syncthreads();
+    }
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int m = 0; m < M; ++m) v[m] = sh.d[m][threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int m = 0; m < M; ++m) v[m] += __shfl_down_sync(0xffffffffu, v[m], o);
+    }
+}
+template <int M>
+struct BlockPairs {
+    float2 p[M][32];
+};
+template <int M>
+__device__ __forceinline__ void block_totals(PairSum (&a)[M], BlockPairs<M> &sh) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        warp_merge(a[m]);
+        if (lane == 0) sh.p[m][threadIdx.x >> 5] = make_float2(a[m].hi, a[m].lo);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            PairSum b;
+            if (lane < blockDim.x / 32) b.hi = sh.p[m][lane].x, b.lo = sh.p[m][lane].y;
+            warp_merge(b);
+            a[m] = b;
+        }
+    }
+}
+
+// one entry of the iteration's vectors
+template <class T>
+struct CgEntry {
+    T x, r, u, p, s, w, d;
+};
+
+// a running inner product: float64, or a float32 pair
+struct Sum64 {
+    double v = 0.0;
+    __device__ __forceinline__ void add_prod(double a, double b) { v = fma(a, b, v); }
+    __device__ __forceinline__ void merge(Sum64 o) { v += o.v; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+__device__ __forceinline__ void warp_merge(Sum64 &a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a.v += __shfl_down_sync(0xffffffffu, a.v, o);
+}
+
+// U > 0: at most U slices per warp, their vector entries kept in registers; U = 0: any number,
+// the vectors in memory.
+template <int NC, class T, int U>
+__global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __grid_constant__ CgArgs<T> a) {
+    constexpr bool F32 = std::is_same<T, float>::value;
+    constexpr int BB = NC * NC;
+    using Sum = typename std::conditional<F32, PairSum, Sum64>::type;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ typename std::conditional<F32, BlockPairs<2>, BlockSums<2>>::type sh2;
+    __shared__ typename std::conditional<F32, BlockPairs<1>, BlockSums<1>>::type sh1;
+    __shared__ int2 s_slice[kCgTable];  // place (in shared memory, if cached) and length of the CTA's first slices
+    __shared__ int s_cached;
+    __shared__ Sum s_part[3 * ((kCgMaxBlocks + 31) / 32)];
+    __shared__ T s_alpha, s_beta;
+    __shared__ int s_ok, s_more;
+    unsigned *state = reinterpret_cast<unsigned *>(a.sc + S_MATRIX), *bar = reinterpret_cast<unsigned *>(a.sc + S_BARRIER);
+    if (state[1] != 0u) return;  // the matrix did not fit: the host takes the element form
+    const int64_t V = a.V;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int64_t slices = (V + 31) / 32;
+    const int64_t s0 = slices * blockIdx.x / gridDim.x, s1 = slices * (blockIdx.x + 1) / gridDim.x;
+    const int nslices = static_cast<int>(s1 - s0);
+
+    // the CTA's first slices into shared memory, as many as fit
+    int32_t *scols = reinterpret_cast<int32_t *>(dyn);
+    T *svals = reinterpret_cast<T *>(dyn + size_t(a.cache_slots) * 32 * sizeof(int32_t));
+    const int ntab = min(nslices, kCgTable);
+    for (int t = threadIdx.x; t < ntab; t += blockDim.x) s_slice[t] = a.slice[s0 + t];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int used = 0, t = 0;
+        for (; t < ntab && used + s_slice[t].y <= a.cache_slots; ++t) used += s_slice[t].y;
+        s_cached = t;
+    }
+    __syncthreads();
+    const int cached = s_cached;
+    {
+        int used = 0, t0 = 0;
+        for (int t = warp; t < cached; t += nw) {
+            for (; t0 < t; ++t0) used += s_slice[t0].y;
+            const int2 g = a.slice[s0 + t];
+            for (int q = 0; q < g.y; ++q) {
+                scols[(used + q) * 32 + lane] = ld_matrix(a.cols + (int64_t(g.x) + q) * 32 + lane);
+#pragma unroll
+                for (int m = 0; m < BB; ++m)
+                    svals[((used + q) * BB + m) * 32 + lane] = ld_matrix(a.vals + ((int64_t(g.x) + q) * BB + m) * 32 + lane);
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int used = 0;
+        for (int t = 0; t < cached; ++t) s_slice[t].x = used, used += s_slice[t].y;
+    }
+    __syncthreads();
+
+    // (A v) in the row n of the CTA's slice t
+    auto product = [&](const T *v, int t, int64_t n, T (&w)[NC]) {
+        if (t < cached) sell_row<NC, T, true>(scols, svals, s_slice[t], lane, n, v, V, w);
+        else sell_row<NC, T, false>(a.cols, a.vals, t < kCgTable ? s_slice[t] : a.slice[s0 + t], lane, n, v, V, w);
+    };
+    // f(entries, slice of the CTA, row, whether the row exists) for each of this thread's rows;
+    // in memory: `in` names the members read first, `out` those written after
+    enum { MX = 1, MR = 2, MU = 4, MP = 8, MS = 16, MW = 32, MD = 64 };
+    CgEntry<T> own[U > 0 ? U : 1][NC];
+    auto rows = [&](auto in, auto out, auto f) {
+        if constexpr (U > 0) {
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                const int t = warp + j * nw;
+                if (t < nslices) {
+                    const int64_t n = (s0 + t) * 32 + lane;
+                    f(own[j], t, min(n, V - 1), n < V);
+                }
+            }
+        } else {
+            constexpr int I = decltype(in)::value, O = decltype(out)::value;
+            for (int t = warp; t < nslices; t += nw) {
+                const int64_t n = (s0 + t) * 32 + lane, row = min(n, V - 1);
+                CgEntry<T> e[NC];
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    const int64_t i = k * V + row;
+                    e[k] = CgEntry<T>{};
+                    if (I & MX) e[k].x = a.x[i];
+                    if (I & MR) e[k].r = a.r[i];
+                    if (I & MU) e[k].u = a.u[i];
+                    if (I & MP) e[k].p = a.p[i];
+                    if (I & MS) e[k].s = a.s[i];
+                    if (I & MW) e[k].w = a.w[i];
+                    if (I & MD) e[k].d = a.Dinv[i];
+                }
+                f(e, t, row, n < V);
+                if (n < V) {
+#pragma unroll
+                    for (int k = 0; k < NC; ++k) {
+                        const int64_t i = k * V + row;
+                        if (O & MX) a.x[i] = e[k].x;
+                        if (O & MR) a.r[i] = e[k].r;
+                        if (O & MP) a.p[i] = e[k].p;
+                        if (O & MS) a.s[i] = e[k].s;
+                        if (O & MW) a.w[i] = e[k].w;
+                    }
+                }
+            }
+        }
+    };
+    // r = b - A x on the free vertices (0 on fixed ones), u = D^-1 r, p = s = 0, with r.u and r.r
+    Sum sums[2], wu[1];
+    rows(std::integral_constant<int, MX | MD>(), std::integral_constant<int, MR | MP | MS>(),
+         [&](CgEntry<T> (&e)[NC], int t, int64_t n, bool in) {
+             T ax[NC];
+             product(a.x, t, n, ax);
+             const bool held = !in || a.fixed[n];
+#pragma unroll
+             for (int k = 0; k < NC; ++k) {
+                 const int64_t i = k * V + n;
+                 if constexpr (U > 0) e[k].x = a.x[i], e[k].d = a.Dinv[i];
+                 e[k].r = held ? T(0) : (a.b ? a.b[i] : T(0)) - ax[k];
+                 e[k].u = e[k].r * e[k].d;
+                 e[k].p = e[k].s = T(0);
+                 if (in) a.u[i] = e[k].u;
+                 sums[0].add_prod(e[k].r, e[k].u), sums[1].add_prod(e[k].r, e[k].r);
+             }
+         });
+    double inv_gamma = 0.0, inv_ga = 0.0, rr = 0.0, rr0 = 0.0, tol2 = 0.0;  // in thread 0
+    int it = 0;
+    // the grid's barrier, in two halves: what the CTA has written before it arrives is visible
+    // to every CTA that has waited
+    unsigned arrivals = 0;
+    auto barrier_arrive = [&]() -> unsigned {
+        __syncthreads();
+        arrivals += gridDim.x;
+        if (threadIdx.x == 0) {
+            asm volatile("fence.acq_rel.gpu;\n\tred.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        }
+        return arrivals;
+    };
+    auto barrier_wait = [&](unsigned target) -> bool {
+        if (threadIdx.x == 0) {
+            s_ok = wait_reached(bar, target, bar + 1, a.err);
+        }
+        __syncthreads();
+        return s_ok != 0;
+    };
+    for (;;) {
+        // all CTAs' entries of u are in memory; the sums over them are formed while waiting
+        const unsigned here = barrier_arrive();
+        if constexpr (F32) {
+            block_totals(sums, sh2);
+        } else {
+            double v[2] = {sums[0].v, sums[1].v};
+            block_totals(v, sh2);
+            sums[0].v = v[0], sums[1].v = v[1];
+        }
+        const Sum ru = sums[0], rsq = sums[1];  // totals, in thread 0
+        if (!barrier_wait(here)) return;
+        // w = A u and w.u
+        wu[0] = Sum();
+        rows(std::integral_constant<int, MU>(), std::integral_constant<int, MW>(),
+             [&](CgEntry<T> (&e)[NC], int t, int64_t n, bool in) {
+                 T w[NC];
+                 product(a.u, t, n, w);
+#pragma unroll
+                 for (int k = 0; k < NC; ++k) {
+                     e[k].w = w[k];
+                     if (in) wu[0].add_prod(w[k], e[k].u);
+                 }
+             });
+        if constexpr (F32) {
+            block_totals(wu, sh1);
+        } else {
+            double v[1] = {wu[0].v};
+            block_totals(v, sh1);
+            wu[0].v = v[0];
+        }
+        // publish this CTA's sums, wait for all CTAs', and add them up: warp m the sums of value m
+        if (threadIdx.x == 0) {
+            const Sum mine[3] = {ru, wu[0], rsq};
+            for (int m = 0; m < 3; ++m) {
+                if constexpr (F32)
+                    reinterpret_cast<float2 *>(a.partial)[m * kCgMaxBlocks + blockIdx.x] = make_float2(mine[m].hi, mine[m].lo);
+                else
+                    a.partial[m * kCgMaxBlocks + blockIdx.x] = mine[m].v;
+            }
+        }
+        if (!barrier_wait(barrier_arrive())) return;
+        const int chunks = (gridDim.x + 31) / 32;  // warp c + chunks m: 32 CTAs' sums of value m
+        for (int t = warp; t < 3 * chunks; t += nw) {
+            const int m = t / chunks, i = (t - m * chunks) * 32 + lane;
+            Sum v;
+            if (i < gridDim.x) {
+                if constexpr (F32) {
+                    const float2 q = __ldcg(reinterpret_cast<const float2 *>(a.partial) + m * kCgMaxBlocks + i);
+                    v.hi = q.x, v.lo = q.y;
+                } else {
+                    v.v = __ldcg(a.partial + m * kCgMaxBlocks + i);
+                }
+            }
+            warp_merge(v);
+            if (lane == 0) s_part[t] = v;
+        }
+        __syncthreads();
+        // the scalars by one thread (their divisions in every thread would keep the float64 pipe
+        // busy for 10 us), with one division between the sums and alpha:
+        //     beta = gamma' / gamma,  alpha = gamma' / (delta - beta gamma' / alpha_old)
+        double total = 0.0;
+        if (threadIdx.x < 32) {
+            if (lane < 3) {
+                Sum v = s_part[lane * chunks];
+                for (int c = 1; c < chunks; ++c) v.merge(s_part[lane * chunks + c]);
+                total = v.value();
+            }
+            rr = __shfl_sync(0xffffffffu, total, 2);
+        }
+        const double delta = __shfl_sync(0xffffffffu, total, 1);
+        if (threadIdx.x == 0) {
+            const double g = total;
+            double beta = 0.0, den = delta;
+            if (it == 0) {
+                rr0 = rr;
+                const double tol = a.rtol * sqrt(rr0);
+                tol2 = tol * tol;
+            } else {
+                beta = g * inv_gamma;
+                den = delta - g * g * inv_ga;
+            }
+            const double alpha = den != 0.0 ? copysign(quot_abs(g, den), den) : 0.0;
+            inv_gamma = g != 0.0 ? copysign(quot_abs(1.0, g), g) : 0.0;
+            inv_ga = den * inv_gamma * inv_gamma;  // 1 / (gamma alpha)
+            s_alpha = static_cast<T>(alpha), s_beta = static_cast<T>(beta);
+            // a NaN residual ends the loop: every comparison with it is false
+            s_more = it < a.max_iter && rr > tol2 && rr > 0.0;
+        }
+        __syncthreads();
+        if (!s_more) break;
+        ++it;
+        // p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s, u = D^-1 r
+        const T al = s_alpha, be = s_beta;
+        sums[0] = sums[1] = Sum();
+        rows(std::integral_constant<int, MX | MR | MU | MP | MS | MW | MD>(),
+             std::integral_constant<int, MX | MR | MP | MS>(), [&](CgEntry<T> (&e)[NC], int, int64_t n, bool in) {
+#pragma unroll
+                 for (int k = 0; k < NC; ++k) {
+                     e[k].p = e[k].u + be * e[k].p;
+                     e[k].s = e[k].w + be * e[k].s;
+                     e[k].x += al * e[k].p;
+                     e[k].r -= al * e[k].s;
+                     e[k].u = e[k].r * e[k].d;
+                     if (in) {
+                         a.u[k * V + n] = e[k].u;
+                         sums[0].add_prod(e[k].r, e[k].u), sums[1].add_prod(e[k].r, e[k].r);
+                     }
+                 }
+             });
+    }
+    if constexpr (U > 0) {
+        rows(std::integral_constant<int, 0>(), std::integral_constant<int, 0>(),
+             [&](CgEntry<T> (&e)[NC], int, int64_t n, bool in) {
+#pragma unroll
+                 for (int k = 0; k < NC; ++k)
+                     if (in) a.x[k * V + n] = e[k].x;
+             });
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.sc[S_RR] = rr;
+        a.sc[S_RR0] = rr0;
+        a.sc[S_ITER] = it;
+    }
+}
+
+// Launch sell_cg_kernel: one CTA per SM at most, four slices each while they last (fewer CTAs
+// make the barriers cheaper, more spread the rows' latency), a warp per slice up to the CTA's
+// limit.
+template <int NC, class T>
+static cudaError_t launch_sell_cg(CgArgs<T> a, cudaStream_t s) {
+    constexpr int U = cg_units<NC>(), kWarps = cg_threads<NC>() / 32;
+    const int64_t slices = (a.V + 31) / 32;
+    const int grid = slices <= kWarps ? 1 : static_cast<int>(std::min<int64_t>({(slices + 3) / 4, int64_t(sm_count()), int64_t(kCgMaxBlocks)}));
+    const int64_t per = (slices + grid - 1) / grid;  // the largest range of a CTA
+    const int64_t rounds = (per + kWarps - 1) / kWarps;
+    const int threads = static_cast<int>((per + rounds - 1) / rounds * 32);
+    const bool resident = rounds <= U;
+    const void *k = resident ? reinterpret_cast<const void *>(sell_cg_kernel<NC, T, U>)
+                             : reinterpret_cast<const void *>(sell_cg_kernel<NC, T, 0>);
+    // shared memory for the matrix: what the static part leaves, in whole slots
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, k);
+    if (e != cudaSuccess) return e;
+    const size_t slot = 32 * (sizeof(int32_t) + size_t(NC) * NC * sizeof(T));
+    const size_t room = 227 * 1024 - at.sharedSizeBytes;
+    const int64_t most = per * kSellMaxRow;  // slots the CTA's slices can have
+    a.cache_slots = static_cast<int>(std::min<int64_t>(int64_t(room / slot), most));
+    const size_t smem = size_t(a.cache_slots) * slot;
+    // (the same value on every call: calls on other host threads may be between here and their launch)
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(room));
+    if (e != cudaSuccess) return e;
+    void *args[] = {&a};
+    return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(threads), args, smem, s);
 }
 
 __global__ void loop_init_kernel(double *sc, double tol2) {
@@ -445,9 +908,15 @@ static size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 struct Workspace {
     void *elem, *D, *r, *z, *p, *q, *sv;  // D holds D^-1, z holds u = D^-1 r, q holds w = A u, sv s = A p
     double *partial, *scalars;
+    SellMatrix mat;  // the assembled operator (mat.cols: nullptr where the workspace has no room for it)
+    double *mat_partial;
 };
 
-static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Workspace *w, int ncomp = 1) {
+// The assembled operator is provided for up to kMatrixMaxBytes of workspace; beyond that (3D:
+// some 600 M cells for the Laplacian, 70 M for elasticity in float64) the solve runs in element form.
+constexpr size_t kMatrixMaxBytes = size_t(32) << 30;
+
+static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Workspace *w, int ncomp, bool matrix) {
     size_t off = 0;
     char *b = static_cast<char *>(base);
     auto take = [&](size_t bytes) {
@@ -461,7 +930,22 @@ static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Worksp
     void *p = take(N * vs), *q = take(N * vs), *sv = take(N * vs);
     double *partial = static_cast<double *>(take(sizeof(double) * 3 * kDotBlocks));
     double *scalars = static_cast<double *>(take(sizeof(double) * S_COUNT));
-    if (w) *w = Workspace{elem, D, r, z, p, q, sv, partial, scalars};
+    SellMatrix mat;
+    double *mat_partial = nullptr;
+    const int64_t slots = sell_slots(C, V);
+    const size_t bb = size_t(ncomp) * size_t(ncomp);
+    if (matrix && C > 0 && slots < (int64_t(1) << 31) && size_t(slots) * 32 * (4 + bb * vs) <= kMatrixMaxBytes) {
+        mat.cap = slots;
+        mat.cols = static_cast<int32_t *>(take(size_t(slots) * 32 * sizeof(int32_t)));
+        mat.vals = take(size_t(slots) * 32 * bb * vs);
+        mat.slice = static_cast<int2 *>(take(size_t((V + 31) / 32) * sizeof(int2)));
+        mat.state = reinterpret_cast<int32_t *>(scalars + S_MATRIX);
+        // the cells' numbers lie in the element vectors' place where they fit there
+        const int nv = sell_cell_values(dim, ncomp);
+        mat.cell = nv <= (dim + 1) * ncomp ? elem : take(size_t(nv) * size_t(C) * vs);
+        mat_partial = static_cast<double *>(take(3 * sizeof(double) * kCgMaxBlocks));
+    }
+    if (w) *w = Workspace{elem, D, r, z, p, q, sv, partial, scalars, mat, mat_partial};
     return off;
 }
 
@@ -472,15 +956,17 @@ struct Operator {
     int ncomp(int dim) const { return physics == 0 ? 1 : dim; }
 };
 
+// what a workspace holds of its operator from an earlier solve of the same call
+enum class Kept { Nothing, Matrix, Diagonal };
+
 template <class T>
 static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, const int32_t *conn,
                           const Operator &op, int n_q, const double *qpts, const double *qw, const int32_t *ptr,
                           const int32_t *idx, const uint8_t *fixed, const void *b, void *x, int max_iter,
                           double rtol, const Workspace &w, int *iters_out, double *resid_out, fem_precision prec,
-                          cudaStream_t s, bool diag_ready = false) {
+                          cudaStream_t s, Kept &kept) {
     // the residual runs in `prec`; every other kernel sees the value type (FEM_FP64_DF
-    // values are float64). diag_ready: w.D already holds the reciprocal of this operator's
-    // diagonal (a repeated solve with the same workspace).
+    // values are float64). kept: what a repeated solve with the same workspace finds there.
     const fem_precision vprec = prec == FEM_FP64_DF ? FEM_FP64 : prec;
     T *X = static_cast<T *>(x);
     T *D = static_cast<T *>(w.D), *r = static_cast<T *>(w.r), *z = static_cast<T *>(w.z);
@@ -492,8 +978,59 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
     QuadW qwt;
     fem_status st = load_quadrature(dim, n_q, qpts, qw, qwt);
     if (st != FEM_OK) return st;
-    // assembled diagonal
-    if (!diag_ready) {
+    // the assembled operator, where the workspace holds it
+    const bool f64 = std::is_same<T, double>::value;
+    T *mvals = static_cast<T *>(w.mat.vals);
+    bool use_matrix = w.mat.cols != nullptr && kept != Kept::Diagonal;
+    auto by_comps = [&](auto go) {
+        if (nc == 1) go(std::integral_constant<int, 1>());
+        else if (nc == 2) go(std::integral_constant<int, 2>());
+        else go(std::integral_constant<int, 3>());
+    };
+    auto assemble = [&]() -> fem_status {
+        unsigned *err = device_error_word();
+        if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
+        const uint32_t V32 = static_cast<uint32_t>(V);
+        const float tau = mixed_tau();
+        T *cell = static_cast<T *>(w.mat.cell);
+        const unsigned rows = static_cast<unsigned>((V + 127) / 128), slices = static_cast<unsigned>((V + 31) / 32);
+        auto cells = [&](auto dimc, auto pc) {
+            constexpr int D_ = decltype(dimc)::value, P_ = decltype(pc)::value;
+            if constexpr (std::is_same<T, val_t<P_>>::value) {
+                if (op.physics == 0) {
+                    auto k = sell_lap_cells_kernel<D_, P_>;
+                    k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(
+                        coords, C, V32, conn, static_cast<const T *>(op.K), qwt, tau * tau, cell, err);
+                } else {
+                    auto k = sell_el_cells_kernel<D_, P_>;
+                    k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(
+                        coords, C, V32, conn, static_cast<const T *>(op.lam), static_cast<const T *>(op.mu), qwt,
+                        tau * tau, cell, err);
+                }
+            }
+        };
+        auto all = [&](auto dimc) {
+            constexpr int D_ = decltype(dimc)::value;
+            if (f64) cells(dimc, std::integral_constant<int, FEM_FP64>());
+            else if (prec == FEM_FP32_MIXED) cells(dimc, std::integral_constant<int, FEM_FP32_MIXED>());
+            else cells(dimc, std::integral_constant<int, FEM_FP32>());
+            if (op.physics == 0) {
+                sell_rows_kernel<D_ + 1, T, true><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, cell, w.mat.cols,
+                                                                       mvals, w.mat.slice, w.mat.state, w.mat.cap, D);
+            } else {
+                sell_rows_kernel<D_ + 1, T, false><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, cell, w.mat.cols,
+                                                                        mvals, w.mat.slice, w.mat.state, w.mat.cap, D);
+                sell_blocks_kernel<D_, T><<<slices, 128, 0, s>>>(C, V, conn, ptr, idx, cell, w.mat.cols, mvals,
+                                                                 w.mat.slice);
+                sell_diag_kernel<D_, T><<<rows, 128, 0, s>>>(V, mvals, w.mat.slice, D);
+            }
+        };
+        if (dim == 2) all(std::integral_constant<int, 2>());
+        else all(std::integral_constant<int, 3>());
+        return check_launch("fem_pcg assembly");
+    };
+    // the element form's diagonal
+    auto element_diagonal = [&]() -> fem_status {
         const int g = static_cast<int>(std::min<int64_t>((C + 255) / 256, 4096));
         unsigned *err = device_error_word();
         if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
@@ -508,10 +1045,12 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
             if (dim == 2) el_diag_kernel<2, T><<<g, 256, 0, s>>>(coords, C, V32, conn, lam, mu, n_q, qwt, el, err);
             else el_diag_kernel<3, T><<<g, 256, 0, s>>>(coords, C, V32, conn, lam, mu, n_q, qwt, el, err);
         }
-        if ((st = check_launch("fem_pcg diagonal")) != FEM_OK) return st;
-        if ((st = launch_gather(dim, nc, C, V, w.elem, ptr, idx, D, vprec, s)) != FEM_OK) return st;
+        fem_status e = check_launch("fem_pcg diagonal");
+        if (e != FEM_OK) return e;
+        if ((e = launch_gather(dim, nc, C, V, w.elem, ptr, idx, D, vprec, s)) != FEM_OK) return e;
         diag_fix_kernel<T><<<gV, 256, 0, s>>>(N, V, fixed, D);
-    }
+        return FEM_OK;
+    };
     // the element vectors of v in w.elem
     auto residual = [&](const T *v, cudaStream_t cs) -> fem_status {
         if (op.physics == 0)
@@ -552,15 +1091,50 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
         if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
         return FEM_OK;
     };
-    // r0 = b - A x0 on the free vertices, u0 = D^-1 r0, w0 = A u0, gamma0, delta0, alpha0
+    if (use_matrix) {
+        // a repeated solve keeps the matrix' state words
+        const bool have = kept == Kept::Matrix;
+        cudaError_t e = cudaMemsetAsync(w.scalars, 0, sizeof(double) * S_MATRIX, s);
+        if (e == cudaSuccess)
+            e = have ? cudaMemsetAsync(w.scalars + S_BARRIER, 0, sizeof(double), s)
+                     : cudaMemsetAsync(w.scalars + S_MATRIX, 0, 2 * sizeof(double), s);
+        if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
+        if (!have && (st = assemble()) != FEM_OK) return st;
+        unsigned *err = device_error_word();
+        if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
+        const CgArgs<T> a{V, w.mat.cols, mvals, w.mat.slice, B, D, fixed, X, r, z, p, sv, q, w.mat_partial, w.scalars,
+                          rtol, max_iter, 0, err};
+        by_comps([&](auto ncc) { e = launch_sell_cg<decltype(ncc)::value, T>(a, s); });
+        if (e == cudaSuccess) {
+            double head[S_COUNT];
+            if ((st = read(0, S_COUNT, head)) != FEM_OK) return st;
+            uint32_t state[2], bar[2];
+            std::memcpy(state, &head[S_MATRIX], sizeof(state));
+            std::memcpy(bar, &head[S_BARRIER], sizeof(bar));
+            if (bar[1] != 0u) return fail(FEM_ERR_TIMEOUT, "fem_pcg_laplacian: a grid barrier gave up");
+            if (state[1] == 0u) {
+                kept = Kept::Matrix;
+                if (iters_out) *iters_out = static_cast<int>(head[S_ITER]);
+                if (resid_out) *resid_out = head[S_RR0] > 0.0 ? std::sqrt(head[S_RR]) / std::sqrt(head[S_RR0]) : 0.0;
+                return check_launch("fem_pcg_laplacian");
+            }
+        } else {
+            cudaGetLastError();  // no cooperative launch (a device partition smaller than the device): element form
+        }
+        // rows too long or too many for the workspace: element form
+        use_matrix = false;
+    }
+    // element form: r0 = b - A x0 on the free vertices, u0 = D^-1 r0, w0 = A u0, gamma0, delta0, alpha0
+    double rr0 = 0.0;
     {
         const cudaError_t e = cudaMemsetAsync(w.scalars, 0, sizeof(double) * S_COUNT, s);
         if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
     }
+    if (kept != Kept::Diagonal && (st = element_diagonal()) != FEM_OK) return st;
+    kept = Kept::Diagonal;
     if ((st = matvec(X, q, s)) != FEM_OK) return st;
     cg_init_kernel<T><<<gV, 256, 0, s>>>(N, V, B, q, D, fixed, r, z, p, sv);
     if ((st = apply_dots(true, 0, s)) != FEM_OK) return st;
-    double rr0 = 0.0;
     if ((st = read(S_RR, 1, &rr0)) != FEM_OK) return st;
     const double r0 = std::sqrt(rr0);
     double rn = r0;
@@ -626,7 +1200,7 @@ using namespace fem;
 extern "C" int64_t fem_pcg_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, true));
 }
 
 extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -646,27 +1220,30 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
         return FEM_OK;
     }
     if (!K || !node_ptr || !node_idx || !fixed || !x || !work) return fail(FEM_ERR_ARG, "a NULL array argument");
-    const int64_t need = fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
+    const bool f64 = prec == FEM_FP64 || prec == FEM_FP64_DF;
+    const size_t vs = f64 ? 8 : 4;
+    const int64_t need = static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, false));
     if (work_bytes < need)
         return fail(FEM_ERR_OOM, "fem_pcg_laplacian: workspace of %lld bytes, %lld needed",
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
-    const bool f64 = prec == FEM_FP64 || prec == FEM_FP64_DF;
-    carve(n_cells, n_verts, dim, f64 ? 8 : 4, work, &w);
+    const bool matrix = work_bytes >= fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
+    carve(n_cells, n_verts, dim, vs, work, &w, 1, matrix);
+    Kept kept = Kept::Nothing;
     if (f64)
         return pcg_run<double>(dim, n_cells, n_verts, coords, conn, Operator{0, K, nullptr, nullptr}, n_q, qpts, qw,
                                node_ptr, node_idx, fixed, b, x,
-                               max_iter, rtol, w, iters_out, resid_out, prec, stream);
+                               max_iter, rtol, w, iters_out, resid_out, prec, stream, kept);
     return pcg_run<float>(dim, n_cells, n_verts, coords, conn, Operator{0, K, nullptr, nullptr}, n_q, qpts, qw,
                           node_ptr, node_idx, fixed, b, x,
-                          max_iter, rtol, w, iters_out, resid_out, prec, stream);
+                          max_iter, rtol, w, iters_out, resid_out, prec, stream, kept);
 }
 
 extern "C" int64_t fem_pcg_elasticity_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, true));
 }
 
 extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -688,20 +1265,23 @@ extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_ver
     }
     if (!lam || !mu || !node_ptr || !node_idx || !fixed || !x || !work)
         return fail(FEM_ERR_ARG, "a NULL array argument");
-    const int64_t need = fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
+    const bool f64 = prec == FEM_FP64 || prec == FEM_FP64_DF;
+    const size_t vs = f64 ? 8 : 4;
+    const int64_t need = static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, false));
     if (work_bytes < need)
         return fail(FEM_ERR_OOM, "fem_pcg_elasticity: workspace of %lld bytes, %lld needed",
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
-    const bool f64 = prec == FEM_FP64 || prec == FEM_FP64_DF;
-    carve(n_cells, n_verts, dim, f64 ? 8 : 4, work, &w, dim);
+    const bool matrix = work_bytes >= fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
+    carve(n_cells, n_verts, dim, vs, work, &w, dim, matrix);
+    Kept kept = Kept::Nothing;
     const Operator op{1, nullptr, lam, mu};
     if (f64)
         return pcg_run<double>(dim, n_cells, n_verts, coords, conn, op, n_q, qpts, qw, node_ptr, node_idx, fixed, b, x,
-                               max_iter, rtol, w, iters_out, resid_out, prec, stream);
+                               max_iter, rtol, w, iters_out, resid_out, prec, stream, kept);
     return pcg_run<float>(dim, n_cells, n_verts, coords, conn, op, n_q, qpts, qw, node_ptr, node_idx, fixed, b, x,
-                          max_iter, rtol, w, iters_out, resid_out, prec, stream);
+                          max_iter, rtol, w, iters_out, resid_out, prec, stream, kept);
 }
 
 // ------------------------------------------------------------------ mixed-precision refinement
@@ -749,10 +1329,11 @@ struct RefineWork {
 };
 
 // physics 0: Laplacian (one coefficient, one component), 1: elasticity (two, dim)
-static size_t carve_refined(int64_t C, int64_t V, int dim, int n_q, int physics, void *base, RefineWork *w) {
+static size_t carve_refined(int64_t C, int64_t V, int dim, int n_q, int physics, void *base, RefineWork *w,
+                            bool matrix) {
     const int nc = physics == 0 ? 1 : dim, ncoef = physics == 0 ? 1 : 2;
     Workspace inner;
-    size_t off = carve(C, V, dim, sizeof(float), base, &inner, nc);
+    size_t off = carve(C, V, dim, sizeof(float), base, &inner, nc, matrix);
     char *b = static_cast<char *>(base);
     auto take = [&](size_t bytes) {
         void *p = b ? b + off : nullptr;
@@ -792,6 +1373,7 @@ static fem_status refined_run(int physics, int dim, int64_t C, int64_t V, const 
                                        : Operator{1, nullptr, w.coef32[0], w.coef32[1]};
     double rn0 = 0.0, rn = 0.0;
     int outer = 0, inner_total = 0;
+    Kept kept = Kept::Nothing;
     for (;;) {
         // the true residual of the float64 iterate
         st = physics == 0 ? fem_integrate_laplacian(dim, C, V, coords, conn, x, coef64[0], n_q, qpts, qw, w.elem,
@@ -819,7 +1401,7 @@ static fem_status refined_run(int physics, int dim, int64_t C, int64_t V, const 
         int it = 0;
         double res = 0.0;
         st = pcg_run<float>(dim, C, V, coords, conn, op32, n_q, qpts, qw, ptr, idx, fixed, w.r32, w.d32, max_inner,
-                            tol_k, w.inner, &it, &res, FEM_FP32_MIXED, stream, outer > 0);
+                            tol_k, w.inner, &it, &res, FEM_FP32_MIXED, stream, kept);
         if (st != FEM_OK) return st;
         inner_total += it;
         refine_update_kernel<<<gV, 256, 0, stream>>>(N, V, fixed, w.d32, x);
@@ -853,12 +1435,12 @@ static fem_status refined_check(int dim, int64_t C, int64_t V, const double *coo
 
 extern "C" int64_t fem_pcg_refined_work_bytes(int dim, int64_t n_cells, int64_t n_verts, int n_q) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0 || n_q < 1 || n_q > FEM_MAX_QPTS) return -1;
-    return static_cast<int64_t>(carve_refined(n_cells, n_verts, dim, n_q, 0, nullptr, nullptr));
+    return static_cast<int64_t>(carve_refined(n_cells, n_verts, dim, n_q, 0, nullptr, nullptr, true));
 }
 
 extern "C" int64_t fem_pcg_elasticity_refined_work_bytes(int dim, int64_t n_cells, int64_t n_verts, int n_q) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0 || n_q < 1 || n_q > FEM_MAX_QPTS) return -1;
-    return static_cast<int64_t>(carve_refined(n_cells, n_verts, dim, n_q, 1, nullptr, nullptr));
+    return static_cast<int64_t>(carve_refined(n_cells, n_verts, dim, n_q, 1, nullptr, nullptr, true));
 }
 
 extern "C" fem_status fem_pcg_laplacian_refined(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -872,13 +1454,15 @@ extern "C" fem_status fem_pcg_laplacian_refined(int dim, int64_t n_cells, int64_
                                   residual_prec, outer_out, inner_out, resid_out);
     if (st != FEM_OK || n_verts == 0) return st;
     if (!K || !node_ptr || !node_idx || !fixed || !x || !work) return fail(FEM_ERR_ARG, "a NULL array argument");
-    const int64_t need = fem_pcg_refined_work_bytes(dim, n_cells, n_verts, n_q);
+    const int64_t need =
+        static_cast<int64_t>(carve_refined(n_cells, n_verts, dim, n_q, 0, nullptr, nullptr, false));
     if (work_bytes < need)
         return fail(FEM_ERR_OOM, "fem_pcg_laplacian_refined: workspace of %lld bytes, %lld needed",
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     RefineWork w;
-    carve_refined(n_cells, n_verts, dim, n_q, 0, work, &w);
+    carve_refined(n_cells, n_verts, dim, n_q, 0, work, &w,
+                  work_bytes >= fem_pcg_refined_work_bytes(dim, n_cells, n_verts, n_q));
     const double *coef[1] = {K};
     return refined_run(0, dim, n_cells, n_verts, coords, conn, coef, n_q, qpts, qw, node_ptr, node_idx, fixed, b, x,
                        max_outer, max_inner, inner_rtol, rtol, w, outer_out, inner_out, resid_out, residual_prec,
@@ -899,13 +1483,15 @@ extern "C" fem_status fem_pcg_elasticity_refined(int dim, int64_t n_cells, int64
     if (int64_t(dim) * n_verts >= (int64_t(1) << 31)) return fail(FEM_ERR_SHAPE, "too many vertices");
     if (!lam || !mu || !node_ptr || !node_idx || !fixed || !x || !work)
         return fail(FEM_ERR_ARG, "a NULL array argument");
-    const int64_t need = fem_pcg_elasticity_refined_work_bytes(dim, n_cells, n_verts, n_q);
+    const int64_t need =
+        static_cast<int64_t>(carve_refined(n_cells, n_verts, dim, n_q, 1, nullptr, nullptr, false));
     if (work_bytes < need)
         return fail(FEM_ERR_OOM, "fem_pcg_elasticity_refined: workspace of %lld bytes, %lld needed",
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     RefineWork w;
-    carve_refined(n_cells, n_verts, dim, n_q, 1, work, &w);
+    carve_refined(n_cells, n_verts, dim, n_q, 1, work, &w,
+                  work_bytes >= fem_pcg_elasticity_refined_work_bytes(dim, n_cells, n_verts, n_q));
     const double *coef[2] = {lam, mu};
     return refined_run(1, dim, n_cells, n_verts, coords, conn, coef, n_q, qpts, qw, node_ptr, node_idx, fixed, b, x,
                        max_outer, max_inner, inner_rtol, rtol, w, outer_out, inner_out, resid_out, residual_prec,
