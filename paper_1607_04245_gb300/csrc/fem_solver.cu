@@ -6,12 +6,12 @@
 //
 // The iteration is CG in Chronopoulos and Gear's form. A solve takes one of two forms:
 //   * assembled: the operator's rows are formed once on the device (fem_sell.cuh) and the
-//     whole loop runs in one cooperative kernel (sell_cg_kernel). Taken whenever the caller's
-//     workspace has room for the matrix.
+//     whole loop runs in one cooperative kernel (sell_cg_kernel). Taken by the float32 forms
+//     and by FEM_FP64 in 3D whenever the caller's workspace has room for the matrix.
 //   * element form: each application is the residual kernel and the vertex sum; one iteration
-//     is captured into the body of a CUDA graph WHILE node. For workspaces without room for
-//     the matrix, meshes whose rows do not fit it, and device partitions that refuse the
-//     cooperative launch.
+//     is captured into the body of a CUDA graph WHILE node. For FEM_FP64_DF and FEM_FP64 in 2D
+//     (assembled_form), workspaces without room for the matrix, meshes whose rows do not fit
+//     it, and device partitions that refuse the cooperative launch.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -912,6 +912,16 @@ struct Workspace {
     double *mat_partial;
 };
 
+// Which solves take the assembled form. The two forms' roundings differ, and CG amplifies that
+// over its iterations: solved to 1e-8, their x differ by up to 3e-11 in float64 on 3D meshes up
+// to 1.6 M cells (the same iteration counts), but by up to 9e-9 in 2D (three times the
+// iterations, ending one to three apart) and against the double-float operator, whose entries
+// are 5e-14 off. Neither is further from the solution (2e-8 at that tolerance), but float64
+// results are held to 1e-9 of the element form's.
+static bool assembled_form(int dim, fem_precision prec) {
+    return prec == FEM_FP32_MIXED || prec == FEM_FP32 || (prec == FEM_FP64 && dim == 3);
+}
+
 // The assembled operator is provided for up to kMatrixMaxBytes of workspace; beyond that (3D:
 // some 600 M cells for the Laplacian, 70 M for elasticity in float64) the solve runs in element form.
 constexpr size_t kMatrixMaxBytes = size_t(32) << 30;
@@ -1200,7 +1210,7 @@ using namespace fem;
 extern "C" int64_t fem_pcg_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, true));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, assembled_form(dim, prec)));
 }
 
 extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -1228,7 +1238,7 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
-    const bool matrix = work_bytes >= fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
+    const bool matrix = assembled_form(dim, prec) && work_bytes >= fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
     carve(n_cells, n_verts, dim, vs, work, &w, 1, matrix);
     Kept kept = Kept::Nothing;
     if (f64)
@@ -1243,7 +1253,7 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
 extern "C" int64_t fem_pcg_elasticity_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, true));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, assembled_form(dim, prec)));
 }
 
 extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -1273,7 +1283,8 @@ extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_ver
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
-    const bool matrix = work_bytes >= fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
+    const bool matrix =
+        assembled_form(dim, prec) && work_bytes >= fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
     carve(n_cells, n_verts, dim, vs, work, &w, dim, matrix);
     Kept kept = Kept::Nothing;
     const Operator op{1, nullptr, lam, mu};

@@ -1,5 +1,6 @@
 """The two forms of the PCG solves against each other: with a full workspace the operator is
-assembled and the loop runs in one kernel; one byte less and the solve runs in element form.
+assembled and the loop runs in one kernel; one byte less and the solve runs in element form
+(which double-float, and float64 in 2D, always take: there the workspace has no room for more).
 Sizes at the edges of what the assembled form distinguishes: slices of 32 rows (V around
 multiples of 32), one CTA or several, vector entries in registers or in memory, a matrix that
 fits shared memory or does not, and rows at and past the longest that is assembled (64).
@@ -9,8 +10,7 @@ rounding alone. One application sums at most 64 products of relative error 3 eps
 adds some ten operations per entry, and the two divisions of an iteration amplify errors of the
 inner products by at most a few units at these first iterations: 64 * 3 * ITERS * 10 eps
 < 1e4 eps of the largest entry, i.e. 1e4 * 1.1e-16 ~ 1e-12 in float64 and 1e4 * 6e-8 ~ 6e-4 in
-float32. The double-float form's element residual carries 5e-14 of its own per application:
-1e-11."""
+float32."""
 
 import numpy as np
 import pytest
@@ -23,7 +23,7 @@ from gpu_util import to_dev
 pytestmark = pytest.mark.gpu
 
 ITERS = 5
-TOL = {"fp64": 1e-12, "fp64_df": 1e-11, "mixed": 6e-4, "fp32": 6e-4}
+TOL = {"fp64": 1e-12, "mixed": 6e-4, "fp32": 6e-4}
 
 
 def _mesh(dim, cells):
@@ -75,6 +75,7 @@ def _element_form_bytes(p):
 
 def _compare(p, **kw):
     full = _work_bytes(p)
+    assert full > _element_form_bytes(p)
     xa, ia, ra = _solve(p, full, **kw)
     xe, ie, re = _solve(p, full - 1, **kw)
     xm, im, rm = _solve(p, _element_form_bytes(p), **kw)
@@ -94,20 +95,27 @@ def _compare(p, **kw):
 
 # cells: tiny meshes; slices of 32 rows at their edges; one CTA (512 rows) and more; a few
 # slices per CTA; ragged counts
-@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "mixed"])
 @pytest.mark.parametrize("physics,dim,cells", [
     ("laplacian", 2, 2), ("laplacian", 2, 50), ("laplacian", 2, 961), ("laplacian", 2, 2047), ("laplacian", 2, 30011),
     ("laplacian", 3, 6), ("laplacian", 3, 163), ("laplacian", 3, 2058), ("laplacian", 3, 20577),
     ("elasticity", 2, 3), ("elasticity", 2, 1117), ("elasticity", 2, 25001),
     ("elasticity", 3, 7), ("elasticity", 3, 3001), ("elasticity", 3, 24001)])
 def test_assembled_equals_element_form(physics, dim, cells, prec):
+    if prec == "fp64" and dim == 2:
+        pytest.skip("float64 in 2D has the element form alone")
     _compare(_problem(_mesh(dim, cells), physics, prec))
 
 
-@pytest.mark.parametrize("prec", ["fp64_df", "fp32"])
-@pytest.mark.parametrize("physics,dim,cells", [("laplacian", 3, 5001), ("elasticity", 3, 5001), ("elasticity", 2, 1117)])
-def test_other_precisions(physics, dim, cells, prec):
-    _compare(_problem(_mesh(dim, cells), physics, prec))
+@pytest.mark.parametrize("physics,dim,prec", [("laplacian", 2, "fp64"), ("laplacian", 3, "fp64_df"),
+                                              ("elasticity", 2, "fp64"), ("elasticity", 3, "fp64_df")])
+def test_element_form_alone(physics, dim, prec):
+    p = _problem(_mesh(dim, 2001), physics, prec)
+    assert _work_bytes(p) == _element_form_bytes(p)
+    x, it, _ = _solve(p, _work_bytes(p))
+    assert it == ITERS and bool(torch.isfinite(x).all())
+    with pytest.raises(fem.FemError):
+        _solve(p, _work_bytes(p) - 1)
 
 
 # every SM with several slices per warp: entries still in registers (64^3 x 6 tets), and past that
@@ -117,8 +125,9 @@ def test_large_meshes(physics, dim, cells):
     _compare(_problem(_mesh(dim, cells), physics, "mixed"))
 
 
-def test_float64_in_memory():
-    _compare(_problem(_mesh(2, 721801), "laplacian", "fp64"))
+@pytest.mark.parametrize("physics,cells", [("laplacian", 1950001), ("elasticity", 600001)])
+def test_float64_in_memory(physics, cells):
+    _compare(_problem(_mesh(3, cells), physics, "fp64"))
 
 
 def test_no_load_and_no_iterations():
@@ -142,7 +151,7 @@ def _fan(k):
 def test_long_rows(k, physics):
     """Rows of up to 64 neighbours are assembled; a mesh with a longer one is solved in element form."""
     mesh = _fan(k)
-    p = _problem(mesh, physics, "fp64")
+    p = _problem(mesh, physics, "mixed")
     fixed = np.zeros(mesh.n_verts, dtype=np.uint8)
     fixed[1:4] = 1
     p["lists"] = (*p["lists"][:2], to_dev(fixed, torch.uint8))
@@ -150,7 +159,7 @@ def test_long_rows(k, physics):
     xa, ia, _ = _solve(p, full)
     xe, ie, _ = _solve(p, full - 1)
     assert ia == ie
-    assert float((xa - xe).abs().max()) <= TOL["fp64"] * float(xe.abs().max())
+    assert float((xa - xe).abs().max()) <= TOL["mixed"] * float(xe.abs().max())
     if k > 64:
         assert torch.equal(xa, xe)
 
