@@ -6,6 +6,11 @@ the sizes, allocates outputs with torch when the caller passes none, and hands r
 pointers and the current CUDA stream to the library. All arithmetic runs in the
 library's CUDA kernels. There is no fallback: if libfem.so is missing or the call
 fails, a RuntimeError is raised.
+
+The integration, adjoint and assembly functions first offer their arguments to the native
+marshalling module (csrc/fem_marshal.cpp), which makes the call if every argument is exactly
+what the entry point takes, at about a fifth of the host time, and returns None if not: then
+the code here converts what can be converted, or raises the error that names the argument.
 """
 
 from __future__ import annotations
@@ -26,6 +31,7 @@ _PREC_NAMES = {"fp64": FEM_FP64, "mixed": FEM_FP32_MIXED, "fp32_mixed": FEM_FP32
 FEM_MAX_QPTS = 32
 
 _lib = None
+_native = None
 
 
 class FemError(RuntimeError):
@@ -99,6 +105,24 @@ def lib():
         L.fem_status_string.restype = ctypes.c_char_p
         _lib = L
     return _lib
+
+
+def native():
+    """The native marshalling module, bound to the loaded libfem (raises if it has not been built)."""
+    global _native
+    if _native is None:
+        L = lib()
+        try:
+            from . import _marshal
+        except ImportError as e:
+            raise RuntimeError("the marshalling module is not built: run __graft_entry__.build() "
+                               f"or python -m paper_1607_04245_gb300.build ({e})") from e
+        names = ("fem_integrate_laplacian", "fem_integrate_laplacian_fields", "fem_integrate_elasticity",
+                 "fem_integrate_reaction_diffusion", "fem_integrate_pointwise", "fem_integrate_laplacian_geom",
+                 "fem_adjoint_laplacian", "fem_build_node2cell", "fem_gather_nodes", "fem_node2cell_work_size")
+        _marshal.init(_check, {n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in names})
+        _native = _marshal
+    return _native
 
 
 def _check(fn: str, st: int):
@@ -215,6 +239,9 @@ def _laplacian_call(coords, conn, u, K, qpts, qw, out, prec, stream):
 
 def fem_integrate_laplacian(coords, conn, u, K, qpts, qw, out=None, prec="mixed", stream=None) -> torch.Tensor:
     """Element residuals [dim+1][C] of the variable-coefficient Laplacian."""
+    r = (_native or native()).laplacian(coords, conn, u, K, qpts, qw, out, prec, stream)
+    if r is not None:
+        return r
     out, args, _keep = _laplacian_call(coords, conn, u, K, qpts, qw, out, prec, stream)
     _check("fem_integrate_laplacian", lib().fem_integrate_laplacian(*args))
     return out
@@ -230,6 +257,10 @@ def prepared_integrate_laplacian(coords, conn, u, K, qpts, qw, out, prec="mixed"
 def fem_integrate_laplacian_fields(coords, conn, u, K, qpts, qw, out=None, prec="mixed", stream=None, prepare=False):
     """Element residuals [F][dim+1][C] of the variable-coefficient Laplacian for F nodal
     fields u [F][V] on one mesh (geometry computed once per cell)."""
+    if not prepare:
+        r = (_native or native()).laplacian_fields(coords, conn, u, K, qpts, qw, out, prec, stream)
+        if r is not None:
+            return r
     p = precision(prec)
     dt = value_dtype(p)
     dim, V, C = _mesh_sizes(coords, conn)
@@ -266,6 +297,9 @@ def _elasticity_call(coords, conn, u, lam, mu, qpts, qw, out, prec, stream):
 
 def fem_integrate_elasticity(coords, conn, u, lam, mu, qpts, qw, out=None, prec="mixed", stream=None) -> torch.Tensor:
     """Element residuals [(dim+1)*dim][C] of linear elasticity (row b*dim + k)."""
+    r = (_native or native()).elasticity(coords, conn, u, lam, mu, qpts, qw, out, prec, stream)
+    if r is not None:
+        return r
     out, args, _keep = _elasticity_call(coords, conn, u, lam, mu, qpts, qw, out, prec, stream)
     _check("fem_integrate_elasticity", lib().fem_integrate_elasticity(*args))
     return out
@@ -320,6 +354,10 @@ def fem_integrate_pointwise(coords, conn, u, coef, qpts, qw, f1=None, f0=None, o
     source text: f1 and f0 are function bodies (see fem_integrate_pointwise in
     include/fem.h for the names in scope), compiled at run time and cached. u is [V] or
     [n_comp][V]; coef is [n_coef][n_q][C] or None. An empty mesh (C = 0) only compiles."""
+    if not prepare:
+        r = (_native or native()).pointwise(coords, conn, u, coef, qpts, qw, f1, f0, out, prec, stream)
+        if r is not None:
+            return r
     p = precision(prec)
     dt = value_dtype(p)
     dim, V, C = _mesh_sizes(coords, conn)
@@ -348,6 +386,10 @@ def fem_integrate_reaction_diffusion(coords, conn, u, a, qpts, qw, c=None, a_spa
     """Element vectors [dim+1][C] of f1 = a grad u, f0 = c u + drift grad a . grad u (Eqs. 2
     and 8): a is P1 nodal ([V], a_space=1) or P0 ([C], a_space=0, grad a = 0); c is
     [n_q][C] or None."""
+    if not prepare:
+        r = (_native or native()).reaction(coords, conn, u, a, qpts, qw, c, a_space, drift, out, prec, stream)
+        if r is not None:
+            return r
     p = precision(prec)
     dt = value_dtype(p)
     dim, V, C = _mesh_sizes(coords, conn)
@@ -561,6 +603,10 @@ def fem_precompute_geometry(coords, conn, geom=None, prec="mixed", stream=None) 
 def fem_integrate_laplacian_geom(conn, n_verts: int, u, K, qpts, qw, geom, out=None, prec="mixed",
                                  stream=None, prepare=False):
     """Laplacian element residuals [dim+1][C] from the precomputed geometry."""
+    if not prepare:
+        r = (_native or native()).laplacian_geom(conn, n_verts, u, K, qpts, qw, geom, out, prec, stream)
+        if r is not None:
+            return r
     p = precision(prec)
     dt = value_dtype(p)
     dim, C = int(conn.shape[0]) - 1, int(conn.shape[1])
@@ -580,6 +626,9 @@ def fem_integrate_laplacian_geom(conn, n_verts: int, u, K, qpts, qw, geom, out=N
 
 def fem_build_node2cell(conn, n_verts: int, node_ptr=None, node_idx=None, work=None, stream=None):
     """Vertex-to-(cell, local vertex) lists: (node_ptr [V+1], node_idx [(dim+1)*C])."""
+    r = (_native or native()).node2cell(conn, n_verts, node_ptr, node_idx, work, stream)
+    if r is not None:
+        return r
     dim = int(conn.shape[0]) - 1
     C = int(conn.shape[1])
     dev = conn.device
@@ -602,6 +651,11 @@ def fem_build_node2cell(conn, n_verts: int, node_ptr=None, node_idx=None, work=N
 def fem_adjoint_laplacian(coords, conn, u, K, qpts, qw, lam_adj, node_ptr, node_idx, dK=None, du=None,
                           scratch=None, prec="mixed", stream=None, prepare=False):
     """Gradient of J = sum lambda . r: returns (dK [n_q][C], du [V])."""
+    if not prepare:
+        r = (_native or native()).adjoint(coords, conn, u, K, qpts, qw, lam_adj, node_ptr, node_idx, dK, du, scratch,
+                                          prec, stream)
+        if r is not None:
+            return r
     p = precision(prec)
     dt = value_dtype(p)
     dim, V, C = _mesh_sizes(coords, conn)
@@ -626,6 +680,9 @@ def fem_adjoint_laplacian(coords, conn, u, K, qpts, qw, lam_adj, node_ptr, node_
 
 def fem_gather_nodes(elem, node_ptr, node_idx, n_verts: int, dim: int, out=None, prec="mixed", stream=None):
     """Assembly E^T of element vectors [(dim+1)*n_comp][C] into nodal values [n_comp][V]."""
+    r = (_native or native()).gather(elem, node_ptr, node_idx, n_verts, dim, out, prec, stream)
+    if r is not None:
+        return r
     p = precision(prec)
     dt = value_dtype(p)
     rows, C = int(elem.shape[0]), int(elem.shape[1])

@@ -1,8 +1,11 @@
-"""Build libfem (the CUDA C-ABI library) in-tree for sm_103a.
+"""Build libfem (the CUDA C-ABI library) in-tree for sm_103a, and the binding's native
+marshalling module.
 
 Each .cu translation unit is compiled in parallel with nvcc, then linked into
 ``paper_1607_04245_gb300/libfem.so``. No cmake, no torch extension machinery: the
-library is a plain shared object with the C ABI of ``include/fem.h``.
+library is a plain shared object with the C ABI of ``include/fem.h``. Beside it,
+``fem_marshal.cpp`` is compiled with g++ against the installed torch into the extension
+module ``paper_1607_04245_gb300/_marshal`` (host code; it links no libfem).
 
     python -m paper_1607_04245_gb300.build [--verbose-ptxas]
 """
@@ -14,6 +17,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -39,8 +43,32 @@ def _deps_mtime() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+MARSHAL = os.path.join(PKG, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def _build_marshal() -> None:
+    """fem_marshal.cpp against this interpreter and the installed torch."""
+    import torch
+
+    t = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc())))
+    cuda_inc = [d for d in (os.path.join(cuda, "include"), "/usr/local/cuda/include") if os.path.isdir(d)]
+    tmp = MARSHAL + ".tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", sysconfig.get_path("include"),
+           "-I", os.path.join(t, "include"), "-I", os.path.join(t, "include", "torch", "csrc", "api", "include")]
+    cmd += [x for d in cuda_inc for x in ("-I", d)]
+    cmd += [os.path.join(CSRC, "fem_marshal.cpp"), "-o", tmp, "-L", os.path.join(t, "lib"), "-ltorch_python",
+            "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on fem_marshal.cpp:\n{r.stderr}")
+    os.replace(tmp, MARSHAL)
+
+
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
-    if not force and not verbose_ptxas and os.path.exists(OUT) and os.path.getmtime(OUT) >= _deps_mtime():
+    done = all(os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime() for f in (OUT, MARSHAL))
+    if not force and not verbose_ptxas and done:
         return OUT
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
@@ -56,8 +84,10 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr}")
         return obj, r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        marshal = ex.submit(_build_marshal)
         results = list(ex.map(compile_one, SOURCES))
+        marshal.result()
     if verbose_ptxas:
         for _, log in results:
             sys.stderr.write(log)
