@@ -92,6 +92,41 @@ __device__ __forceinline__ void store_row(double *p, const double (&v)[CPT]) {
     }
 }
 
+// The CPT cells that thread g of a grid-stride loop owns. STRIDED = false: consecutive ones, whose
+// rows are read and written as one vector (the rows must be aligned for it). STRIDED = true: cells
+// 32 apart, lane l of a warp taking l, l + 32, .. of the warp's 32 CPT cells, so that every access
+// is a coalesced one of single values whatever the rows' alignment and the cell count; cells past
+// the last are computed as copies of it and not stored.
+template <int CPT, bool STRIDED>
+struct Cells {
+    int64_t c0, C;
+    static __host__ __device__ int64_t groups(int64_t C) {
+        return STRIDED ? (C + 32 * CPT - 1) / (32 * CPT) * 32 : (C + CPT - 1) / CPT;
+    }
+    __device__ __forceinline__ Cells(int64_t g, int64_t n) : c0(STRIDED ? (g >> 5) * (32 * CPT) + (g & 31) : g * CPT), C(n) {}
+    __device__ __forceinline__ int64_t at(int i) const { return STRIDED ? min(c0 + 32 * i, C - 1) : c0 + i; }
+    __device__ __forceinline__ bool in(int i) const { return !STRIDED || c0 + 32 * i < C; }
+    template <class T>
+    __device__ __forceinline__ void load(const T *row, T (&v)[CPT]) const {
+        if constexpr (STRIDED) {
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) v[i] = ld_stream(row + at(i));
+        } else {
+            load_row<CPT>(row + c0, v);
+        }
+    }
+    template <class T>
+    __device__ __forceinline__ void store(T *row, const T (&v)[CPT]) const {
+        if constexpr (STRIDED) {
+#pragma unroll
+            for (int i = 0; i < CPT; ++i)
+                if (in(i)) __stcs(row + c0 + 32 * i, v[i]);
+        } else {
+            store_row<CPT>(row + c0, v);
+        }
+    }
+};
+
 // ------------------------------------------------------------------ generic arithmetic
 // The cell algebra below is written once for double, float and f2 (two cells per value).
 

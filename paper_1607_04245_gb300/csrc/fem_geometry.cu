@@ -94,21 +94,21 @@ __global__ void __launch_bounds__(kBlock) lap_geom_kernel(const __grid_constant_
     const int nq = NQ > 0 ? NQ : a.w.nq;
     uint32_t vmax = 0;
     bool bad_det = false;
-    const int64_t ngroups = (C + CPT - 1) / CPT;
+    const int64_t ngroups = Cells<CPT, false>::groups(C);
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
-        const int64_t c0 = g * CPT;
+        const Cells<CPT, false> cells(g, C);
         int32_t vid[NB][CPT];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) load_row<CPT>(a.conn + b * C + c0, vid[b]);
+        for (int b = 0; b < NB; ++b) cells.load(a.conn + b * C, vid[b]);
         T gm[DIM * DIM + 1][CPT];
 #pragma unroll
-        for (int r = 0; r <= DIM * DIM; ++r) load_row<CPT>(geom + r * C + c0, gm[r]);
+        for (int r = 0; r <= DIM * DIM; ++r) cells.load(geom + r * C, gm[r]);
         qsum_t<P> ks[CPT];
 #pragma unroll(NQ > 0 ? NQ : 1)
         for (int q = 0; q < nq; ++q) {
             T kq[CPT];
-            load_row<CPT>(K + q * C + c0, kq);
+            cells.load(K + q * C, kq);
 #pragma unroll
             for (int i = 0; i < CPT; ++i) {
                 if (q == 0) ks[i].first(gweight<P>(a.w, 0), kq[i]);
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kBlock) lap_geom_kernel(const __grid_constant_
             r[0][i] = -sum;
         }
 #pragma unroll
-        for (int b = 0; b < NB; ++b) store_row<CPT>(out + b * C + c0, r[b]);
+        for (int b = 0; b < NB; ++b) cells.store(out + b * C, r[b]);
     }
     report_mesh(a.err, vmax, a.V, bad_det);
 }
@@ -158,6 +158,11 @@ static fem_status launch_geom_lap(const LapGeomArgs &a, bool vec, cudaStream_t s
         // one wave of resident CTAs (24.5 against 24.7 us per step with up to 8 waves)
         auto k = lap_geom_kernel<DIM, P, 4, DIM + 1>;
         launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, (a.C + 3) / 4), kBlock, 0, s, a);
+    } else if (a.w.nq == DIM + 1) {
+        // ragged rows: one cell per thread (999,999 cells, float32: 3D 18.8 -> 17.3 us, 2D 14.4 ->
+        // 10.1 us against the run-time rule; two cells 32 apart 19.2 / 11.4, four 23.7 / 11.9)
+        auto k = lap_geom_kernel<DIM, P, 1, DIM + 1>;
+        launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, a.C), kBlock, 0, s, a);
     } else if (vec) {
         auto k = lap_geom_kernel<DIM, P, 4, 0>;
         launch_overlapped(k, grid_for((a.C + 3) / 4, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);

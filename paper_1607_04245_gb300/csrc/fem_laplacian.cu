@@ -162,11 +162,10 @@ __device__ __forceinline__ void lap_cell(const double (&xs)[DIM + 1][DIM],
 }
 
 // Direct kernel: one thread owns CPT consecutive cells and reads the cell-indexed rows
-// with (vector) loads from global memory. Used where neither the pair kernel (float32
-// forms: an even cell count, 8-byte aligned rows) nor the staged kernel (float64 form:
-// 16-byte aligned rows, stages that fit in shared memory) applies, and by the host-buffer
-// path, which reads page-locked host memory.
-template <int DIM, int P, int CPT, int NQ, bool ADJ>
+// (or, STR, 32 apart) with (vector) loads from global memory. Used where neither the pair kernel
+// (float32 forms) nor the staged kernel (float64 form: 16-byte aligned rows, stages that fit in
+// shared memory) applies, and by the host-buffer path, which reads page-locked host memory.
+template <int DIM, int P, int CPT, int NQ, bool ADJ, bool STR = false>
 __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ LapArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
@@ -182,13 +181,13 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
 
     uint32_t vmax = 0;     // largest vertex id seen (bad ids are clamped and reported)
     bool bad_det = false;  // a cell with det J = 0 or non-finite
-    const int64_t ngroups = (C + CPT - 1) / CPT;
+    const int64_t ngroups = Cells<CPT, STR>::groups(C);
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
-        const int64_t c0 = g * CPT;
+        const Cells<CPT, STR> cells(g, C);
         int32_t vid[NB][CPT];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) load_row<CPT>(a.conn + b * C + c0, vid[b]);
+        for (int b = 0; b < NB; ++b) cells.load(a.conn + b * C, vid[b]);
 
         // quadrature sum of the coefficient: Kbar = sum_q w_q K_q (with NQ > 0 every row
         // load is issued before the first sum)
@@ -196,7 +195,7 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
         if constexpr (NQ > 0) {
             T kq[NQ][CPT];
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) load_row<CPT>(K + q * C + c0, kq[q]);
+            for (int q = 0; q < NQ; ++q) cells.load(K + q * C, kq[q]);
 #pragma unroll
             for (int i = 0; i < CPT; ++i) ks[i].first(weight<P>(a.w, 0), kq[0][i]);
 #pragma unroll
@@ -206,13 +205,13 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
         } else {
             {
                 T kq[CPT];
-                load_row<CPT>(K + c0, kq);
+                cells.load(K, kq);
 #pragma unroll
                 for (int i = 0; i < CPT; ++i) ks[i].first(weight<P>(a.w, 0), kq[i]);
             }
             for (int q = 1; q < a.w.nq; ++q) {
                 T kq[CPT];
-                load_row<CPT>(K + q * C + c0, kq);
+                cells.load(K + q * C, kq);
                 const T wq = weight<P>(a.w, q);
 #pragma unroll
                 for (int i = 0; i < CPT; ++i) ks[i].add(wq, kq[i]);
@@ -222,7 +221,7 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
         T lamv[ADJ ? NB : 1][CPT];
         if constexpr (ADJ) {
 #pragma unroll
-            for (int b = 0; b < NB; ++b) load_row<CPT>(static_cast<const T *>(a.lam) + b * C + c0, lamv[b]);
+            for (int b = 0; b < NB; ++b) cells.load(static_cast<const T *>(a.lam) + b * C, lamv[b]);
         }
 
         T r[NB][CPT];
@@ -247,7 +246,7 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
             tfac[i] = tf;
         }
 #pragma unroll
-        for (int b = 0; b < NB; ++b) store_row<CPT>(out + b * C + c0, r[b]);
+        for (int b = 0; b < NB; ++b) cells.store(out + b * C, r[b]);
         if constexpr (ADJ) {
             T *dK = static_cast<T *>(a.dK);
             for (int q = 0; q < a.w.nq; ++q) {
@@ -255,7 +254,7 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
                 T row[CPT];
 #pragma unroll
                 for (int i = 0; i < CPT; ++i) row[i] = wq * tfac[i];
-                store_row<CPT>(dK + q * C + c0, row);
+                cells.store(dK + q * C, row);
             }
         }
     }
@@ -304,7 +303,7 @@ __device__ __noinline__ void lap_fields_fallback(const FieldsArgs &fa, int64_t c
     }
 }
 
-template <int DIM, int P, int CPT, int NQ>
+template <int DIM, int P, int CPT, int NQ, bool STR = false>
 __global__ void __launch_bounds__(kBlock) lap_fields_kernel(const __grid_constant__ FieldsArgs fa) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
@@ -322,24 +321,24 @@ __global__ void __launch_bounds__(kBlock) lap_fields_kernel(const __grid_constan
     const int nq = NQ > 0 ? NQ : a.w.nq;
     uint32_t vmax = 0;
     bool bad_det = false;
-    const int64_t ngroups = (C + CPT - 1) / CPT;
+    const int64_t ngroups = Cells<CPT, STR>::groups(C);
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
-        const int64_t c0 = g * CPT;
+        const Cells<CPT, STR> cells(g, C);
         int32_t vid[NB][CPT];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) load_row<CPT>(a.conn + b * C + c0, vid[b]);
+        for (int b = 0; b < NB; ++b) cells.load(a.conn + b * C, vid[b]);
         qsum_t<P> ks[CPT];
         {
             T kq[CPT];
-            load_row<CPT>(K + c0, kq);
+            cells.load(K, kq);
 #pragma unroll
             for (int i = 0; i < CPT; ++i) ks[i].first(weight<P>(a.w, 0), kq[i]);
         }
 #pragma unroll(NQ > 0 ? NQ - 1 : 1)
         for (int q = 1; q < nq; ++q) {
             T kq[CPT];
-            load_row<CPT>(K + q * C + c0, kq);
+            cells.load(K + q * C, kq);
 #pragma unroll
             for (int i = 0; i < CPT; ++i) ks[i].add(weight<P>(a.w, q), kq[i]);
         }
@@ -376,12 +375,12 @@ __global__ void __launch_bounds__(kBlock) lap_fields_kernel(const __grid_constan
                 for (int b = 0; b < NB; ++b) r[b][i] = rr[b];
             }
 #pragma unroll
-            for (int b = 0; b < NB; ++b) store_row<CPT>(out + (int64_t(f) * NB + b) * C + c0, r[b]);
+            for (int b = 0; b < NB; ++b) cells.store(out + (int64_t(f) * NB + b) * C, r[b]);
         }
         if constexpr (P == FEM_FP32_MIXED) {
 #pragma unroll
             for (int i = 0; i < CPT; ++i)
-                if (!ok[i]) lap_fields_fallback<DIM>(fa, c0 + i, ks[i].value_f64());
+                if (!ok[i] && cells.in(i)) lap_fields_fallback<DIM>(fa, cells.at(i), ks[i].value_f64());
         }
     }
     report_mesh(a.err, vmax, a.V, bad_det);
@@ -398,6 +397,11 @@ static fem_status launch_fields(const FieldsArgs &fa, bool vec, cudaStream_t s) 
         const int64_t n = (fa.a.C + CPTV - 1) / CPTV;
         const void *kp = reinterpret_cast<const void *>(k);
         launch_overlapped(k, P == FEM_FP64 ? grid_for(n, kBlock, kp) : resident_grid(kp, kBlock, n), kBlock, 0, s, fa);
+    } else if (P != FEM_FP64 && fa.a.w.nq == NQN) {
+        // ragged rows, float32 forms: two cells per thread, 32 apart (four fields, 999,999 cells:
+        // 3D 35.0 -> 27.6 us, 2D 27.9 -> 22.6 us against one cell with the run-time rule)
+        auto k = lap_fields_kernel<DIM, P, 2, NQN, true>;
+        launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, Cells<2, true>::groups(fa.a.C)), kBlock, 0, s, fa);
     } else {
         auto k = lap_fields_kernel<DIM, P, 1, 0>;
         launch_overlapped(k, grid_for(fa.a.C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, fa);
@@ -497,7 +501,8 @@ __device__ __forceinline__ void lap_pair(const double *const (&X)[DIM], const ui
 
 // ------------------------------------------------------------------ pair kernel
 //
-// The float32 forms' kernel for rows that are 8-byte aligned (an even cell count): each
+// The float32 forms' kernel for rows that are 8-byte aligned (an even cell count; STR: any count
+// and alignment, with two cells 32 apart instead of consecutive ones and 4-byte accesses): each
 // thread owns two consecutive cells at a time and computes them as f32x2 pairs
 // (lap_pair), reading every cell-indexed row with 8-byte loads and writing 8-byte
 // streaming stores, grid-stride over the cell pairs with one wave of resident CTAs (3 of
@@ -518,13 +523,13 @@ __device__ __forceinline__ void lap_pair(const double *const (&X)[DIM], const ui
 template <int P, bool ADJ>
 constexpr int pair_min_blocks() { return (P == FEM_FP32 && !ADJ) ? 4 : 3; }
 
-template <int DIM, int P, int NQ, bool ADJ>
+template <int DIM, int P, int NQ, bool ADJ, bool STR>
 __global__ void __launch_bounds__(kBlock, pair_min_blocks<P, ADJ>()) lap_pair_kernel(const __grid_constant__ LapArgs a) {
     static_assert(P != FEM_FP64, "float32 forms only");
     pdl_wait();  // launched overlapped: the previous kernel's writes are visible from here
     pdl_trigger();
     constexpr int NB = DIM + 1;
-    const int64_t C = a.C;  // even
+    const int64_t C = a.C;  // even, unless STR
     const float *__restrict__ u = static_cast<const float *>(a.u);
     const float *__restrict__ K = static_cast<const float *>(a.K);
     const float *__restrict__ L = static_cast<const float *>(a.lam);
@@ -536,31 +541,34 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<P, ADJ>()) lap_pair_ke
     const int nq = NQ > 0 ? NQ : a.w.nq;
     uint32_t vmax = 0;     // largest vertex id seen (bad ids are clamped and reported)
     bool bad_det = false;  // float32 ablation: a cell with det J = 0 or non-finite, or repeated ids
-    const int64_t np = C / 2;
+    const int64_t np = Cells<2, STR>::groups(C);
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < np; g += stride) {
-        const int64_t c = 2 * g;
+        const Cells<2, STR> cells(g, C);
         uint32_t va[NB], vb[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-            const int2 t = __ldcs(reinterpret_cast<const int2 *>(a.conn + b * C + c));
-            va[b] = clamp_vid(t.x, a.V, vmax);
-            vb[b] = clamp_vid(t.y, a.V, vmax);
+            int32_t t[2];
+            cells.load(a.conn + b * C, t);
+            va[b] = clamp_vid(t[0], a.V, vmax);
+            vb[b] = clamp_vid(t[1], a.V, vmax);
         }
         qsum2_t<P> ks;
 #pragma unroll(NQ > 0 ? NQ : 1)
         for (int q = 0; q < nq; ++q) {
-            const float2 k = __ldcs(reinterpret_cast<const float2 *>(K + q * C + c));
-            if (q == 0) ks.first(a.w.wf[0], f2_make(k.x, k.y));
-            else ks.add(a.w.wf[q], f2_make(k.x, k.y));
+            float k[2];
+            cells.load(K + q * C, k);
+            if (q == 0) ks.first(a.w.wf[0], f2_make(k[0], k[1]));
+            else ks.add(a.w.wf[q], f2_make(k[0], k[1]));
         }
         f2 uu[NB], ll[NB], rr[NB], tf = zero<f2>();
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             uu[b] = f2_make(ld_gather(u + va[b]), ld_gather(u + vb[b]));
             if constexpr (ADJ) {
-                const float2 l = __ldcs(reinterpret_cast<const float2 *>(L + b * C + c));
-                ll[b] = f2_make(l.x, l.y);
+                float l[2];
+                cells.load(L + b * C, l);
+                ll[b] = f2_make(l[0], l[1]);
             } else {
                 ll[b] = zero<f2>();
             }
@@ -568,17 +576,20 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<P, ADJ>()) lap_pair_ke
         bool oka, okb;
         lap_pair<DIM, P, ADJ>(X, va, vb, uu, ll, ks, a.tau2, rr, tf, oka, okb);
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-            __stcs(reinterpret_cast<float2 *>(out + b * C + c), make_float2(f2_x(rr[b]), f2_y(rr[b])));
+        for (int b = 0; b < NB; ++b) {
+            const float o[2] = {f2_x(rr[b]), f2_y(rr[b])};
+            cells.store(out + b * C, o);
+        }
         if constexpr (ADJ) {
             for (int q = 0; q < nq; ++q) {
                 const float wq = a.w.wf[q];
-                __stcs(reinterpret_cast<float2 *>(dK + q * C + c), make_float2(wq * f2_x(tf), wq * f2_y(tf)));
+                const float o[2] = {wq * f2_x(tf), wq * f2_y(tf)};
+                cells.store(dK + q * C, o);
             }
         }
         if constexpr (P == FEM_FP32_MIXED) {
-            if (!oka) lap_fallback_store<DIM, ADJ>(a, c, ks.value_f64_x());
-            if (!okb) lap_fallback_store<DIM, ADJ>(a, c + 1, ks.value_f64_y());
+            if (!oka && cells.in(0)) lap_fallback_store<DIM, ADJ>(a, cells.at(0), ks.value_f64_x());
+            if (!okb && cells.in(1)) lap_fallback_store<DIM, ADJ>(a, cells.at(1), ks.value_f64_y());
         } else {
             bad_det |= !oka | !okb | ids_repeat<NB>(va) | ids_repeat<NB>(vb);
         }
@@ -586,10 +597,11 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<P, ADJ>()) lap_pair_ke
     report_mesh(a.err, vmax, a.V, bad_det);
 }
 
-template <int DIM, int P, int NQ, bool ADJ>
+template <int DIM, int P, int NQ, bool ADJ, bool STR>
 static void launch_pair(const LapArgs &a, cudaStream_t s) {
-    auto k = lap_pair_kernel<DIM, P, NQ, ADJ>;
-    launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, a.C / 2), kBlock, 0, s, a);
+    auto k = lap_pair_kernel<DIM, P, NQ, ADJ, STR>;
+    const int64_t n = Cells<2, STR>::groups(a.C);
+    launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, n), kBlock, 0, s, a);
 }
 
 // ------------------------------------------------------------------ prepared vertex records
@@ -873,8 +885,15 @@ static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_
         // Its plain 8-byte loads also serve rows in page-locked host memory (staged_ok
         // false): from host buffers 0.309 against 0.331 ms per step with lap_kernel.
         if (pairs) {
-            if (native_nq) launch_pair<DIM, P, DIM + 1, ADJ>(a, s);
-            else launch_pair<DIM, P, 0, ADJ>(a, s);
+            if (native_nq) launch_pair<DIM, P, DIM + 1, ADJ, false>(a, s);
+            else launch_pair<DIM, P, 0, ADJ, false>(a, s);
+            return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
+        }
+        // an odd cell count (every second row starts between 8-byte words): the same pairs from
+        // cells 32 apart, single-value accesses (999,999 tets: 23.8 -> 17.0 us, the adjoint 45.7
+        // -> 36.7, against one cell per thread; an even count takes 14.8: twice the row accesses)
+        if (a.C % 2 != 0 && native_nq) {
+            launch_pair<DIM, P, DIM + 1, ADJ, true>(a, s);
             return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
         }
     }
@@ -894,6 +913,12 @@ static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_
     } else if (vec) {
         auto k = lap_kernel<DIM, P, 4, 0, ADJ>;
         int grid = grid_for((a.C + 3) / 4, kBlock, reinterpret_cast<const void *>(k));
+        launch_overlapped(k, grid, kBlock, 0, s, a);
+    } else if (P != FEM_FP64 && native_nq) {
+        // rows misaligned by their base pointers: two cells per thread, 32 apart (10^6 tets: 23.4 ->
+        // 17.8 us against one cell with the run-time rule, bitwise the same results)
+        auto k = lap_kernel<DIM, P, 2, DIM + 1, ADJ, true>;
+        int grid = grid_for(Cells<2, true>::groups(a.C), kBlock, reinterpret_cast<const void *>(k));
         launch_overlapped(k, grid, kBlock, 0, s, a);
     } else {
         auto k = lap_kernel<DIM, P, 1, 0, ADJ>;

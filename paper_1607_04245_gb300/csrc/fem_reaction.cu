@@ -247,7 +247,7 @@ constexpr int rd_min_blocks() {
     return (P != FEM_FP64 && DIM == 3 && CPT == 2) ? 3 : 1;
 }
 
-template <int DIM, int P, bool A_P1, bool REACT, bool DRIFT, int CPT, int NQ>
+template <int DIM, int P, bool A_P1, bool REACT, bool DRIFT, int CPT, int NQ, bool STR = false>
 __global__ void __launch_bounds__(kBlock, rd_min_blocks<DIM, P, CPT>()) rd_kernel(const __grid_constant__ RdArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
@@ -266,19 +266,19 @@ __global__ void __launch_bounds__(kBlock, rd_min_blocks<DIM, P, CPT>()) rd_kerne
     for (int k = 0; k < DIM; ++k) X[k] = a.X[k];
     uint32_t vmax = 0;     // largest vertex id seen (bad ids are clamped and reported)
     bool bad_det = false;  // a cell with det J = 0 or non-finite
-    const int64_t ngroups = (C + CPT - 1) / CPT;
+    const int64_t ngroups = Cells<CPT, STR>::groups(C);
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
-        const int64_t c0 = g * CPT;
+        const Cells<CPT, STR> cells(g, C);
         int32_t vid[NB][CPT];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) load_row<CPT>(a.conn + b * C + c0, vid[b]);
+        for (int b = 0; b < NB; ++b) cells.load(a.conn + b * C, vid[b]);
         T a0[CPT];
-        if constexpr (!A_P1) load_row<CPT>(af + c0, a0);
+        if constexpr (!A_P1) cells.load(af, a0);
         T cq[REACT ? NQA : 1][CPT];
         if constexpr (REACT) {
 #pragma unroll(NQ > 0 ? NQ : 1)
-            for (int q = 0; q < nq; ++q) load_row<CPT>(cf + q * C + c0, cq[q]);
+            for (int q = 0; q < nq; ++q) cells.load(cf + q * C, cq[q]);
         }
         T r[NB][CPT];
         bool ok[CPT];
@@ -298,11 +298,11 @@ __global__ void __launch_bounds__(kBlock, rd_min_blocks<DIM, P, CPT>()) rd_kerne
             for (int b = 0; b < NB; ++b) r[b][i] = rr[b];
         }
 #pragma unroll
-        for (int b = 0; b < NB; ++b) store_row<CPT>(out + b * C + c0, r[b]);
+        for (int b = 0; b < NB; ++b) cells.store(out + b * C, r[b]);
         if constexpr (P == FEM_FP32_MIXED) {
 #pragma unroll
             for (int i = 0; i < CPT; ++i)
-                if (!ok[i]) rd_fallback_store<DIM, A_P1, REACT, DRIFT>(a, c0 + i);
+                if (!ok[i] && cells.in(i)) rd_fallback_store<DIM, A_P1, REACT, DRIFT>(a, cells.at(i));
         }
     }
     report_mesh(a.err, vmax, a.V, bad_det);
@@ -319,6 +319,12 @@ static void launch_rd_one(const RdArgs &a, bool vec4, bool vec2, cudaStream_t s)
     if (P != FEM_FP64 && vec && a.w.nq == NQN) {
         auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, CPTV, NQN>;
         launch_overlapped(k, grid_for((a.C + CPTV - 1) / CPTV, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
+    } else if (P != FEM_FP64 && a.w.nq == NQN) {
+        // ragged rows: the same cells per thread, 32 apart (999,999 cells: 3D 44.2 -> 21.2 us, 2D
+        // 35.8 -> 13.6 us against one cell with the run-time rule, whose values per point go
+        // through local memory)
+        auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, CPTV, NQN, true>;
+        launch_overlapped(k, grid_for(Cells<CPTV, true>::groups(a.C), kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
     } else {
         auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, 1, 0>;
         launch_overlapped(k, grid_for(a.C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
