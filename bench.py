@@ -1331,7 +1331,7 @@ def run_ours(args):
                      "achieved_tflops": fp64_flops / t64 / 1e12,
                      "peak_kind": f"nominal {FP64_NOMINAL_TFLOPS} TFLOP/s float64 = 2 FMA instructions/clock/SM, "
                                   f"at the sampled {sm_mhz:.0f} MHz",
-                     "kernel": "lap_staged_kernel<3, FP64, NQ=4>",
+                     "kernel": "lap_kernel<3, FP64, 1 cell per thread, NQ=4>",
                      "inst_per_cell": FP64_INST_PER_CELL_LAP3D}
 
     probe = measure_fp64_fma_rate(device)

@@ -470,9 +470,6 @@ fem_status fem_adjoint_laplacian(int dim, int64_t n_cells, int64_t n_verts, cons
  *     contents. Each call writes every entry it reads before reading it, so nothing
  *     needs clearing; but calls that overlap on the GPU (different streams, or host
  *     threads) race on the array and must be serialised by the caller.
- *   - Validity: dK and du are valid only if the next fem_device_error() returns FEM_OK.
- *     A bounded wait that gave up (FEM_ERR_TIMEOUT) leaves a tile of the array unwritten,
- *     and du then includes the previous call's values for it.
  * Arguments, layouts and results are those of fem_adjoint_laplacian without `scratch`.
  * ------------------------------------------------------------------------------- */
 #define FEM_NOALLOC_SCRATCH_BYTES (16u << 20)
@@ -629,9 +626,9 @@ fem_status fem_probe(int kind, int64_t n_threads, int iters, void *out, fem_stre
 /* ---------------------------------------------------------------------------------
  * fem_device_error -- the device-side status of the kernels since the last call: a
  * per-device error word that kernels set bits in. Two conditions: (1) bounded waits (not
- * in the paper): the staged kernels wait on the bulk copies of their inputs with a time
- * budget (0.5 s per wait); a wait that runs out stops that CTA without writing the tile
- * it waited for; (2) the mesh check (the boundary's debug check, always on): a vertex id
+ * in the paper): the loop kernel of a solve waits for its other CTAs with a time budget (4 s
+ * per wait) and ends when a wait runs out (the solve itself then returns FEM_ERR_TIMEOUT), and
+ * fem_selftest_wait; (2) the mesh check (the boundary's debug check, always on): a vertex id
  * outside [0, n_verts) (clamped, so nothing is read out of bounds), or a cell with
  * det J = 0, a non-finite det J or a repeated vertex id. fem_device_error synchronises
  * `stream`, reads and clears the word of the current device, and returns
@@ -643,8 +640,7 @@ fem_status fem_probe(int kind, int64_t n_threads, int iters, void *out, fem_stre
  * ------------------------------------------------------------------------------- */
 fem_status fem_device_error(fem_stream stream);
 
-/* fem_selftest_wait -- launches one CTA that waits, with the bounded wait of the staged
- * kernels and a budget of budget_ns (0 .. 10 s), for a barrier phase that never
+/* fem_selftest_wait -- launches one CTA that waits, with a bounded wait and a budget of budget_ns (0 .. 10 s), for a barrier phase that never
  * completes, so that the next fem_device_error() returns FEM_ERR_TIMEOUT. For tests of
  * the timeout path; it faults nothing and leaves the context usable. */
 fem_status fem_selftest_wait(int64_t budget_ns, fem_stream stream);

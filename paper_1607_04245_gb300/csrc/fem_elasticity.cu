@@ -236,18 +236,27 @@ template <int DIM, int P>
 static fem_status launch_el(const ElArgs &a, bool vec4, bool vec2, cudaStream_t s) {
     // 3D float32 forms: two cells per thread (four would hold 48 output registers until the
     // row stores); otherwise four
-    constexpr int CPTV = (DIM == 3 && P != FEM_FP64) ? 2 : 4;
+    constexpr int CPTV = DIM == 3 ? 2 : 4;
     const bool vec = CPTV == 2 ? vec2 : vec4;
+    if constexpr (P == FEM_FP64) {
+        if (a.w.nq == DIM + 1) {
+            auto k = el_kernel<DIM, P, 1, DIM + 1>;
+            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+        } else {
+            auto k = el_kernel<DIM, P, 1, 0>;
+            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+        }
+        return check_launch("fem_integrate_elasticity");
+    } else
     // the quadrature size of the workloads' rules (3 points in 2D, 4 in 3D) is compiled in.
     // The float32 forms run one wave of resident CTAs (steps back to back: 3D 52.9 -> 48.3
-    // us, 2D 55.9 -> 54.6 us against up to 8 waves); float64 keeps the waves.
+    // us, 2D 55.9 -> 54.6 us against up to 8 waves).
     if (vec && a.w.nq == DIM + 1) {
         auto k = el_kernel<DIM, P, CPTV, DIM + 1>;
         const int64_t n = (a.C + CPTV - 1) / CPTV;
-        const void *kp = reinterpret_cast<const void *>(k);
-        launch_overlapped(k, P == FEM_FP64 ? grid_for(n, kBlock, kp) : resident_grid(kp, kBlock, n), kBlock, 0, s, a);
-    } else if (P != FEM_FP64 && a.w.nq == DIM + 1) {
-        // ragged rows, float32 forms: 3D two cells per thread, 32 apart (999,999 tets: 44.5 us with
+        launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, n), kBlock, 0, s, a);
+    } else if (a.w.nq == DIM + 1) {
+        // ragged rows: 3D two cells per thread, 32 apart (999,999 tets: 44.5 us with
         // one cell and the run-time rule, 31.9 with one cell, 28.8); 2D one cell (999,999 triangles:
         // 24.3 -> 17.3 us; four cells 24.8, two 18.2)
         constexpr int CPTS = DIM == 3 ? 2 : 1;

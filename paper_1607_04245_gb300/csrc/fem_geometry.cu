@@ -154,12 +154,20 @@ __global__ void __launch_bounds__(kBlock) lap_geom_kernel(const __grid_constant_
 
 template <int DIM, int P>
 static fem_status launch_geom_lap(const LapGeomArgs &a, bool vec, cudaStream_t s) {
-    if (vec && a.w.nq == DIM + 1) {
+    if constexpr (P == FEM_FP64) {
+        if (a.w.nq == DIM + 1) {
+            auto k = lap_geom_kernel<DIM, P, 1, DIM + 1>;
+            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+        } else {
+            auto k = lap_geom_kernel<DIM, P, 1, 0>;
+            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+        }
+    } else if (vec && a.w.nq == DIM + 1) {
         // one wave of resident CTAs (24.5 against 24.7 us per step with up to 8 waves)
         auto k = lap_geom_kernel<DIM, P, 4, DIM + 1>;
         launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, (a.C + 3) / 4), kBlock, 0, s, a);
     } else if (a.w.nq == DIM + 1) {
-        // ragged rows: one cell per thread (999,999 cells, float32: 3D 18.8 -> 17.3 us, 2D 14.4 ->
+        // ragged rows: one cell per thread (999,999 cells: 3D 18.8 -> 17.3 us, 2D 14.4 ->
         // 10.1 us against the run-time rule; two cells 32 apart 19.2 / 11.4, four 23.7 / 11.9)
         auto k = lap_geom_kernel<DIM, P, 1, DIM + 1>;
         launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, a.C), kBlock, 0, s, a);

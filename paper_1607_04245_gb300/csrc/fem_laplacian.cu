@@ -15,7 +15,6 @@
 #include <algorithm>
 
 #include "fem_cell.cuh"
-#include "fem_pipe.cuh"
 
 namespace fem {
 
@@ -161,10 +160,11 @@ __device__ __forceinline__ void lap_cell(const double (&xs)[DIM + 1][DIM],
     }
 }
 
-// Direct kernel: one thread owns CPT consecutive cells and reads the cell-indexed rows
-// (or, STR, 32 apart) with (vector) loads from global memory. Used where neither the pair kernel
-// (float32 forms) nor the staged kernel (float64 form: 16-byte aligned rows, stages that fit in
-// shared memory) applies, and by the host-buffer path, which reads page-locked host memory.
+// Direct kernel: one thread owns CPT consecutive cells (or, STR, 32 apart) and reads the
+// cell-indexed rows with (vector) loads from global memory. The float64 form's kernel, with one
+// cell per thread; in the float32 forms, used where the pair kernel does not apply (rows
+// misaligned by their base pointers, odd counts with other rules); and, with four cells, for
+// float64 rows in page-locked host memory.
 template <int DIM, int P, int CPT, int NQ, bool ADJ, bool STR = false>
 __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ LapArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
@@ -388,18 +388,22 @@ __global__ void __launch_bounds__(kBlock) lap_fields_kernel(const __grid_constan
 
 template <int DIM, int P>
 static fem_status launch_fields(const FieldsArgs &fa, bool vec, cudaStream_t s) {
-    // float64 keeps two cells per thread (the geometry of four would crowd the registers)
-    constexpr int CPTV = P == FEM_FP64 ? 2 : 4;
     constexpr int NQN = DIM == 3 ? 4 : 3;  // the workloads' rules
-    if (vec && fa.a.w.nq == NQN) {
-        // float32 forms: one wave of resident CTAs (8 fields: 69.5 -> 68.0 us per step)
-        auto k = lap_fields_kernel<DIM, P, CPTV, NQN>;
-        const int64_t n = (fa.a.C + CPTV - 1) / CPTV;
-        const void *kp = reinterpret_cast<const void *>(k);
-        launch_overlapped(k, P == FEM_FP64 ? grid_for(n, kBlock, kp) : resident_grid(kp, kBlock, n), kBlock, 0, s, fa);
-    } else if (P != FEM_FP64 && fa.a.w.nq == NQN) {
-        // ragged rows, float32 forms: two cells per thread, 32 apart (four fields, 999,999 cells:
-        // 3D 35.0 -> 27.6 us, 2D 27.9 -> 22.6 us against one cell with the run-time rule)
+    if constexpr (P == FEM_FP64) {
+        if (fa.a.w.nq == NQN) {
+            auto k = lap_fields_kernel<DIM, P, 1, NQN>;
+            launch_overlapped(k, warp_ctas(fa.a.C), kWarpCta, 0, s, fa);
+        } else {
+            auto k = lap_fields_kernel<DIM, P, 1, 0>;
+            launch_overlapped(k, warp_ctas(fa.a.C), kWarpCta, 0, s, fa);
+        }
+    } else if (vec && fa.a.w.nq == NQN) {
+        // one wave of resident CTAs (8 fields: 69.5 -> 68.0 us per step)
+        auto k = lap_fields_kernel<DIM, P, 4, NQN>;
+        launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, fa.a.C / 4), kBlock, 0, s, fa);
+    } else if (fa.a.w.nq == NQN) {
+        // ragged rows: two cells per thread, 32 apart (four fields, 999,999 cells: 3D 35.0 -> 27.6
+        // us, 2D 27.9 -> 22.6 us against one cell with the run-time rule)
         auto k = lap_fields_kernel<DIM, P, 2, NQN, true>;
         launch_overlapped(k, resident_grid(reinterpret_cast<const void *>(k), kBlock, Cells<2, true>::groups(fa.a.C)), kBlock, 0, s, fa);
     } else {
@@ -510,9 +514,9 @@ __device__ __forceinline__ void lap_pair(const double *const (&X)[DIM], const ui
 // recomputed in float64 out of line (lap_fallback_store) after its pair's stores.
 //
 // Measured on the 1,572,864-tet workload (L2 flushed, CUDA events): 25.9 us against
-// 27.8 us for the bulk-copy staged kernel with the same per-cell arithmetic (bitwise the
-// same results): the staged kernel's pipeline fill costs more than its prefetching saves
-// at this size; at 2^23 cells the two are within 1 %. Both are bound by the latency of
+// 27.8 us for a persistent kernel that staged the rows with bulk copies (bitwise the
+// same results): its pipeline fill cost more than its prefetching saved at this size; at
+// 2^23 cells the two were within 1 %. Both are bound by the latency of
 // the 16 vertex gathers per cell and by the integer float64 -> float32 splits (ALU pipe
 // half busy), not by DRAM (30 % of peak over the launch).
 // The mixed form and the adjoint run 3 CTAs per SM at up to 80 registers: with launches
@@ -714,196 +718,41 @@ __global__ void __launch_bounds__(kBlock, 3) lap_rec_kernel(const __grid_constan
     report_mesh(a.err, vmax, a.V, false);
 }
 
-// Staged Laplacian kernel (the chunk loop of fem_pipe.cuh): each consumer thread owns kCPT
-// consecutive cells of a chunk, with vector shared-memory reads of every row, vector
-// streaming stores of every output row, and (float32 forms) the cells processed as f32x2
-// pairs. NQ > 0 fixes the quadrature size at compile time; NQ = 0 reads it from the
-// arguments.
-template <class T>
-__host__ __device__ constexpr uint32_t lap_stage_bytes(int nb, int nq, bool adj) {
-    return uint32_t(kTile) * (4u * nb + uint32_t(sizeof(T)) * (nq + (adj ? nb : 0)));
-}
-
-// Streaming stores of kCPT consecutive cells starting at cell c: element vectors and
-// (adjoint) dK = w_q * factor.
+// host_rows: the cell-indexed rows lie in page-locked host memory and are reached across the
+// host link
 template <int DIM, int P, bool ADJ>
-__device__ __forceinline__ void store_cells(const LapArgs &a, int nq, int64_t c, const val_t<P> (&r)[DIM + 1][kCPT],
-                                            const val_t<P> (&tfv)[kCPT]) {
-    using T = val_t<P>;
-    const int64_t C = a.C;
-    T *__restrict__ out = static_cast<T *>(a.out);
-#pragma unroll
-    for (int b = 0; b <= DIM; ++b) store_row<kCPT>(out + b * C + c, r[b]);
-    if constexpr (ADJ) {
-        T *__restrict__ dK = static_cast<T *>(a.dK);
-        for (int q = 0; q < nq; ++q) {
-            const T wq = weight<P>(a.w, q);
-            T row[kCPT];
-#pragma unroll
-            for (int i = 0; i < kCPT; ++i) row[i] = wq * tfv[i];
-            store_row<kCPT>(dK + q * C + c, row);
-        }
-    }
-}
-
-// The consumer work of one chunk (float64 form): thread j0/kCPT's cells j0 .. j0+kCPT-1 of
-// the chunk starting at cell c0, rows read from one shared-memory stage.
-template <int DIM, int P, int NQ, bool ADJ>
-__device__ __forceinline__ void lap_chunk(const LapArgs &a, const double *const (&X)[DIM], int nq,
-                                          const int32_t *sc, const val_t<P> *sK, const val_t<P> *sL, int j0,
-                                          int64_t c0, uint32_t &vmax, bool &bad_det) {
-    static_assert(P == FEM_FP64, "the float32 forms take the pair kernel");
-    constexpr int NB = DIM + 1;
-    using T = val_t<P>;
-    const T *__restrict__ u = static_cast<const T *>(a.u);
-    uint32_t v[kCPT][NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        int32_t id[kCPT];
-        lds_row<kCPT>(sc + b * kTile + j0, id);
-#pragma unroll
-        for (int c = 0; c < kCPT; ++c) v[c][b] = clamp_vid(id[c], a.V, vmax);
-    }
-    T lv[kCPT][NB];
-    if constexpr (ADJ) {
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            T lr[kCPT];
-            lds_row<kCPT>(sL + b * kTile + j0, lr);
-#pragma unroll
-            for (int c = 0; c < kCPT; ++c) lv[c][b] = lr[c];
-        }
-    }
-    T r[NB][kCPT], tfv[kCPT];
-    qsum_t<P> ks[kCPT];
-#pragma unroll(NQ > 0 ? NQ : 1)
-    for (int q = 0; q < nq; ++q) {
-        T kr[kCPT];
-        lds_row<kCPT>(sK + q * kTile + j0, kr);
-#pragma unroll
-        for (int c = 0; c < kCPT; ++c) {
-            if (q == 0) ks[c].first(weight<P>(a.w, 0), kr[c]);
-            else ks[c].add(weight<P>(a.w, q), kr[c]);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < kCPT; ++c) {
-        double xs[NB][DIM];
-        T uu[NB], rr[NB], tf = T(0), ll[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            uu[b] = ld_gather(u + v[c][b]);
-            ll[b] = ADJ ? lv[c][b] : T(0);
-        }
-        gather_coords<DIM>(X, v[c], xs);
-        lap_cell<DIM, P, ADJ>(xs, uu, ll, ks[c], a.tau2, rr, tf, ids_repeat<NB>(v[c]), bad_det);
-#pragma unroll
-        for (int b = 0; b < NB; ++b) r[b][c] = rr[b];
-        tfv[c] = tf;
-    }
-    store_cells<DIM, P, ADJ>(a, nq, c0 + j0, r, tfv);
-}
-
-template <int DIM, int P, int NQ, bool ADJ>
-__global__ void __launch_bounds__(kStagedThreads, FEM_STAGED_MIN_CTAS)
-    lap_staged_kernel(const __grid_constant__ LapArgs a, int stages, unsigned *err) {
-    pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
-    constexpr int NB = DIM + 1;
-    using T = val_t<P>;
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int64_t C = a.C;
-    const int nq = NQ > 0 ? NQ : a.w.nq;
-    const uint32_t stage_bytes = lap_stage_bytes<T>(NB, nq, ADJ);
-    // stage layout: conn[NB][kTile] int32 | K[nq][kTile] T | lambda[NB][kTile] T
-    auto stage_conn = [&](int s) { return reinterpret_cast<int32_t *>(smem + size_t(s) * stage_bytes); };
-    auto stage_K = [&](int s) { return reinterpret_cast<T *>(stage_conn(s) + NB * kTile); };
-    auto stage_lam = [&](int s) { return stage_K(s) + nq * kTile; };
-    const double *X[DIM];
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) X[k] = a.X[k];
-    const uint64_t pol = l2_evict_first_policy();
-    uint32_t vmax = 0;     // largest vertex id seen by this consumer thread
-    bool bad_det = false;  // a cell with det J = 0 or non-finite (float64 form)
-    staged_chunks(
-        C, stages, err,
-        [&](int s, int64_t c0, uint32_t n, uint64_t *bar) {
-            const T *K = static_cast<const T *>(a.K);
-            const T *L = static_cast<const T *>(a.lam);
-            mbar_arrive_expect_tx(bar, n * (4u * NB + uint32_t(sizeof(T)) * (nq + (ADJ ? NB : 0))));
-            for (int b = 0; b < NB; ++b) bulk_copy_g2s(stage_conn(s) + b * kTile, a.conn + b * C + c0, n * 4u, bar, pol);
-            for (int q = 0; q < nq; ++q)
-                bulk_copy_g2s(stage_K(s) + q * kTile, K + q * C + c0, n * uint32_t(sizeof(T)), bar, pol);
-            if constexpr (ADJ) {
-                for (int b = 0; b < NB; ++b)
-                    bulk_copy_g2s(stage_lam(s) + b * kTile, L + b * C + c0, n * uint32_t(sizeof(T)), bar, pol);
-            }
-        },
-        [&](int s, int64_t c0, int j0) {
-            lap_chunk<DIM, P, NQ, ADJ>(a, X, nq, stage_conn(s), stage_K(s), stage_lam(s), j0, c0, vmax, bad_det);
-        });
-    report_mesh(err, vmax, a.V, bad_det);
-}
-
-template <int DIM, int P, int NQ, bool ADJ>
-static fem_status launch_staged(const LapArgs &a, uint32_t sb, cudaStream_t s) {
-    auto k = lap_staged_kernel<DIM, P, NQ, ADJ>;
-    const int stages = ring_stages(sb);
-    const size_t smem = size_t(stages) * sb;
-    unsigned *err = device_error_word();
-    if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
-    int grid = 0;
-    fem_status st = staged_grid(reinterpret_cast<const void *>(k), kStagedThreads, smem, (a.C + kTile - 1) / kTile, grid);
-    if (st != FEM_OK) return st;
-    launch_overlapped(k, grid, kStagedThreads, smem, s, a, stages, err);
-    return FEM_OK;
-}
-
-template <int DIM, int P, bool ADJ>
-static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_t s, bool staged_ok = true) {
-    using T = val_t<P>;
-    const uint32_t sb = lap_stage_bytes<T>(DIM + 1, a.w.nq, ADJ);
-    fem_status st = FEM_OK;
+static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_t s, bool host_rows) {
+    constexpr const char *kName = ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian";
     // the quadrature size of the workloads' rules (3 points in 2D, 4 in 3D) is compiled in
-    const bool native_nq = (DIM == 3 && a.w.nq == 4) || (DIM == 2 && a.w.nq == 3);
+    const bool native_nq = a.w.nq == DIM + 1;
     if constexpr (P == FEM_FP64) {
-        // few cells: 1024-cell tiles would leave most SMs idle while the float64 pipe, not
-        // memory, bounds the launch, so the cells are spread over every SM (one per thread)
-        const int64_t sms = sm_count();
-        if ((a.C + kTile - 1) / kTile < sms) {
-            const int64_t per = (a.C + 2 * sms - 1) / (2 * sms);
-            int block = static_cast<int>((per + 31) / 32 * 32);
-            block = block < 32 ? 32 : (block > kBlock ? kBlock : block);
-            const unsigned grid = static_cast<unsigned>((a.C + block - 1) / block);
-            if (native_nq) launch_overlapped((lap_kernel<DIM, P, 1, DIM + 1, ADJ>), grid, block, 0, s, a);
-            else launch_overlapped((lap_kernel<DIM, P, 1, 0, ADJ>), grid, block, 0, s, a);
-            return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
+        // one cell per thread, 3D 1,572,864 / 200,000 tets: residual 212 -> 191.5 / 40.6 -> 27.2 us,
+        // adjoint 301 -> 273 / 60.7 -> 42.6, against a persistent kernel that staged 1024-cell
+        // chunks with bulk copies (its last round of chunks left SMs idle: 5.05 chunks a CTA)
+        if (!(host_rows && vec)) {
+            if (native_nq) {
+                auto k = lap_kernel<DIM, P, 1, DIM + 1, ADJ>;
+                launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+            } else {
+                auto k = lap_kernel<DIM, P, 1, 0, ADJ>;
+                launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+            }
+            return check_launch(kName);
         }
-    }
-    if constexpr (P != FEM_FP64) {
-        // float32 forms: the pair kernel (the bulk-copy staged kernel is the float64 form's).
-        // Its plain 8-byte loads also serve rows in page-locked host memory (staged_ok
-        // false): from host buffers 0.309 against 0.331 ms per step with lap_kernel.
+    } else {
+        // the pair kernel; its plain 8-byte loads also serve host rows: from host buffers 0.309
+        // against 0.331 ms per step with lap_kernel
         if (pairs) {
             if (native_nq) launch_pair<DIM, P, DIM + 1, ADJ, false>(a, s);
             else launch_pair<DIM, P, 0, ADJ, false>(a, s);
-            return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
+            return check_launch(kName);
         }
         // an odd cell count (every second row starts between 8-byte words): the same pairs from
         // cells 32 apart, single-value accesses (999,999 tets: 23.8 -> 17.0 us, the adjoint 45.7
         // -> 36.7, against one cell per thread; an even count takes 14.8: twice the row accesses)
         if (a.C % 2 != 0 && native_nq) {
             launch_pair<DIM, P, DIM + 1, ADJ, true>(a, s);
-            return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
-        }
-    }
-    if constexpr (P == FEM_FP64) {
-        if (staged_ok && vec && 2u * sb <= kStageMax) {
-            if (a.w.nq == DIM + 1 && DIM == 3) st = launch_staged<DIM, P, 4, ADJ>(a, sb, s);
-            else if (a.w.nq == 3 && DIM == 2) st = launch_staged<DIM, P, 3, ADJ>(a, sb, s);
-            else st = launch_staged<DIM, P, 0, ADJ>(a, sb, s);
-            if (st != FEM_OK) return st;
-            return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
+            return check_launch(kName);
         }
     }
     if (vec && native_nq) {
@@ -914,9 +763,9 @@ static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_
         auto k = lap_kernel<DIM, P, 4, 0, ADJ>;
         int grid = grid_for((a.C + 3) / 4, kBlock, reinterpret_cast<const void *>(k));
         launch_overlapped(k, grid, kBlock, 0, s, a);
-    } else if (P != FEM_FP64 && native_nq) {
-        // rows misaligned by their base pointers: two cells per thread, 32 apart (10^6 tets: 23.4 ->
-        // 17.8 us against one cell with the run-time rule, bitwise the same results)
+    } else if (native_nq) {
+        // float32 rows misaligned by their base pointers: two cells per thread, 32 apart (10^6
+        // tets: 23.4 -> 17.8 us against one cell with the run-time rule, bitwise the same results)
         auto k = lap_kernel<DIM, P, 2, DIM + 1, ADJ, true>;
         int grid = grid_for(Cells<2, true>::groups(a.C), kBlock, reinterpret_cast<const void *>(k));
         launch_overlapped(k, grid, kBlock, 0, s, a);
@@ -925,28 +774,28 @@ static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_
         int grid = grid_for(a.C, kBlock, reinterpret_cast<const void *>(k));
         launch_overlapped(k, grid, kBlock, 0, s, a);
     }
-    return check_launch(ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian");
+    return check_launch(kName);
 }
 
 // vec: every cell-indexed row 16-byte aligned (C % 4 == 0); the pair kernel needs 8 bytes
 template <bool ADJ>
 static fem_status dispatch_lap(int dim, fem_precision prec, const LapArgs &args, bool vec, cudaStream_t s,
-                               bool staged_ok = true) {
+                               bool host_rows = false) {
     LapArgs a = args;
     if (!(a.err = device_error_word())) return fail(FEM_ERR_CUDA, "device error word unavailable");
     const bool pairs = a.C % 2 == 0 && aligned8(a.conn) && aligned8(a.K) && aligned8(a.out) &&
                        (!ADJ || (aligned8(a.lam) && aligned8(a.dK)));
     if (dim == 2) {
         switch (prec) {
-            case FEM_FP64: return launch_lap<2, FEM_FP64, ADJ>(a, vec, pairs, s, staged_ok);
-            case FEM_FP32_MIXED: return launch_lap<2, FEM_FP32_MIXED, ADJ>(a, vec, pairs, s, staged_ok);
-            case FEM_FP32: return launch_lap<2, FEM_FP32, ADJ>(a, vec, pairs, s, staged_ok);
+            case FEM_FP64: return launch_lap<2, FEM_FP64, ADJ>(a, vec, pairs, s, host_rows);
+            case FEM_FP32_MIXED: return launch_lap<2, FEM_FP32_MIXED, ADJ>(a, vec, pairs, s, host_rows);
+            case FEM_FP32: return launch_lap<2, FEM_FP32, ADJ>(a, vec, pairs, s, host_rows);
         }
     } else {
         switch (prec) {
-            case FEM_FP64: return launch_lap<3, FEM_FP64, ADJ>(a, vec, pairs, s, staged_ok);
-            case FEM_FP32_MIXED: return launch_lap<3, FEM_FP32_MIXED, ADJ>(a, vec, pairs, s, staged_ok);
-            case FEM_FP32: return launch_lap<3, FEM_FP32, ADJ>(a, vec, pairs, s, staged_ok);
+            case FEM_FP64: return launch_lap<3, FEM_FP64, ADJ>(a, vec, pairs, s, host_rows);
+            case FEM_FP32_MIXED: return launch_lap<3, FEM_FP32_MIXED, ADJ>(a, vec, pairs, s, host_rows);
+            case FEM_FP32: return launch_lap<3, FEM_FP32, ADJ>(a, vec, pairs, s, host_rows);
         }
     }
     return fail(FEM_ERR_ARG, "unknown precision %d", static_cast<int>(prec));
@@ -1037,8 +886,7 @@ extern "C" fem_status fem_integrate_laplacian_fields(int dim, int64_t n_cells, i
 }
 
 namespace fem {
-// The residual with plain (vector) loads and stores only -- never the bulk-copy staged
-// kernel -- for connectivity, coefficient and output arrays that live in page-locked host
+// The residual for connectivity, coefficient and output arrays that live in page-locked host
 // memory and are reached across the host link (fem_integrate_laplacian_host, chunks = 0).
 fem_status integrate_laplacian_plain(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
                                      const int32_t *conn, const void *u, const void *K, int n_q, const double *qpts,
@@ -1048,7 +896,7 @@ fem_status integrate_laplacian_plain(int dim, int64_t n_cells, int64_t n_verts, 
     if (st != FEM_OK || n_cells == 0) return st;
     a.out = elem_out;
     const bool vec = n_cells % 4 == 0 && aligned16(conn) && aligned16(K) && aligned16(elem_out);
-    return dispatch_lap<false>(dim, prec, a, vec, stream, false);
+    return dispatch_lap<false>(dim, prec, a, vec, stream, true);
 }
 
 fem_status launch_gather(int dim, int n_comp, int64_t C, int64_t V, const void *elem, const int32_t *node_ptr,

@@ -70,9 +70,7 @@ extern "C" fem_status fem_adjoint_laplacian_noalloc(int dim, int64_t n_cells, in
     fem_status st = noalloc_scratch(&scratch);
     if (st != FEM_OK) return st;
     // Every workspace entry the gather reads is written by the element kernel earlier in
-    // this same call, so nothing has to be cleared between calls -- unless a staged element
-    // kernel gave up a bounded wait (FEM_ERR_TIMEOUT from fem_device_error): it then skips
-    // that tile's writes, and du mixes in the previous call's values; the header says so.
+    // this same call, so nothing has to be cleared between calls.
     return fem_adjoint_laplacian(dim, n_cells, n_verts, coords, conn, u, K, n_q, qpts, qw, lambda, dK, du, node_ptr,
                                  node_idx, scratch, prec, stream);
 }

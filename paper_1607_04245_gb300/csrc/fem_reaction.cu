@@ -311,15 +311,18 @@ __global__ void __launch_bounds__(kBlock, rd_min_blocks<DIM, P, CPT>()) rd_kerne
 template <int DIM, int P, bool A_P1, bool REACT, bool DRIFT>
 static void launch_rd_one(const RdArgs &a, bool vec4, bool vec2, cudaStream_t s) {
     constexpr int NQN = DIM + 1 == 4 ? 4 : 3;  // the workloads' rules: 3 points in 2D, 4 in 3D
-    // float32 forms: two cells per thread in 3D, four in 2D (rd_min_blocks); the float64 form
-    // is bound by the float64 pipe and keeps one cell per thread (four cost it occupancy: 457
-    // against 416 us on the 1,572,864-tet workload)
+    // float32 forms: two cells per thread in 3D, four in 2D (rd_min_blocks). float64: one, with
+    // the rule read at run time (380 us on the 1,572,864-tet workload against 386 with it
+    // compiled in)
     constexpr int CPTV = DIM == 3 ? 2 : 4;
     const bool vec = CPTV == 2 ? vec2 : vec4;
-    if (P != FEM_FP64 && vec && a.w.nq == NQN) {
+    if constexpr (P == FEM_FP64) {
+        auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, 1, 0>;
+        launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+    } else if (vec && a.w.nq == NQN) {
         auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, CPTV, NQN>;
         launch_overlapped(k, grid_for((a.C + CPTV - 1) / CPTV, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
-    } else if (P != FEM_FP64 && a.w.nq == NQN) {
+    } else if (a.w.nq == NQN) {
         // ragged rows: the same cells per thread, 32 apart (999,999 cells: 3D 44.2 -> 21.2 us, 2D
         // 35.8 -> 13.6 us against one cell with the run-time rule, whose values per point go
         // through local memory)
