@@ -409,8 +409,40 @@ struct NodeSum<float> {
     __device__ __forceinline__ float value() const { return s + c; }
 };
 
-// list entries whose loads a gather keeps in flight at once
-constexpr int kGatherBatch = 8;
+// Sums of the element vectors' entries idx[b .. e) (entry t = NB cell + a stands for row
+// a * NCOMP + k, cell `cell`, of elem) into acc[k], one by one in list order. The loads of eight
+// entries are in flight together, of a remainder those of four, two and one: each batch costs two
+// dependent loads' latency, and a remainder taken entry by entry up to seven times that (triangles'
+// lists have 6 entries: 1,000,000 / 50,000 cells, two float32 components, 10.7 -> 9.9 / 2.8 -> 2.6 us).
+template <int NB, int NCOMP, int N, class T>
+__device__ __forceinline__ void gather_batch(const T *__restrict__ elem, const int32_t *__restrict__ idx, int64_t C,
+                                             NodeSum<T> (&acc)[NCOMP]) {
+    int32_t t[N];
+    T val[N][NCOMP];
+#pragma unroll
+    for (int i = 0; i < N; ++i) t[i] = __ldg(idx + i);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int k = 0; k < NCOMP; ++k) {
+            const int32_t cell = t[i] / NB, a = t[i] - cell * NB;
+            val[i][k] = __ldg(elem + int64_t(a * NCOMP + k) * C + cell);
+        }
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int k = 0; k < NCOMP; ++k) acc[k].add(val[i][k]);
+}
+
+template <int NB, int NCOMP, class T>
+__device__ __forceinline__ void gather_list(const T *__restrict__ elem, const int32_t *__restrict__ idx, int32_t b,
+                                            int32_t e, int64_t C, NodeSum<T> (&acc)[NCOMP]) {
+    int32_t j = b;
+    for (; j + 8 <= e; j += 8) gather_batch<NB, NCOMP, 8>(elem, idx + j, C, acc);
+    if (j + 4 <= e) gather_batch<NB, NCOMP, 4>(elem, idx + j, C, acc), j += 4;
+    if (j + 2 <= e) gather_batch<NB, NCOMP, 2>(elem, idx + j, C, acc), j += 2;
+    if (j < e) gather_batch<NB, NCOMP, 1>(elem, idx + j, C, acc);
+}
 
 template <int P>
 using qsum_t = typename std::conditional<P == FEM_FP64, PlainSum<double>,

@@ -176,6 +176,12 @@ __device__ __forceinline__ double widen(float x) {
 
 __device__ __forceinline__ double df_to_double(dfl a) { return widen(a.hi) + widen(a.lo); }
 
+// Threads per CTA: 128 against 256 (steps back to back, us): 2,097,152 tets, Laplacian 83.4 ->
+// 79.2, elasticity 167.6 -> 159.3, adjoint 144 -> 137; 50,000 tets 5.2 -> 4.6, 8.4 -> 7.3, 11.4 ->
+// 10.6 (a launch ends and small ones spread more evenly). 64 threads are the same, 32 lose
+// occupancy in 2D (32 CTAs an SM at most).
+constexpr int kDfBlock = 128;
+
 struct DfArgs {
     const double *X[3];
     const int32_t *conn;
@@ -189,7 +195,7 @@ struct DfArgs {
 };
 
 template <int DIM>
-__global__ void __launch_bounds__(kBlock, 5) lap_df_kernel(const __grid_constant__ DfArgs a) {
+__global__ void __launch_bounds__(kDfBlock, 10) lap_df_kernel(const __grid_constant__ DfArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
     constexpr int NB = DIM + 1;
@@ -263,10 +269,10 @@ fem_status launch_lap_df(int dim, int64_t n_cells, int64_t n_verts, const double
     for (int q = 0; q < FEM_MAX_QPTS; ++q) a.wd[q] = q < n_q ? qw[q] : 0.0;
     if (dim == 2) {
         auto k = lap_df_kernel<2>;
-        launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, stream, a);
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, stream, a);
     } else {
         auto k = lap_df_kernel<3>;
-        launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, stream, a);
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, stream, a);
     }
     return check_launch("fem_integrate_laplacian (FEM_FP64_DF)");
 }
@@ -288,13 +294,13 @@ struct DfElArgs {
     float whi[FEM_MAX_QPTS], wlo[FEM_MAX_QPTS];
 };
 
-// 3D: 4 CTAs per SM at up to 64 registers (73 unbounded, 3 CTAs: 190.3 -> 167.6 us on 2^21
-// tets, steps back to back; 5 CTAs spill); 2D stays unbounded (59 registers, 4 CTAs).
+// 3D: 32 warps per SM at up to 64 registers (73 unbounded, 24 warps: 190.3 -> 167.6 us on 2^21
+// tets with CTAs of 256, steps back to back; 40 warps spill); 2D stays unbounded (59 registers).
 template <int DIM>
-constexpr int el_df_min_blocks() { return DIM == 3 ? 4 : 0; }  // 0: no minimum
+constexpr int el_df_min_blocks() { return DIM == 3 ? 8 : 0; }  // 0: no minimum
 
 template <int DIM>
-__global__ void __launch_bounds__(kBlock, el_df_min_blocks<DIM>()) el_df_kernel(const __grid_constant__ DfElArgs a) {
+__global__ void __launch_bounds__(kDfBlock, el_df_min_blocks<DIM>()) el_df_kernel(const __grid_constant__ DfElArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
     constexpr int NB = DIM + 1;
@@ -387,10 +393,10 @@ fem_status launch_el_df(int dim, int64_t n_cells, int64_t n_verts, const double 
     }
     if (dim == 2) {
         auto k = el_df_kernel<2>;
-        launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, stream, a);
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, stream, a);
     } else {
         auto k = el_df_kernel<3>;
-        launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, stream, a);
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, stream, a);
     }
     return check_launch("fem_integrate_elasticity (FEM_FP64_DF)");
 }
@@ -412,7 +418,7 @@ struct DfAdjArgs {
 };
 
 template <int DIM>
-__global__ void __launch_bounds__(kBlock) adj_df_kernel(const __grid_constant__ DfAdjArgs a) {
+__global__ void __launch_bounds__(kDfBlock) adj_df_kernel(const __grid_constant__ DfAdjArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
     constexpr int NB = DIM + 1;
@@ -490,10 +496,10 @@ fem_status launch_adj_df(int dim, int64_t n_cells, int64_t n_verts, const double
     }
     if (dim == 2) {
         auto k = adj_df_kernel<2>;
-        launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, stream, a);
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, stream, a);
     } else {
         auto k = adj_df_kernel<3>;
-        launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, stream, a);
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, stream, a);
     }
     return check_launch("fem_adjoint_laplacian (FEM_FP64_DF)");
 }

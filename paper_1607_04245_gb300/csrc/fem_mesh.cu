@@ -170,59 +170,44 @@ __global__ void gather_kernel(int64_t C, int64_t V, const T *__restrict__ elem, 
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
     pdl_trigger();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    auto entry = [&](int32_t t, int k) {
-        const int32_t cell = t / NB, a = t - cell * NB;
-        return __ldg(elem + int64_t(a * NCOMP + k) * C + cell);
-    };
     for (int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; n < V; n += stride) {
-        const int32_t b = ptr[n], e = ptr[n + 1];
-        NodeSum<T> acc[NCOMP];
-        // kGatherBatch list entries at a time: their loads are independent and in flight
-        // together; the sums still take the entries one by one in list order. (A warp
-        // reading 32 vertices' lists together with coalesced loads and summing from shared
+        // (A warp reading 32 vertices' lists together with coalesced loads and summing from shared
         // memory was slower: 60.4 against 48.8 us for the adjoint on 1,572,864 tets.)
-        int32_t j = b;
-        for (; j + kGatherBatch <= e; j += kGatherBatch) {
-            int32_t t[kGatherBatch];
-            T val[kGatherBatch][NCOMP];
-#pragma unroll
-            for (int i = 0; i < kGatherBatch; ++i) t[i] = __ldg(idx + j + i);
-#pragma unroll
-            for (int i = 0; i < kGatherBatch; ++i)
-#pragma unroll
-                for (int k = 0; k < NCOMP; ++k) val[i][k] = entry(t[i], k);
-#pragma unroll
-            for (int i = 0; i < kGatherBatch; ++i)
-#pragma unroll
-                for (int k = 0; k < NCOMP; ++k) acc[k].add(val[i][k]);
-        }
-        for (; j < e; ++j) {
-            const int32_t t = __ldg(idx + j);
-#pragma unroll
-            for (int k = 0; k < NCOMP; ++k) acc[k].add(entry(t, k));
-        }
+        NodeSum<T> acc[NCOMP];
+        gather_list<NB, NCOMP>(elem, idx, ptr[n], ptr[n + 1], C, acc);
 #pragma unroll
         for (int k = 0; k < NCOMP; ++k) out[k * V + n] = acc[k].value();
     }
 }
 
+// Large 3D meshes (lists of 24 entries, more than 512 vertices per SM) in one-warp CTAs, which
+// hold 1024 threads to an SM: with all 2048 the sectors that neighbouring vertices' lists share
+// are gone from L1 before their second use (1,000,000 tets, one component 14.6 -> 11.1 us in
+// float32, 21.3 -> 15.7 in float64; three 26.5 -> 22.9, 53.3 -> 36.7; 400,000 tets 7.4 -> 8.8 in
+// float32, so not there). Small meshes (at most 128 vertices per SM)
+// in CTAs of 128 threads (50,000 tets, three components, float64: 8.3 -> 7.2 us against 256). 2D lists (6 entries) want full occupancy: one-warp CTAs take 35
+// against 19.5 us on 2,097,152 triangles. Rejected: list indices by 16-byte loads (no change in
+// 3D, 22-60 % slower in 2D), 12 or 24 entries in flight, larger CTAs.
 template <int NB, class T>
 static void launch_gather_t(int n_comp, int64_t C, int64_t V, const void *elem, const int32_t *ptr,
                             const int32_t *idx, void *out, cudaStream_t s) {
     const T *el = static_cast<const T *>(elem);
     T *o = static_cast<T *>(out);
+    const int64_t sms = sm_count();
+    const unsigned cta = NB == 4 && V > 512 * sms ? kWarpCta : (V > 128 * sms ? kBlock : 128);
+    const unsigned grid = static_cast<unsigned>((V + cta - 1) / cta);
     switch (n_comp) {
         case 1: {
             auto k = gather_kernel<NB, 1, T>;
-            launch_overlapped(k, grid_for(V, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, C, V, el, ptr, idx, o);
+            launch_overlapped(k, grid, cta, 0, s, C, V, el, ptr, idx, o);
         } break;
         case 2: {
             auto k = gather_kernel<NB, 2, T>;
-            launch_overlapped(k, grid_for(V, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, C, V, el, ptr, idx, o);
+            launch_overlapped(k, grid, cta, 0, s, C, V, el, ptr, idx, o);
         } break;
         default: {
             auto k = gather_kernel<NB, 3, T>;
-            launch_overlapped(k, grid_for(V, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, C, V, el, ptr, idx, o);
+            launch_overlapped(k, grid, cta, 0, s, C, V, el, ptr, idx, o);
         } break;
     }
 }

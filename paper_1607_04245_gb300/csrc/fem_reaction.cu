@@ -308,6 +308,10 @@ __global__ void __launch_bounds__(kBlock, rd_min_blocks<DIM, P, CPT>()) rd_kerne
     report_mesh(a.err, vmax, a.V, bad_det);
 }
 
+// CTAs of 128 threads for the float32 forms, on one wave of resident CTAs in 2D (2,097,152 cells:
+// 3D 35.4 -> 34.6 us, one wave 37.3; 2D 28.1 -> 24.1 us, up to eight waves 26.6)
+constexpr int kRdBlock = 128;
+
 template <int DIM, int P, bool A_P1, bool REACT, bool DRIFT>
 static void launch_rd_one(const RdArgs &a, bool vec4, bool vec2, cudaStream_t s) {
     constexpr int NQN = DIM + 1 == 4 ? 4 : 3;  // the workloads' rules: 3 points in 2D, 4 in 3D
@@ -321,13 +325,17 @@ static void launch_rd_one(const RdArgs &a, bool vec4, bool vec2, cudaStream_t s)
         launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
     } else if (vec && a.w.nq == NQN) {
         auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, CPTV, NQN>;
-        launch_overlapped(k, grid_for((a.C + CPTV - 1) / CPTV, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
+        const int64_t n = (a.C + CPTV - 1) / CPTV;
+        const void *kp = reinterpret_cast<const void *>(k);
+        launch_overlapped(k, DIM == 2 ? resident_grid(kp, kRdBlock, n) : grid_for(n, kRdBlock, kp), kRdBlock, 0, s, a);
     } else if (a.w.nq == NQN) {
         // ragged rows: the same cells per thread, 32 apart (999,999 cells: 3D 44.2 -> 21.2 us, 2D
         // 35.8 -> 13.6 us against one cell with the run-time rule, whose values per point go
         // through local memory)
         auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, CPTV, NQN, true>;
-        launch_overlapped(k, grid_for(Cells<CPTV, true>::groups(a.C), kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
+        const int64_t n = Cells<CPTV, true>::groups(a.C);
+        const void *kp = reinterpret_cast<const void *>(k);
+        launch_overlapped(k, DIM == 2 ? resident_grid(kp, kRdBlock, n) : grid_for(n, kRdBlock, kp), kRdBlock, 0, s, a);
     } else {
         auto k = rd_kernel<DIM, P, A_P1, REACT, DRIFT, 1, 0>;
         launch_overlapped(k, grid_for(a.C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);

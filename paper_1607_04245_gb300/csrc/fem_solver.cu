@@ -342,36 +342,11 @@ __global__ void __launch_bounds__(256) cg_apply_dots_kernel(int64_t C, int64_t V
     constexpr bool F32 = std::is_same<T, float>::value;
     __shared__ double sh[F32 ? 1 : 3 * 256];
     __shared__ float2 sh2[3 * 8];
-    // list entry t = NB cell + a: element row (a, component k)
-    auto entry = [&](int32_t t, int k) {
-        const int32_t cell = t / NB, a = t - cell * NB;
-        return __ldg(elem + int64_t(a * NCOMP + k) * C + cell);
-    };
     double ru = 0.0, wu = 0.0, rr = 0.0;  // float64 vectors
     PairSum pd[3];                         // float32 vectors: r.u, w.u, r.r
     for (int64_t n = int64_t(blockIdx.x) * 256 + threadIdx.x; n < V; n += int64_t(kDotBlocks) * 256) {
-        const int32_t b = ptr[n], e = ptr[n + 1];
         NodeSum<T> acc[NCOMP];
-        int32_t j = b;
-        for (; j + kGatherBatch <= e; j += kGatherBatch) {
-            int32_t t[kGatherBatch];
-            T val[kGatherBatch][NCOMP];
-#pragma unroll
-            for (int i = 0; i < kGatherBatch; ++i) t[i] = __ldg(idx + j + i);
-#pragma unroll
-            for (int i = 0; i < kGatherBatch; ++i)
-#pragma unroll
-                for (int k = 0; k < NCOMP; ++k) val[i][k] = entry(t[i], k);
-#pragma unroll
-            for (int i = 0; i < kGatherBatch; ++i)
-#pragma unroll
-                for (int k = 0; k < NCOMP; ++k) acc[k].add(val[i][k]);
-        }
-        for (; j < e; ++j) {
-            const int32_t t = __ldg(idx + j);
-#pragma unroll
-            for (int k = 0; k < NCOMP; ++k) acc[k].add(entry(t, k));
-        }
+        gather_list<NB, NCOMP>(elem, idx, ptr[n], ptr[n + 1], C, acc);
         const bool fx = fixed[n] != 0;
 #pragma unroll
         for (int k = 0; k < NCOMP; ++k) {
