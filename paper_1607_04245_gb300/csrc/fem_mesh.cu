@@ -46,6 +46,8 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t x, int32_t *tota
 
 // in-place inclusive scan of one tile; the tile's total goes to tile_sums[tile]
 __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(int32_t *data, int64_t n, int32_t *tile_sums) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int32_t s_total;
     const int64_t base = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanItems;
     int32_t v[kScanItems];
@@ -64,6 +66,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(int32_t *data,
 
 // exclusive scan of the tile sums in place (one CTA, chunks of a tile with a carry)
 __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(int32_t *sums, int64_t n) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int32_t s_total;
     int32_t carry = 0;
     for (int64_t c = 0; c < n; c += kScanTile) {
@@ -83,80 +87,166 @@ __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(int32_t *sums, 
     }
 }
 
-__global__ void add_offsets_kernel(int32_t *data, int64_t n, const int32_t *tile_sums) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < n) data[i] += tile_sums[i / kScanTile];
+// data[i] += the sums of the tiles before i's (summed: tile_sums holds these offsets already;
+// otherwise the CTA, one per tile, adds them up); cursor[i + 1] = data[i], cursor[0] = 0
+__global__ void __launch_bounds__(kScanThreads) add_offsets_kernel(int32_t *data, int64_t n, const int32_t *tile_sums,
+                                                                   bool summed, int32_t *cursor) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ int32_t s_total;
+    const int64_t tile = blockIdx.x;
+    int32_t off;
+    if (summed) {
+        off = tile_sums[tile];
+    } else {
+        int32_t part = 0;
+        for (int64_t t = threadIdx.x; t < tile; t += kScanThreads) part += tile_sums[t];
+        block_exclusive_scan(part, &s_total);
+        off = s_total;
+    }
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const int64_t j = tile * kScanTile + int64_t(i) * kScanThreads + threadIdx.x;
+        if (j < n) {
+            const int32_t x = data[j] + off;
+            data[j] = x;
+            if (j + 1 < n) cursor[j + 1] = x;
+        }
+    }
+    if (tile == 0 && threadIdx.x == 0) cursor[0] = 0;
 }
 
-// inclusive scan of data[0..n) with workspace tile_sums[scan_tiles_for(n)]
-static fem_status inclusive_scan(int32_t *data, int64_t n, int32_t *tile_sums, cudaStream_t s) {
-    if (n == 0) return FEM_OK;
+// data[0..n) inclusive-scanned in place, cursor[0..n) the exclusive sums; workspace
+// tile_sums[scan_tiles_for(n)]. Up to kSumTiles tiles the tiles' offsets are summed where they
+// are used, one kernel less.
+constexpr int64_t kSumTiles = 2048;
+static fem_status scan_with_cursor(int32_t *data, int64_t n, int32_t *tile_sums, int32_t *cursor, cudaStream_t s) {
     const int64_t tiles = scan_tiles_for(n);
-    scan_tiles_kernel<<<static_cast<unsigned>(tiles), kScanThreads, 0, s>>>(data, n, tile_sums);
-    scan_sums_kernel<<<1, kScanThreads, 0, s>>>(tile_sums, tiles);
-    add_offsets_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(data, n, tile_sums);
+    const unsigned grid = static_cast<unsigned>(tiles);
+    const bool summed = tiles > kSumTiles;
+    launch_overlapped(scan_tiles_kernel, grid, kScanThreads, 0, s, data, n, tile_sums);
+    if (summed) launch_overlapped(scan_sums_kernel, 1, kScanThreads, 0, s, tile_sums, tiles);
+    const int32_t *sums = tile_sums;
+    launch_overlapped(add_offsets_kernel, grid, kScanThreads, 0, s, data, n, sums, summed, cursor);
     return check_launch("scan");
 }
 
 // ------------------------------------------------------------------ vertex-to-cell lists
+//
+// zero, count, scan (two kernels), fill, sort, launched overlapped. On 524,286 tets (93,000
+// vertices; ncu, cold caches, us): count 10.3, scan 9, fill 11.7 (14 with one atomic per cell and
+// vertex), sort 12.5; the lists and the adjoint after them 66 -> 57 us with the eight-lane sort, 110
+// with the sort by one thread per vertex in local memory (41), a scan of four kernels and plain
+// launches. What bounds them is latency: of the atomics that return a place, and of the chain
+// pointer -> list -> place -> list per vertex.
 
-__global__ void count_kernel(const int32_t *conn, int64_t total, uint32_t V, int32_t *ptr1, unsigned *err) {
-    uint32_t vmax = 0;
+__global__ void __launch_bounds__(kBlock) zero_kernel(int32_t *data, int64_t n) {
+    pdl_wait();
+    pdl_trigger();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < total; j += stride)
-        atomicAdd(ptr1 + clamp_vid(conn[j], V, vmax), 1);
-    report_mesh(err, vmax, V, false);
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) data[i] = 0;
 }
 
-__global__ void copy_kernel(const int32_t *src, int32_t *dst, int64_t n) {
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) dst[i] = src[i];
+// One atomic per run of equal vertices among a warp's 32 cells (in one row): meshes that list the
+// cells of one vertex or one grid box together have such runs, and atomics on one address go one
+// by one. Lanes without a cell carry an id no vertex has. Every lane gets the old value of its
+// vertex' counter plus its place in the run.
+__device__ __forceinline__ int32_t warp_add(int32_t *counters, uint32_t v, bool in) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t w = in ? v : 0xffffffffu;
+    const uint32_t before = __shfl_up_sync(0xffffffffu, w, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || before != w);
+    const unsigned from = heads & (0xffffffffu >> (31 - lane));  // heads at or below this lane
+    const int head = 31 - __clz(from);
+    const unsigned above = heads & ~(0xffffffffu >> (31 - lane));
+    const int end = above ? __ffs(above) - 1 : 32;
+    int32_t old = 0;
+    if (in && lane == head) old = atomicAdd(counters + v, end - lane);
+    return __shfl_sync(0xffffffffu, old, head) + lane - head;
 }
 
 template <int NB>
-__global__ void fill_kernel(const int32_t *conn, int64_t C, uint32_t V, int32_t *cursor, int32_t *idx) {
-    const int a = blockIdx.y;
+__global__ void __launch_bounds__(kBlock) count_kernel(const int32_t *conn, int64_t C, uint32_t V, int32_t *ptr1,
+                                                       unsigned *err) {
+    pdl_wait();
+    pdl_trigger();
+    uint32_t vmax = 0;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < C; e += stride) {
-        const uint32_t v = clamp_vid(conn[a * C + e], V);
-        const int32_t pos = atomicAdd(cursor + v, 1);
-        idx[pos] = static_cast<int32_t>(e * NB + a);
+    const int64_t warps_end = (C + 31) / 32 * 32;  // whole warps: warp_add is a warp's work
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < warps_end; e += stride) {
+        const bool in = e < C;
+        uint32_t v[NB];
+#pragma unroll
+        for (int a = 0; a < NB; ++a) v[a] = in ? clamp_vid(conn[a * C + e], V, vmax) : 0u;
+#pragma unroll
+        for (int a = 0; a < NB; ++a) warp_add(ptr1, v[a], in);
+    }
+    report_mesh(err, vmax, V, false);
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kBlock) fill_kernel(const int32_t *conn, int64_t C, uint32_t V, int32_t *cursor,
+                                                      int32_t *idx) {
+    pdl_wait();
+    pdl_trigger();
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    const int64_t warps_end = (C + 31) / 32 * 32;
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < warps_end; e += stride) {
+        const bool in = e < C;
+        uint32_t v[NB];
+        int32_t pos[NB];
+#pragma unroll
+        for (int a = 0; a < NB; ++a) v[a] = in ? clamp_vid(conn[a * C + e], V) : 0u;
+#pragma unroll
+        for (int a = 0; a < NB; ++a) pos[a] = warp_add(cursor, v[a], in);
+        if (in)
+#pragma unroll
+            for (int a = 0; a < NB; ++a) idx[pos[a]] = static_cast<int32_t>(e * NB + a);
     }
 }
 
-// per-vertex insertion sort: the list order becomes cell order, independent of the
-// order in which the atomics above landed. Lists of up to kSortLocal entries (every
-// vertex of the workloads' meshes: 6 in 2D, up to 24 in 3D) are sorted in a per-thread
-// array and written back once; longer ones in place.
-constexpr int kSortLocal = 32;
+// Sort every vertex' list: cell order, independent of the order in which the atomics above
+// landed. G = 8 lanes per vertex (32: 20.6 us on the mesh above, 4: 13.0) bring lists of up to kSortShared
+// entries to shared memory; an entry's place is the number of smaller ones. (All entries of a
+// list are distinct.) Longer lists: insertion sort in place by one lane.
+constexpr int kSortShared = 128;
 
-__global__ void sort_segments_kernel(const int32_t *ptr, int32_t *idx, int64_t V) {
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; n < V; n += stride) {
-        const int32_t b = ptr[n], e = ptr[n + 1];
-        if (e - b <= kSortLocal) {
-            int32_t t[kSortLocal];
-            const int m = e - b;
-            for (int i = 0; i < m; ++i) t[i] = idx[b + i];
-            for (int i = 1; i < m; ++i) {
-                const int32_t x = t[i];
-                int j = i - 1;
-                while (j >= 0 && t[j] > x) {
-                    t[j + 1] = t[j];
+template <int G>
+__global__ void __launch_bounds__(kBlock) sort_segments_kernel(const int32_t *ptr, int32_t *idx, int64_t V) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ __align__(16) int32_t list[kBlock / G][kSortShared + 4];  // + 4: the groups' rows in different banks
+    const int lane = threadIdx.x % G, group = threadIdx.x / G;
+    const unsigned mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << ((threadIdx.x & 31) / G * G);
+    const int64_t stride = int64_t(gridDim.x) * (kBlock / G);
+    int32_t *s = list[group];
+    for (int64_t n = int64_t(blockIdx.x) * (kBlock / G) + group; n < V; n += stride) {
+        const int32_t b = ptr[n], m = ptr[n + 1] - b;
+        if (m <= kSortShared) {
+            // padded to a multiple of four with the largest value, which no entry exceeds
+            const int pad = (m + 3) & ~3;
+            for (int k = lane; k < pad; k += G) s[k] = k < m ? idx[b + k] : 0x7fffffff;
+            __syncwarp(mask);
+            for (int k = lane; k < m; k += G) {
+                const int32_t x = s[k];
+                int r = 0;
+                for (int j = 0; j < m; j += 4) {
+                    const int4 q = *reinterpret_cast<const int4 *>(s + j);
+                    r += (q.x < x) + (q.y < x) + (q.z < x) + (q.w < x);
+                }
+                idx[b + r] = x;
+            }
+            __syncwarp(mask);
+        } else if (lane == 0) {
+            for (int32_t i = b + 1; i < b + m; ++i) {
+                const int32_t x = idx[i];
+                int32_t j = i - 1;
+                while (j >= b && idx[j] > x) {
+                    idx[j + 1] = idx[j];
                     --j;
                 }
-                t[j + 1] = x;
+                idx[j + 1] = x;
             }
-            for (int i = 0; i < m; ++i) idx[b + i] = t[i];
-            continue;
-        }
-        for (int32_t i = b + 1; i < e; ++i) {
-            int32_t x = idx[i], j = i - 1;
-            while (j >= b && idx[j] > x) {
-                idx[j + 1] = idx[j];
-                --j;
-            }
-            idx[j + 1] = x;
         }
     }
 }
@@ -294,24 +384,39 @@ extern "C" fem_status fem_build_node2cell(int dim, int64_t n_cells, int64_t n_ve
     fem_status st;
     if (!node_ptr || (n_verts > 0 && !work) || (n_cells > 0 && !node_idx))
         return fail(FEM_ERR_ARG, "node_ptr, node_idx or work is NULL");
-    const int NB = dim + 1;
     cudaStream_t s = stream;
-    if (cudaMemsetAsync(node_ptr, 0, sizeof(int32_t) * (n_verts + 1), s) != cudaSuccess)
-        return check_launch("node2cell memset");
-    if (n_cells == 0 || n_verts == 0) return check_launch("node2cell");
+    if (n_cells == 0 || n_verts == 0) {
+        if (cudaMemsetAsync(node_ptr, 0, sizeof(int32_t) * (n_verts + 1), s) != cudaSuccess)
+            return check_launch("node2cell memset");
+        return check_launch("node2cell");
+    }
     const uint32_t V = static_cast<uint32_t>(n_verts);
     unsigned *err = device_error_word();
     if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
-    count_kernel<<<grid_for(NB * n_cells, kBlock, reinterpret_cast<const void *>(count_kernel)), kBlock, 0, s>>>(
-        conn, NB * n_cells, V, node_ptr + 1, err);
-    if ((st = inclusive_scan(node_ptr + 1, n_verts, work + n_verts, s)) != FEM_OK) return st;
-    copy_kernel<<<grid_for(n_verts, kBlock, reinterpret_cast<const void *>(copy_kernel)), kBlock, 0, s>>>(
-        node_ptr, work, n_verts);
-    dim3 fgrid(grid_for(n_cells, kBlock, reinterpret_cast<const void *>(fill_kernel<4>)), NB);
-    if (dim == 2) fill_kernel<3><<<fgrid, kBlock, 0, s>>>(conn, n_cells, V, work, node_idx);
-    else fill_kernel<4><<<fgrid, kBlock, 0, s>>>(conn, n_cells, V, work, node_idx);
-    sort_segments_kernel<<<grid_for(n_verts, kBlock, reinterpret_cast<const void *>(sort_segments_kernel)), kBlock,
-                           0, s>>>(node_ptr, node_idx, n_verts);
+    int32_t *cursor = work;
+    const int32_t *ptr = node_ptr;
+    {
+        auto k = zero_kernel;
+        launch_overlapped(k, grid_for(n_verts + 1, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, node_ptr, n_verts + 1);
+    }
+    auto lists = [&](auto nb) {
+        constexpr int NBC = decltype(nb)::value;
+        {
+            auto k = count_kernel<NBC>;
+            launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, conn, n_cells, V, node_ptr + 1, err);
+        }
+        const fem_status e = scan_with_cursor(node_ptr + 1, n_verts, work + n_verts, cursor, s);
+        if (e != FEM_OK) return e;
+        {
+            auto k = fill_kernel<NBC>;
+            launch_overlapped(k, grid_for(n_cells, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, conn, n_cells, V, cursor, node_idx);
+        }
+        auto k = sort_segments_kernel<8>;
+        launch_overlapped(k, grid_for(n_verts * 8, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, ptr, node_idx, n_verts);
+        return FEM_OK;
+    };
+    st = dim == 2 ? lists(std::integral_constant<int, 3>()) : lists(std::integral_constant<int, 4>());
+    if (st != FEM_OK) return st;
     return check_launch("fem_build_node2cell");
 }
 
