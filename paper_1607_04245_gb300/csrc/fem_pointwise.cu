@@ -324,10 +324,17 @@ static Nvrtc &nvrtc() {
 
 // ------------------------------------------------------------------ module cache
 
+// Launch of the generated kernel, one cell per thread. Mixed form: CTAs of 256 threads on one wave,
+// or, where the registers that the caller's physics takes leave room for more warps in CTAs of 128,
+// those on up to four waves (nonlinear kappa(u, x) in 3D, 68 registers, 28 warps per SM instead of 24:
+// 1,572,864 cells 30.4 -> 27.7 us back to back, 200,000 5.6 -> 5.1; with the same number of warps CTAs
+// of 128 are up to 6 % slower). float64: CTAs of one warp, as many as the cells need (559 -> 543 us,
+// 200,000 cells 82 -> 75, 8,192 cells 14.8 -> 7.4: the float64 pipe's work evenly over the SMs).
 struct PwModule {
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kernel = nullptr;
-    int grid_per_sm = 1;
+    int block = 256;
+    int grid_per_sm = 1;  // CTAs per SM to launch at most; 0: as many as there are cells
 };
 
 static std::mutex g_pw_mu;
@@ -404,15 +411,19 @@ static fem_status get_module(int dev, int dim, int n_comp, int n_coef, int n_q, 
     PwModule m;
     cudaError_t e = cudaLibraryLoadData(&m.lib, bin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&m.kernel, m.lib, "fem_pointwise_kernel");
+    int ctas256 = 1, ctas128 = 2;
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m.grid_per_sm, reinterpret_cast<const void *>(m.kernel),
-                                                          256, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas256, reinterpret_cast<const void *>(m.kernel), 256, 0);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas128, reinterpret_cast<const void *>(m.kernel), 128, 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         if (m.lib) cudaLibraryUnload(m.lib);
         return fail(FEM_ERR_CUDA, "fem_integrate_pointwise: loading the compiled kernel: %s", cudaGetErrorString(e));
     }
-    if (m.grid_per_sm < 1) m.grid_per_sm = 1;
+    if (!mixed) m.block = 32, m.grid_per_sm = 0;
+    else if (ctas128 > 2 * ctas256) m.block = 128, m.grid_per_sm = 4 * ctas128;
+    else m.grid_per_sm = ctas256 < 1 ? 1 : ctas256;
     g_pw_cache.emplace(key, m);
     out = m;
     return FEM_OK;
@@ -472,8 +483,8 @@ extern "C" fem_status fem_integrate_pointwise(const char *f0_src, const char *f1
         a.wf[q] = static_cast<float>(a.w[q]);
         for (int b = 0; b < 4; ++b) a.phif[q][b] = static_cast<float>(a.phi[q][b]);
     }
-    const int64_t need = (n_cells + 255) / 256, cap = int64_t(m.grid_per_sm) * sm_count();
-    const unsigned grid = static_cast<unsigned>(need < cap ? need : cap);
+    const int64_t need = (n_cells + m.block - 1) / m.block, cap = int64_t(m.grid_per_sm) * sm_count();
+    const unsigned grid = static_cast<unsigned>(cap == 0 || need < cap ? need : cap);
     void *params[] = {&a};
     // overlapped with the previous kernel's tail, as the built-in kernels are (the kernel
     // waits for it first), except while the stream is being captured
@@ -485,7 +496,7 @@ extern "C" fem_status fem_integrate_pointwise(const char *f0_src, const char *f1
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(m.block);
     cfg.stream = stream;
     cfg.attrs = at;
     cfg.numAttrs = (refused || cs != cudaStreamCaptureStatusNone) ? 0 : 1;
