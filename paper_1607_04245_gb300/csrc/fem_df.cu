@@ -197,7 +197,6 @@ struct DfArgs {
 template <int DIM>
 __global__ void __launch_bounds__(kDfBlock, 10) lap_df_kernel(const __grid_constant__ DfArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     const int64_t C = a.C;
     const double *X[DIM];
@@ -302,7 +301,6 @@ constexpr int el_df_min_blocks() { return DIM == 3 ? 8 : 0; }  // 0: no minimum
 template <int DIM>
 __global__ void __launch_bounds__(kDfBlock, el_df_min_blocks<DIM>()) el_df_kernel(const __grid_constant__ DfElArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     const int64_t C = a.C;
     const int64_t V = a.V;
@@ -420,7 +418,6 @@ struct DfAdjArgs {
 template <int DIM>
 __global__ void __launch_bounds__(kDfBlock) adj_df_kernel(const __grid_constant__ DfAdjArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     const int64_t C = a.C;
     const double *X[DIM];

@@ -127,7 +127,6 @@ constexpr int el_min_blocks() {
 template <int DIM, int P, int CPT, int NQ, bool STR = false>
 __global__ void __launch_bounds__(kBlock, el_min_blocks<DIM, P, CPT>()) el_kernel(const __grid_constant__ ElArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     using T = val_t<P>;
     const int64_t C = a.C;

@@ -29,7 +29,6 @@ struct GeomArgs {
 template <int DIM, int P>
 __global__ void __launch_bounds__(kBlock) geometry_kernel(const __grid_constant__ GeomArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     using T = val_t<P>;
     const int64_t C = a.C;
@@ -83,7 +82,6 @@ __device__ __forceinline__ val_t<P> gweight(const QuadW &w, int q) {
 template <int DIM, int P, int CPT, int NQ>
 __global__ void __launch_bounds__(kBlock) lap_geom_kernel(const __grid_constant__ LapGeomArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     using T = val_t<P>;
     const int64_t C = a.C;

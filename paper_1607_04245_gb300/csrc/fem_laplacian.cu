@@ -168,7 +168,6 @@ __device__ __forceinline__ void lap_cell(const double (&xs)[DIM + 1][DIM],
 template <int DIM, int P, int CPT, int NQ, bool ADJ, bool STR = false>
 __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ LapArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     using T = val_t<P>;
     const int64_t C = a.C;
@@ -306,7 +305,6 @@ __device__ __noinline__ void lap_fields_fallback(const FieldsArgs &fa, int64_t c
 template <int DIM, int P, int CPT, int NQ, bool STR = false>
 __global__ void __launch_bounds__(kBlock) lap_fields_kernel(const __grid_constant__ FieldsArgs fa) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     using T = val_t<P>;
     const LapArgs &a = fa.a;
@@ -531,7 +529,6 @@ template <int DIM, int P, int NQ, bool ADJ, bool STR>
 __global__ void __launch_bounds__(kBlock, pair_min_blocks<P, ADJ>()) lap_pair_kernel(const __grid_constant__ LapArgs a) {
     static_assert(P != FEM_FP64, "float32 forms only");
     pdl_wait();  // launched overlapped: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     const int64_t C = a.C;  // even, unless STR
     const float *__restrict__ u = static_cast<const float *>(a.u);
@@ -661,7 +658,6 @@ __device__ __forceinline__ void ld_record(const float *rec, uint32_t v, float (&
 template <int DIM, int NQ>
 __global__ void __launch_bounds__(kBlock, 3) lap_rec_kernel(const __grid_constant__ LapArgs a, const float *rec) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     constexpr int NB = DIM + 1;
     const int64_t C = a.C;  // even
     const float *__restrict__ u = static_cast<const float *>(a.u);

@@ -47,7 +47,6 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t x, int32_t *tota
 // in-place inclusive scan of one tile; the tile's total goes to tile_sums[tile]
 __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(int32_t *data, int64_t n, int32_t *tile_sums) {
     pdl_wait();
-    pdl_trigger();
     __shared__ int32_t s_total;
     const int64_t base = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanItems;
     int32_t v[kScanItems];
@@ -67,7 +66,6 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(int32_t *data,
 // exclusive scan of the tile sums in place (one CTA, chunks of a tile with a carry)
 __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(int32_t *sums, int64_t n) {
     pdl_wait();
-    pdl_trigger();
     __shared__ int32_t s_total;
     int32_t carry = 0;
     for (int64_t c = 0; c < n; c += kScanTile) {
@@ -92,7 +90,6 @@ __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(int32_t *sums, 
 __global__ void __launch_bounds__(kScanThreads) add_offsets_kernel(int32_t *data, int64_t n, const int32_t *tile_sums,
                                                                    bool summed, int32_t *cursor) {
     pdl_wait();
-    pdl_trigger();
     __shared__ int32_t s_total;
     const int64_t tile = blockIdx.x;
     int32_t off;
@@ -142,7 +139,6 @@ static fem_status scan_with_cursor(int32_t *data, int64_t n, int32_t *tile_sums,
 
 __global__ void __launch_bounds__(kBlock) zero_kernel(int32_t *data, int64_t n) {
     pdl_wait();
-    pdl_trigger();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) data[i] = 0;
 }
@@ -169,7 +165,6 @@ template <int NB>
 __global__ void __launch_bounds__(kBlock) count_kernel(const int32_t *conn, int64_t C, uint32_t V, int32_t *ptr1,
                                                        unsigned *err) {
     pdl_wait();
-    pdl_trigger();
     uint32_t vmax = 0;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t warps_end = (C + 31) / 32 * 32;  // whole warps: warp_add is a warp's work
@@ -188,7 +183,6 @@ template <int NB>
 __global__ void __launch_bounds__(kBlock) fill_kernel(const int32_t *conn, int64_t C, uint32_t V, int32_t *cursor,
                                                       int32_t *idx) {
     pdl_wait();
-    pdl_trigger();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     const int64_t warps_end = (C + 31) / 32 * 32;
     for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < warps_end; e += stride) {
@@ -214,7 +208,6 @@ constexpr int kSortShared = 128;
 template <int G>
 __global__ void __launch_bounds__(kBlock) sort_segments_kernel(const int32_t *ptr, int32_t *idx, int64_t V) {
     pdl_wait();
-    pdl_trigger();
     __shared__ __align__(16) int32_t list[kBlock / G][kSortShared + 4];  // + 4: the groups' rows in different banks
     const int lane = threadIdx.x % G, group = threadIdx.x / G;
     const unsigned mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << ((threadIdx.x & 31) / G * G);
@@ -258,7 +251,6 @@ template <int NB, int NCOMP, class T>
 __global__ void gather_kernel(int64_t C, int64_t V, const T *__restrict__ elem, const int32_t *__restrict__ ptr,
                               const int32_t *__restrict__ idx, T *__restrict__ out) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; n < V; n += stride) {
         // (A warp reading 32 vertices' lists together with coalesced loads and summing from shared

@@ -112,7 +112,6 @@ extern "C" __global__ void __launch_bounds__(256) fem_pointwise_kernel(const PwA
     // launched overlapped with the kernel before it on the stream (outside graph capture):
     // its writes are visible from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const i64 C = a.C;
     const T *u = (const T *)a.u;
     const T *coef = (const T *)a.coef;

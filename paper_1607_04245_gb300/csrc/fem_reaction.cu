@@ -250,7 +250,6 @@ constexpr int rd_min_blocks() {
 template <int DIM, int P, bool A_P1, bool REACT, bool DRIFT, int CPT, int NQ, bool STR = false>
 __global__ void __launch_bounds__(kBlock, rd_min_blocks<DIM, P, CPT>()) rd_kernel(const __grid_constant__ RdArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
-    pdl_trigger();
     static_assert(A_P1 || !DRIFT, "grad a vanishes inside a cell for a P0 field");
     static_assert(CPT == 1 || NQ > 0, "vector rows need a compile-time quadrature size");
     constexpr int NB = DIM + 1;
