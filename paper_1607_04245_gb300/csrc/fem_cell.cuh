@@ -228,6 +228,111 @@ __device__ __forceinline__ void columns_f64(const double (&x)[DIM + 1][DIM], dou
         for (int k = 0; k < DIM; ++k) e[j][k] = x[j + 1][k] - x[0][k];
 }
 
+// The differences x[j + 1] - x[0], bitwise those of the float64 subtraction, with integer
+// operations: the float64 pipe issues 2 lanes a clock and SM, the integer pipes about 100, and the
+// float64 kernels wait for the former. The values are brought to fixed point at their largest
+// exponent (53 significant bits, 9 to spare), subtracted exactly as 64-bit integers, normalised and
+// (ROUND) rounded to nearest even. Returns false, with d unusable, where that does not give the
+// correctly rounded difference: a nonzero value more than 9 binades below the largest; -0,
+// subnormal or non-finite values; a difference below the normal range; without ROUND, one of more
+// than 53 significant bits (vertex coordinates of one cell hardly ever have one).
+template <int N, bool ROUND>
+__device__ __forceinline__ bool exact_differences(const double (&x)[N], double (&d)[N - 1]) {
+    uint32_t hw[N], lw[N], ex[N], top = 0;
+#pragma unroll
+    for (int b = 0; b < N; ++b) {
+        hw[b] = static_cast<uint32_t>(__double2hiint(x[b]));
+        lw[b] = static_cast<uint32_t>(__double2loint(x[b]));
+        ex[b] = (hw[b] >> 20) & 0x7ffu;
+        top = max(top, ex[b]);
+    }
+    bool ok = top < 0x7feu;
+    uint32_t fh[N], fl[N];
+#pragma unroll
+    for (int b = 0; b < N; ++b) {
+        const bool zero = (hw[b] | lw[b]) == 0u;  // +0 (-0 is left to the subtraction: its sign counts)
+        const int up = static_cast<int>(ex[b] - top) + 9;
+        ok = ok && (zero || (up >= 0 && ex[b] != 0u));
+        const uint32_t mh = (hw[b] & 0xfffffu) | 0x100000u;
+        uint32_t h = __funnelshift_l(lw[b], mh, up), l = lw[b] << (up & 31);
+        h = zero ? 0u : h;
+        const uint32_t s = static_cast<uint32_t>(static_cast<int32_t>(hw[b]) >> 31);
+        // two's complement of the magnitude where the sign is set
+        const uint64_t f = ((static_cast<uint64_t>(h ^ s) << 32) | (l ^ s)) - (static_cast<uint64_t>(s) << 32 | s);
+        fh[b] = static_cast<uint32_t>(f >> 32), fl[b] = static_cast<uint32_t>(f);
+    }
+    const uint64_t f0 = (static_cast<uint64_t>(fh[0]) << 32) | fl[0];
+    uint32_t dropped = 0;
+#pragma unroll
+    for (int j = 1; j < N; ++j) {
+        const uint64_t df = ((static_cast<uint64_t>(fh[j]) << 32) | fl[j]) - f0;
+        const uint64_t s = static_cast<uint64_t>(static_cast<int64_t>(df) >> 63);
+        const uint64_t mag = (df ^ s) - s;
+        const uint32_t mh = static_cast<uint32_t>(mag >> 32), ml = static_cast<uint32_t>(mag);
+        const bool small = mh == 0u;
+        const uint32_t h = small ? ml : mh, l = small ? 0u : ml;
+        const int n = __clz(static_cast<int>(h));
+        const uint32_t bh = __funnelshift_l(l, h, n), bl = l << (n & 31);  // leading one at bit 63
+        // the leading one of a value at exponent `top` is bit 61
+        const int e = static_cast<int>(top) + 2 - n - (small ? 32 : 0);
+        const bool none = h == 0u;
+        ok = ok && (none || e >= 1);
+        uint32_t hi = (static_cast<uint32_t>(s) & 0x80000000u) + (static_cast<uint32_t>(e - 1) << 20) + (bh >> 11);
+        uint32_t lo = __funnelshift_r(bl, bh, 11);
+        if constexpr (ROUND) {  // half a unit is 0x400; a carry out of the mantissa is the next exponent
+            const uint32_t up1 = ((bl & 0x7ffu) + (lo & 1u)) > 0x400u ? 1u : 0u;
+            lo += up1;
+            hi += lo < up1 ? 1u : 0u;
+        } else {
+            dropped |= bl;
+        }
+        d[j - 1] = __hiloint2double(static_cast<int>(none ? 0u : hi), static_cast<int>(none ? 0u : lo));
+    }
+    return ok && (ROUND || (dropped & 0x7ffu) == 0u);
+}
+
+// out of line: written in place the compiler would execute it predicated in every cell, and a
+// float64 instruction takes its time on the pipe even where every lane is switched off
+static __device__ __noinline__ double subtract_out_of_line(double a, double b) { return a - b; }
+
+// x[j + 1] - x[0] for the kernels that the float64 pipe bounds: by exact_differences where they
+// give them (`by_integer`: the launch is large enough for the pipe to be what it waits for)
+template <int N, bool ROUND>
+__device__ __forceinline__ void differences_f64(const double (&x)[N], double (&d)[N - 1], bool by_integer) {
+    if (by_integer) {
+        if (!exact_differences<N, ROUND>(x, d)) {
+#pragma unroll
+            for (int j = 1; j < N; ++j) d[j - 1] = subtract_out_of_line(x[j], x[0]);
+        }
+    } else {
+#pragma unroll
+        for (int j = 1; j < N; ++j) d[j - 1] = x[j] - x[0];
+    }
+}
+
+// Cells from which it does: below, a scheduler has one or two warps of 32 cells, whose time is their
+// own latency, which the integer operations lengthen. Us, subtractions / integer columns, 1,572,864
+// tets: residual 192 / 167, adjoint 272 / 246, elasticity 366 / 340, reaction-diffusion 375 / 351,
+// three fields 429 / 403; 50,000: 8.0 / 7.6, 14.1 / 13.9, 14.5 / 13.8, 15.2 / 15.2, 16.8 / 16.2;
+// 25,000: 5.0 / 5.3, 10.2 / 10.4, 8.4 / 8.6, 9.3 / 9.7, 9.8 / 10.1. The kernels that use it take one
+// cell per thread; double-float kernels, which the instruction issue bounds, lose a third by it.
+constexpr int64_t kExactFrom = 60000;
+
+// columns_f64 by differences_f64, axis by axis: the same columns, bit for bit
+template <int DIM>
+__device__ __forceinline__ void columns_f64_int(const double (&x)[DIM + 1][DIM], double (&e)[DIM][DIM],
+                                                bool by_integer) {
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        double a[DIM + 1], d[DIM];
+#pragma unroll
+        for (int b = 0; b <= DIM; ++b) a[b] = x[b][k];
+        differences_f64<DIM + 1, false>(a, d, by_integer);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) e[j][k] = d[j];
+    }
+}
+
 // Float32 Jacobian columns from float64 coordinates split into (hi, lo) pairs:
 // e_jk = (hi_jk - hi_0k) + (lo_jk - lo_0k); exact up to float32 rounding of the result.
 template <int DIM>

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kBlock, el_min_blocks<DIM, P, CPT>()) el_kerne
             ok[i] = true;
             if constexpr (P == FEM_FP64) {
                 double e[DIM][DIM], n[DIM][DIM];
-                columns_f64<DIM>(xs, e);
+                columns_f64_int<DIM>(xs, e, C >= kExactFrom);
                 double det = adjugate_rows<DIM>(e, n);
                 bad_det |= det_bad(det) | ids_repeat<NB>(v);
                 el_element<DIM>(n, det, uu, ls[i].value(), ms[i].value(), rr);

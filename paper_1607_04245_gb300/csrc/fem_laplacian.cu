@@ -109,11 +109,11 @@ template <int DIM, int P, bool ADJ>
 __device__ __forceinline__ void lap_cell(const double (&xs)[DIM + 1][DIM],
                                          const val_t<P> (&uu)[DIM + 1], const val_t<P> (&ll)[DIM + 1],
                                          const qsum_t<P> &ks, float tau2, val_t<P> (&rr)[DIM + 1], val_t<P> &tf,
-                                         bool rep, bool &bad_det) {
+                                         bool rep, bool &bad_det, bool by_int) {
     constexpr int NB = DIM + 1;
     if constexpr (P == FEM_FP64) {
         double e[DIM][DIM], n[DIM][DIM];
-        columns_f64<DIM>(xs, e);
+        columns_f64_int<DIM>(xs, e, by_int);
         double det = adjugate_rows<DIM>(e, n);
         bad_det |= det_bad(det) | rep;
         if constexpr (ADJ) {
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
             gather_coords<DIM>(X, v, xs);
             T rr[NB];
             T tf = T(0);
-            lap_cell<DIM, P, ADJ>(xs, uu, ll, ks[i], a.tau2, rr, tf, ids_repeat<NB>(v), bad_det);
+            lap_cell<DIM, P, ADJ>(xs, uu, ll, ks[i], a.tau2, rr, tf, ids_repeat<NB>(v), bad_det, C >= kExactFrom);
 #pragma unroll
             for (int b = 0; b < NB; ++b) r[b][i] = rr[b];
             tfac[i] = tf;
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kBlock) lap_fields_kernel(const __grid_constan
             double xs[NB][DIM];
             gather_coords<DIM>(X, v[i], xs);
             T e[DIM][DIM];
-            if constexpr (P == FEM_FP64) columns_f64<DIM>(xs, e);
+            if constexpr (P == FEM_FP64) columns_f64_int<DIM>(xs, e, C >= kExactFrom);
             else if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, e);
             else columns_f32<DIM>(xs, e);
             const T det = adjugate_rows<DIM>(e, n[i]);

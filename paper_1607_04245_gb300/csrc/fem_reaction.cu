@@ -213,7 +213,7 @@ __device__ __forceinline__ bool rd_cell(const RdArgs &a, const double *const (&X
     gather_coords<DIM>(X, v, xs);
     if constexpr (P == FEM_FP64) {
         double ee[DIM][DIM], n[DIM][DIM];
-        columns_f64<DIM>(xs, ee);
+        columns_f64_int<DIM>(xs, ee, a.C >= kExactFrom);
         const double det = adjugate_rows<DIM>(ee, n);
         bad_det |= det_bad(det) | ids_repeat<NB>(v);
         rd_element<DIM, P, double, REACT, DRIFT, NQA>(a, n, det, uu, aa, ks.value(), ci, nq, rr);
