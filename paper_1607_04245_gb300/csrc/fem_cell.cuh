@@ -232,11 +232,11 @@ __device__ __forceinline__ void columns_f64(const double (&x)[DIM + 1][DIM], dou
 // operations: the float64 pipe issues 2 lanes a clock and SM, the integer pipes about 100, and the
 // float64 kernels wait for the former. The values are brought to fixed point at their largest
 // exponent (53 significant bits, 9 to spare), subtracted exactly as 64-bit integers, normalised and
-// (ROUND) rounded to nearest even. Returns false, with d unusable, where that does not give the
-// correctly rounded difference: a nonzero value more than 9 binades below the largest; -0,
-// subnormal or non-finite values; a difference below the normal range; without ROUND, one of more
-// than 53 significant bits (vertex coordinates of one cell hardly ever have one).
-template <int N, bool ROUND>
+// packed again. Returns false, with d unusable, where that does not give the correctly rounded
+// difference: a nonzero value more than 9 binades below the largest; -0, subnormal or non-finite
+// values; a difference below the normal range or of more than 53 significant bits (vertex
+// coordinates of one cell hardly ever have one).
+template <int N>
 __device__ __forceinline__ bool exact_differences(const double (&x)[N], double (&d)[N - 1]) {
     uint32_t hw[N], lw[N], ex[N], top = 0;
 #pragma unroll
@@ -277,40 +277,19 @@ __device__ __forceinline__ bool exact_differences(const double (&x)[N], double (
         const int e = static_cast<int>(top) + 2 - n - (small ? 32 : 0);
         const bool none = h == 0u;
         ok = ok && (none || e >= 1);
-        uint32_t hi = (static_cast<uint32_t>(s) & 0x80000000u) + (static_cast<uint32_t>(e - 1) << 20) + (bh >> 11);
-        uint32_t lo = __funnelshift_r(bl, bh, 11);
-        if constexpr (ROUND) {  // half a unit is 0x400; a carry out of the mantissa is the next exponent
-            const uint32_t up1 = ((bl & 0x7ffu) + (lo & 1u)) > 0x400u ? 1u : 0u;
-            lo += up1;
-            hi += lo < up1 ? 1u : 0u;
-        } else {
-            dropped |= bl;
-        }
+        const uint32_t hi = (static_cast<uint32_t>(s) & 0x80000000u) + (static_cast<uint32_t>(e - 1) << 20) + (bh >> 11);
+        const uint32_t lo = __funnelshift_r(bl, bh, 11);
+        dropped |= bl;
         d[j - 1] = __hiloint2double(static_cast<int>(none ? 0u : hi), static_cast<int>(none ? 0u : lo));
     }
-    return ok && (ROUND || (dropped & 0x7ffu) == 0u);
+    return ok && (dropped & 0x7ffu) == 0u;
 }
 
 // out of line: written in place the compiler would execute it predicated in every cell, and a
 // float64 instruction takes its time on the pipe even where every lane is switched off
 static __device__ __noinline__ double subtract_out_of_line(double a, double b) { return a - b; }
 
-// x[j + 1] - x[0] for the kernels that the float64 pipe bounds: by exact_differences where they
-// give them (`by_integer`: the launch is large enough for the pipe to be what it waits for)
-template <int N, bool ROUND>
-__device__ __forceinline__ void differences_f64(const double (&x)[N], double (&d)[N - 1], bool by_integer) {
-    if (by_integer) {
-        if (!exact_differences<N, ROUND>(x, d)) {
-#pragma unroll
-            for (int j = 1; j < N; ++j) d[j - 1] = subtract_out_of_line(x[j], x[0]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 1; j < N; ++j) d[j - 1] = x[j] - x[0];
-    }
-}
-
-// Cells from which it does: below, a scheduler has one or two warps of 32 cells, whose time is their
+// Cells from which the float64 kernels take their columns so: below, a scheduler has one or two warps of 32 cells, whose time is their
 // own latency, which the integer operations lengthen. Us, subtractions / integer columns, 1,572,864
 // tets: residual 192 / 167, adjoint 272 / 246, elasticity 366 / 340, reaction-diffusion 375 / 351,
 // three fields 429 / 403; 50,000: 8.0 / 7.6, 14.1 / 13.9, 14.5 / 13.8, 15.2 / 15.2, 16.8 / 16.2;
@@ -318,7 +297,7 @@ __device__ __forceinline__ void differences_f64(const double (&x)[N], double (&d
 // cell per thread; double-float kernels, which the instruction issue bounds, lose a third by it.
 constexpr int64_t kExactFrom = 60000;
 
-// columns_f64 by differences_f64, axis by axis: the same columns, bit for bit
+// columns_f64, bit for bit, axis by axis by exact_differences where they give them
 template <int DIM>
 __device__ __forceinline__ void columns_f64_int(const double (&x)[DIM + 1][DIM], double (&e)[DIM][DIM],
                                                 bool by_integer) {
@@ -327,7 +306,15 @@ __device__ __forceinline__ void columns_f64_int(const double (&x)[DIM + 1][DIM],
         double a[DIM + 1], d[DIM];
 #pragma unroll
         for (int b = 0; b <= DIM; ++b) a[b] = x[b][k];
-        differences_f64<DIM + 1, false>(a, d, by_integer);
+        if (by_integer) {
+            if (!exact_differences<DIM + 1>(a, d)) {
+#pragma unroll
+                for (int j = 0; j < DIM; ++j) d[j] = subtract_out_of_line(a[j + 1], a[0]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < DIM; ++j) d[j] = a[j + 1] - a[0];
+        }
 #pragma unroll
         for (int j = 0; j < DIM; ++j) e[j][k] = d[j];
     }
