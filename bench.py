@@ -95,7 +95,7 @@ def load_peaks():
 
 KERNEL_SOURCES = {
     # fem_core.cu sizes the launches (grid, occupancy), so it belongs to the kernel's definition
-    "lap": ("fem_internal.cuh", "fem_cell.cuh", "fem_f2.cuh", "fem_pipe.cuh", "fem_laplacian.cu", "fem_core.cu"),
+    "lap": ("fem_internal.cuh", "fem_cell.cuh", "fem_f2.cuh", "fem_laplacian.cu", "fem_core.cu"),
     "el": ("fem_internal.cuh", "fem_cell.cuh", "fem_f2.cuh", "fem_elasticity.cu"),
 }
 
