@@ -276,6 +276,125 @@ fem_status launch_lap_df(int dim, int64_t n_cells, int64_t n_verts, const double
     return check_launch("fem_integrate_laplacian (FEM_FP64_DF)");
 }
 
+// The same residual for a solve's repeated applications: the adjugate rows n_j and
+// s = Kbar / |det J| as pairs, [dim * dim + 1][C], formed once, and the rest per application, the
+// same operations on the same values as lap_df_kernel's (the same bits): about 400 instead of 1052
+// instructions a tet, no coordinates and no float64 columns.
+template <int DIM>
+__global__ void __launch_bounds__(kDfBlock) lap_df_factors_kernel(const __grid_constant__ DfArgs a) {
+    pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
+    constexpr int NB = DIM + 1;
+    const int64_t C = a.C;
+    float2 *fac = reinterpret_cast<float2 *>(a.out);
+    const double *X[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) X[k] = a.X[k];
+    uint32_t vmax = 0;     // largest vertex id seen (bad ids are clamped and reported)
+    bool bad_det = false;  // a cell with det J = 0 or non-finite
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < C; c += stride) {
+        uint32_t v[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) v[b] = clamp_vid(ld_stream(a.conn + b * C + c), a.V, vmax);
+        const dfl kbar = df_from_double(weighted64(a.wd, a.K, C, c, a.nq));
+        double xs[NB][DIM];
+        gather_coords<DIM>(X, v, xs);
+        dfl e[DIM][DIM];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) e[j][k] = df_from_double(xs[j + 1][k] - xs[0][k]);
+        dfl n[DIM][DIM];
+        const dfl det = df_adjugate<DIM>(e, n);
+        bad_det |= det_bad(det.hi) | ids_repeat<NB>(v);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) fac[(j * DIM + i) * C + c] = make_float2(n[j][i].hi, n[j][i].lo);
+        const dfl s = df_div(kbar, df_abs(det));
+        fac[DIM * DIM * C + c] = make_float2(s.hi, s.lo);
+    }
+    report_mesh(a.err, vmax, a.V, bad_det);
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kDfBlock) lap_df_factored_kernel(int64_t C, uint32_t V, const int32_t *conn,
+                                                                   const double *u, const float2 *fac, double *out) {
+    pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
+    constexpr int NB = DIM + 1;
+    uint32_t vmax = 0;  // (reported when the factors were formed)
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < C; c += stride) {
+        double uu[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) uu[b] = ld_gather(u + clamp_vid(ld_stream(conn + b * C + c), V, vmax));
+        auto pair = [&](int m) {
+            const float2 f = __ldcs(fac + m * C + c);
+            return dfl{f.x, f.y};
+        };
+        dfl n[DIM][DIM], du[DIM], h[DIM];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) n[j][i] = pair(j * DIM + i);
+        const dfl s = pair(DIM * DIM);
+        const dfl u0 = df_from_double(uu[0]);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) du[j] = df_sub(df_from_double(uu[j + 1]), u0);
+        df_combine<DIM>(du, n, h);
+        dfl sum;
+        double r[NB];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) {
+            const dfl rj = df_mul(s, df_dotv<DIM>(n[j], h));
+            r[j + 1] = df_to_double(rj);
+            sum = j == 0 ? rj : df_add(sum, rj);
+        }
+        r[0] = -df_to_double(sum);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) out[b * C + c] = r[b];
+    }
+}
+
+// called by the solver with arguments that fem_integrate_laplacian has validated
+fem_status launch_lap_df_factors(int dim, int64_t n_cells, int64_t n_verts, const double *coords, const int32_t *conn,
+                                 const double *K, const QuadW &w, double *fac, cudaStream_t s) {
+    DfArgs a{};
+    for (int k = 0; k < 3; ++k) a.X[k] = coords + (k < dim ? k : 0) * n_verts;
+    a.conn = conn;
+    a.K = K;
+    a.out = fac;
+    a.C = n_cells;
+    a.V = static_cast<uint32_t>(n_verts);
+    a.nq = w.nq;
+    if (!(a.err = device_error_word())) return fail(FEM_ERR_CUDA, "device error word unavailable");
+    for (int q = 0; q < FEM_MAX_QPTS; ++q) a.wd[q] = q < w.nq ? w.wd[q] : 0.0;
+    if (dim == 2) {
+        auto k = lap_df_factors_kernel<2>;
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, s, a);
+    } else {
+        auto k = lap_df_factors_kernel<3>;
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, s, a);
+    }
+    return check_launch("fem_pcg_laplacian (factors)");
+}
+
+fem_status launch_lap_df_factored(int dim, int64_t n_cells, int64_t n_verts, const int32_t *conn, const double *u,
+                                  const double *fac, double *out, cudaStream_t s) {
+    const uint32_t V = static_cast<uint32_t>(n_verts);
+    const float2 *f = reinterpret_cast<const float2 *>(fac);
+    if (dim == 2) {
+        auto k = lap_df_factored_kernel<2>;
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, s, n_cells, V,
+                          conn, u, f, out);
+    } else {
+        auto k = lap_df_factored_kernel<3>;
+        launch_overlapped(k, grid_for(n_cells, kDfBlock, reinterpret_cast<const void *>(k)), kDfBlock, 0, s, n_cells, V,
+                          conn, u, f, out);
+    }
+    return check_launch("fem_pcg_laplacian (factored residual)");
+}
+
 // ---- linear elasticity in the same form: f1 = lambda tr(eps) I + 2 mu eps. With the
 // adjugate rows n_j and H[k][i] = sum_j (u_{j,k} - u_{0,k}) n_j[i] (grad u = H / det J):
 //     T = Lbar tr(H) I + Mbar (H + H^T),  r_{b,k} = (T n_b)_k / |det J|,

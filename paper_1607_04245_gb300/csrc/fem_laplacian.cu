@@ -260,6 +260,105 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
     report_mesh(a.err, vmax, a.V, bad_det);
 }
 
+// ------------------------------------------------------------------ repeated applications
+//
+// A solve in element form applies the float64 residual hundreds of times to one mesh and
+// coefficient. What of it does not depend on u, the adjugate rows n_j and s = Kbar / |det J|, is
+// formed once per cell, [dim * dim + 1][C], and an application does the rest: 27 instead of 58
+// float64 operations a tet, the same ones in the same order as lap_kernel's, so the same bits.
+// 80 more bytes per tet: the float64 pipe stays what an application waits for (1,572,864 tets: an
+// iteration of the solve 255 us at first, 125).
+
+template <int DIM>
+__global__ void __launch_bounds__(kWarpCta) lap_factors_kernel(const __grid_constant__ LapArgs a) {
+    pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
+    constexpr int NB = DIM + 1;
+    const int64_t C = a.C;
+    const double *K = static_cast<const double *>(a.K);
+    double *fac = static_cast<double *>(a.out);
+    const double *X[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) X[k] = a.X[k];
+    uint32_t vmax = 0;     // largest vertex id seen (bad ids are clamped and reported)
+    bool bad_det = false;  // a cell with det J = 0 or non-finite
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < C; c += stride) {
+        uint32_t v[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) v[b] = clamp_vid(ld_stream(a.conn + b * C + c), a.V, vmax);
+        qsum_t<FEM_FP64> ks;
+        ks.first(a.w.wd[0], ld_stream(K + c));
+        for (int q = 1; q < a.w.nq; ++q) ks.add(a.w.wd[q], ld_stream(K + q * C + c));
+        double xs[NB][DIM], e[DIM][DIM], n[DIM][DIM];
+        gather_coords<DIM>(X, v, xs);
+        columns_f64<DIM>(xs, e);
+        const double det = adjugate_rows<DIM>(e, n);
+        bad_det |= det_bad(det) | ids_repeat<NB>(v);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) fac[(j * DIM + i) * C + c] = n[j][i];
+        fac[DIM * DIM * C + c] = quot_abs(ks.value(), det);
+    }
+    report_mesh(a.err, vmax, a.V, bad_det);
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kWarpCta) lap_factored_kernel(int64_t C, uint32_t V, const int32_t *conn,
+                                                                const double *u, const double *fac, double *out) {
+    pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
+    constexpr int NB = DIM + 1;
+    uint32_t vmax = 0;  // (reported when the factors were formed)
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < C; c += stride) {
+        double uu[NB], n[DIM][DIM], r[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) uu[b] = ld_gather(u + clamp_vid(ld_stream(conn + b * C + c), V, vmax));
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) n[j][i] = ld_stream(fac + (j * DIM + i) * C + c);
+        lap_apply<DIM>(n, ld_stream(fac + DIM * DIM * C + c), uu, r);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) out[b * C + c] = r[b];
+    }
+}
+
+// called by the solver with arguments that fem_integrate_laplacian has validated
+fem_status launch_lap_factors(int dim, int64_t n_cells, int64_t n_verts, const double *coords, const int32_t *conn,
+                              const double *K, const QuadW &w, double *fac, cudaStream_t s) {
+    LapArgs a{};
+    for (int k = 0; k < 3; ++k) a.X[k] = coords + (k < dim ? k : 0) * n_verts;
+    a.conn = conn;
+    a.K = K;
+    a.out = fac;
+    a.C = n_cells;
+    a.V = static_cast<uint32_t>(n_verts);
+    a.w = w;
+    if (!(a.err = device_error_word())) return fail(FEM_ERR_CUDA, "device error word unavailable");
+    if (dim == 2) {
+        auto k = lap_factors_kernel<2>;
+        launch_overlapped(k, warp_ctas(n_cells), kWarpCta, 0, s, a);
+    } else {
+        auto k = lap_factors_kernel<3>;
+        launch_overlapped(k, warp_ctas(n_cells), kWarpCta, 0, s, a);
+    }
+    return check_launch("fem_pcg_laplacian (factors)");
+}
+
+fem_status launch_lap_factored(int dim, int64_t n_cells, int64_t n_verts, const int32_t *conn, const double *u,
+                               const double *fac, double *out, cudaStream_t s) {
+    const uint32_t V = static_cast<uint32_t>(n_verts);
+    if (dim == 2) {
+        auto k = lap_factored_kernel<2>;
+        launch_overlapped(k, warp_ctas(n_cells), kWarpCta, 0, s, n_cells, V, conn, u, fac, out);
+    } else {
+        auto k = lap_factored_kernel<3>;
+        launch_overlapped(k, warp_ctas(n_cells), kWarpCta, 0, s, n_cells, V, conn, u, fac, out);
+    }
+    return check_launch("fem_pcg_laplacian (factored residual)");
+}
+
 // ------------------------------------------------------------------ several fields
 
 // Element residuals of n_fields nodal fields on one mesh and coefficient: the geometry

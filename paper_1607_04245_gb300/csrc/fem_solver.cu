@@ -7,11 +7,13 @@
 // The iteration is CG in Chronopoulos and Gear's form. A solve takes one of two forms:
 //   * assembled: the operator's rows are formed once on the device (fem_sell.cuh) and the
 //     whole loop runs in one cooperative kernel (sell_cg_kernel). Taken by the float32 forms
-//     and by FEM_FP64 in 3D whenever the caller's workspace has room for the matrix.
+//     and by FEM_FP64 on small 3D meshes (assembled_form) whenever the caller's workspace has
+//     room for the matrix.
 //   * element form: each application is the residual kernel and the vertex sum; one iteration
-//     is captured into the body of a CUDA graph WHILE node. For FEM_FP64_DF and FEM_FP64 in 2D
-//     (assembled_form), workspaces without room for the matrix, meshes whose rows do not fit
-//     it, and device partitions that refuse the cooperative launch.
+//     is captured into the body of a CUDA graph WHILE node. For the other float64 solves,
+//     workspaces without room for the matrix, meshes whose rows do not fit it, and device
+//     partitions that refuse the cooperative launch. The Laplacian's residual is then applied
+//     from factors formed once per solve (launch_lap_factors), where the workspace has room.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -22,6 +24,15 @@
 
 namespace fem {
 
+// fem_laplacian.cu, fem_df.cu: the residual split into what is formed once and the rest
+fem_status launch_lap_factors(int dim, int64_t n_cells, int64_t n_verts, const double *coords, const int32_t *conn,
+                              const double *K, const QuadW &w, double *fac, cudaStream_t s);
+fem_status launch_lap_factored(int dim, int64_t n_cells, int64_t n_verts, const int32_t *conn, const double *u,
+                               const double *fac, double *out, cudaStream_t s);
+fem_status launch_lap_df_factors(int dim, int64_t n_cells, int64_t n_verts, const double *coords, const int32_t *conn,
+                                 const double *K, const QuadW &w, double *fac, cudaStream_t s);
+fem_status launch_lap_df_factored(int dim, int64_t n_cells, int64_t n_verts, const int32_t *conn, const double *u,
+                                  const double *fac, double *out, cudaStream_t s);
 fem_status launch_gather(int dim, int n_comp, int64_t C, int64_t V, const void *elem, const int32_t *node_ptr,
                          const int32_t *node_idx, void *out, fem_precision prec, cudaStream_t s);
 
@@ -891,23 +902,37 @@ struct Workspace {
     double *partial, *scalars;
     SellMatrix mat;  // the assembled operator (mat.cols: nullptr where the workspace has no room for it)
     double *mat_partial;
+    double *fac = nullptr;  // element form: the float64 Laplacian's factors, nullptr where not provided for
 };
 
 // Which solves take the assembled form. The two forms' roundings differ, and CG amplifies that
-// over its iterations: solved to 1e-8, their x differ by up to 3e-11 in float64 on 3D meshes up
-// to 1.6 M cells (the same iteration counts), but by up to 9e-9 in 2D (three times the
-// iterations, ending one to three apart) and against the double-float operator, whose entries
-// are 5e-14 off. Neither is further from the solution (2e-8 at that tolerance), but float64
-// results are held to 1e-9 of the element form's.
-static bool assembled_form(int dim, fem_precision prec) {
-    return prec == FEM_FP32_MIXED || prec == FEM_FP32 || (prec == FEM_FP64 && dim == 3);
+// over its iterations, in some float64 solves until the residual norms differ in their second
+// digit and the stopping test ends one iteration apart (7 of 40 on 1,572,864 tets with 256
+// iterations, 2 of 120 on 200,000 to 1,000,000; elasticity 3 of 32 on 100,000 and 200,000; also in 2D,
+// and against the double-float operator, whose entries are 5e-14 off): x then differs by 3e-9, no
+// further from the solution, but float64 results are held to 1e-9 of the element form's. So float64
+// takes it on 3D meshes of up to kAssembled64 cells times components (the residual norms of 20
+// solves of 60,000 tets agreed to 3e-6, of 16 of elasticity on 20,000 to 3e-10).
+constexpr int64_t kAssembled64 = 45000;
+
+static bool assembled_form(int physics, int dim, int64_t C, fem_precision prec) {
+    return prec == FEM_FP32_MIXED || prec == FEM_FP32 ||
+           (prec == FEM_FP64 && dim == 3 && C * (physics == 0 ? 1 : dim) <= kAssembled64);
 }
 
 // The assembled operator is provided for up to kMatrixMaxBytes of workspace; beyond that (3D:
 // some 600 M cells for the Laplacian, 70 M for elasticity in float64) the solve runs in element form.
 constexpr size_t kMatrixMaxBytes = size_t(32) << 30;
 
-static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Workspace *w, int ncomp, bool matrix) {
+// what a solve's workspace holds beside its vectors: the assembled operator, or (element form of
+// the Laplacian in the float64 value types) the residual's factors
+enum class Room { Vectors, Matrix, Factors };
+static Room room_for(int physics, int dim, int64_t C, fem_precision prec) {
+    if (assembled_form(physics, dim, C, prec)) return Room::Matrix;
+    return physics == 0 && (prec == FEM_FP64 || prec == FEM_FP64_DF) ? Room::Factors : Room::Vectors;
+}
+
+static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Workspace *w, int ncomp, Room room) {
     size_t off = 0;
     char *b = static_cast<char *>(base);
     auto take = [&](size_t bytes) {
@@ -925,7 +950,7 @@ static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Worksp
     double *mat_partial = nullptr;
     const int64_t slots = sell_slots(C, V);
     const size_t bb = size_t(ncomp) * size_t(ncomp);
-    if (matrix && C > 0 && slots < (int64_t(1) << 31) && size_t(slots) * 32 * (4 + bb * vs) <= kMatrixMaxBytes) {
+    if (room == Room::Matrix && C > 0 && slots < (int64_t(1) << 31) && size_t(slots) * 32 * (4 + bb * vs) <= kMatrixMaxBytes) {
         mat.cap = slots;
         mat.cols = static_cast<int32_t *>(take(size_t(slots) * 32 * sizeof(int32_t)));
         mat.vals = take(size_t(slots) * 32 * bb * vs);
@@ -936,7 +961,10 @@ static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Worksp
         mat.cell = nv <= (dim + 1) * ncomp ? elem : take(size_t(nv) * size_t(C) * vs);
         mat_partial = static_cast<double *>(take(3 * sizeof(double) * kCgMaxBlocks));
     }
-    if (w) *w = Workspace{elem, D, r, z, p, q, sv, partial, scalars, mat, mat_partial};
+    double *fac = nullptr;
+    const size_t fac_bytes = size_t(dim * dim + 1) * size_t(C) * sizeof(double);
+    if (room == Room::Factors && C > 0 && fac_bytes <= kMatrixMaxBytes) fac = static_cast<double *>(take(fac_bytes));
+    if (w) *w = Workspace{elem, D, r, z, p, q, sv, partial, scalars, mat, mat_partial, fac};
     return off;
 }
 
@@ -975,8 +1003,8 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
     bool use_matrix = w.mat.cols != nullptr && kept != Kept::Diagonal;
     auto by_comps = [&](auto go) {
         if (nc == 1) go(std::integral_constant<int, 1>());
-        else if (nc == 2) go(std::integral_constant<int, 2>());
-        else go(std::integral_constant<int, 3>());
+        else if (nc == 3) go(std::integral_constant<int, 3>());
+        else if constexpr (std::is_same<T, float>::value) go(std::integral_constant<int, 2>());
     };
     auto assemble = [&]() -> fem_status {
         unsigned *err = device_error_word();
@@ -1044,6 +1072,12 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
     };
     // the element vectors of v in w.elem
     auto residual = [&](const T *v, cudaStream_t cs) -> fem_status {
+        double *el = static_cast<double *>(w.elem);
+        if (w.fac) {
+            if constexpr (std::is_same<T, double>::value)
+                return prec == FEM_FP64 ? launch_lap_factored(dim, C, V, conn, v, w.fac, el, cs)
+                                        : launch_lap_df_factored(dim, C, V, conn, v, w.fac, el, cs);
+        }
         if (op.physics == 0)
             return fem_integrate_laplacian(dim, C, V, coords, conn, v, op.K, n_q, qpts, qw, w.elem, prec, cs);
         return fem_integrate_elasticity(dim, C, V, coords, conn, v, op.lam, op.mu, n_q, qpts, qw, w.elem, prec, cs);
@@ -1122,6 +1156,12 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
         if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
     }
     if (kept != Kept::Diagonal && (st = element_diagonal()) != FEM_OK) return st;
+    if (w.fac && kept != Kept::Diagonal) {
+        const double *K = static_cast<const double *>(op.K);
+        st = prec == FEM_FP64 ? launch_lap_factors(dim, C, V, coords, conn, K, qwt, w.fac, s)
+                              : launch_lap_df_factors(dim, C, V, coords, conn, K, qwt, w.fac, s);
+        if (st != FEM_OK) return st;
+    }
     kept = Kept::Diagonal;
     if ((st = matvec(X, q, s)) != FEM_OK) return st;
     cg_init_kernel<T><<<gV, 256, 0, s>>>(N, V, B, q, D, fixed, r, z, p, sv);
@@ -1191,7 +1231,7 @@ using namespace fem;
 extern "C" int64_t fem_pcg_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, assembled_form(dim, prec)));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, room_for(0, dim, n_cells, prec)));
 }
 
 extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -1213,14 +1253,14 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
     if (!K || !node_ptr || !node_idx || !fixed || !x || !work) return fail(FEM_ERR_ARG, "a NULL array argument");
     const bool f64 = prec == FEM_FP64 || prec == FEM_FP64_DF;
     const size_t vs = f64 ? 8 : 4;
-    const int64_t need = static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, false));
+    const int64_t need = static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, Room::Vectors));
     if (work_bytes < need)
         return fail(FEM_ERR_OOM, "fem_pcg_laplacian: workspace of %lld bytes, %lld needed",
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
-    const bool matrix = assembled_form(dim, prec) && work_bytes >= fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
-    carve(n_cells, n_verts, dim, vs, work, &w, 1, matrix);
+    const bool all = work_bytes >= fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
+    carve(n_cells, n_verts, dim, vs, work, &w, 1, all ? room_for(0, dim, n_cells, prec) : Room::Vectors);
     Kept kept = Kept::Nothing;
     if (f64)
         return pcg_run<double>(dim, n_cells, n_verts, coords, conn, Operator{0, K, nullptr, nullptr}, n_q, qpts, qw,
@@ -1234,7 +1274,7 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
 extern "C" int64_t fem_pcg_elasticity_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, assembled_form(dim, prec)));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, room_for(1, dim, n_cells, prec)));
 }
 
 extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -1258,15 +1298,14 @@ extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_ver
         return fail(FEM_ERR_ARG, "a NULL array argument");
     const bool f64 = prec == FEM_FP64 || prec == FEM_FP64_DF;
     const size_t vs = f64 ? 8 : 4;
-    const int64_t need = static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, false));
+    const int64_t need = static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, Room::Vectors));
     if (work_bytes < need)
         return fail(FEM_ERR_OOM, "fem_pcg_elasticity: workspace of %lld bytes, %lld needed",
                     static_cast<long long>(work_bytes), static_cast<long long>(need));
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
-    const bool matrix =
-        assembled_form(dim, prec) && work_bytes >= fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
-    carve(n_cells, n_verts, dim, vs, work, &w, dim, matrix);
+    const bool all = work_bytes >= fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
+    carve(n_cells, n_verts, dim, vs, work, &w, dim, all ? room_for(1, dim, n_cells, prec) : Room::Vectors);
     Kept kept = Kept::Nothing;
     const Operator op{1, nullptr, lam, mu};
     if (f64)
@@ -1325,7 +1364,7 @@ static size_t carve_refined(int64_t C, int64_t V, int dim, int n_q, int physics,
                             bool matrix) {
     const int nc = physics == 0 ? 1 : dim, ncoef = physics == 0 ? 1 : 2;
     Workspace inner;
-    size_t off = carve(C, V, dim, sizeof(float), base, &inner, nc, matrix);
+    size_t off = carve(C, V, dim, sizeof(float), base, &inner, nc, matrix ? Room::Matrix : Room::Vectors);
     char *b = static_cast<char *>(base);
     auto take = [&](size_t bytes) {
         void *p = b ? b + off : nullptr;
