@@ -172,7 +172,19 @@ __device__ __forceinline__ f2 quot_abs(f2 num, f2 den) {
     return f2_make(__fdividef(f2_x(num), fabsf(f2_x(den))), __fdividef(f2_y(num), fabsf(f2_y(den))));
 }
 
-__device__ __forceinline__ double neg(double x) { return -x; }
+// -x and (first term of a sum) 0 + x, which turns -0 into +0, with integer operations: either is an
+// addition on the float64 pipe otherwise, two of a tet's 58 in the residual
+// (1,572,864 tets, us: residual 166.5 -> 159.9, adjoint 246.3 -> 240.4, elasticity 340 -> 330, three
+// fields 403 -> 377)
+__device__ __forceinline__ double neg(double x) {
+    return __hiloint2double(__double2hiint(x) ^ static_cast<int>(0x80000000u), __double2loint(x));
+}
+__device__ __forceinline__ double from_zero(double x) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+    return __hiloint2double(static_cast<int>(hi == 0x80000000u && lo == 0u ? 0u : hi), static_cast<int>(lo));
+}
+__device__ __forceinline__ float from_zero(float x) { return 0.0f + x; }
+__device__ __forceinline__ f2 from_zero(f2 x) { return f2{0ull} + x; }
 __device__ __forceinline__ float neg(float x) { return -x; }
 __device__ __forceinline__ f2 neg(f2 x) { return f2{0ull} - x; }
 

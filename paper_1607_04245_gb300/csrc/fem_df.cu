@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kDfBlock, 10) lap_df_kernel(const __grid_const
             r[j + 1] = df_to_double(rj);
             sum = j == 0 ? rj : df_add(sum, rj);
         }
-        r[0] = -df_to_double(sum);
+        r[0] = neg(df_to_double(sum));
 #pragma unroll
         for (int b = 0; b < NB; ++b) __stcs(a.out + b * C + c, r[b]);
     }
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kDfBlock) lap_df_factored_kernel(int64_t C, ui
             r[j + 1] = df_to_double(rj);
             sum = j == 0 ? rj : df_add(sum, rj);
         }
-        r[0] = -df_to_double(sum);
+        r[0] = neg(df_to_double(sum));
 #pragma unroll
         for (int b = 0; b < NB; ++b) out[b * C + c] = r[b];
     }
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(kDfBlock) adj_df_kernel(const __grid_constant_
             sum = j == 0 ? rj : df_add(sum, rj);
             __stcs(a.scratch + (j + 1) * C + c, df_to_double(rj));
         }
-        __stcs(a.scratch + c, -df_to_double(sum));
+        __stcs(a.scratch + c, neg(df_to_double(sum)));
         // dK[q] = w_q (h_l . h_u) / |det J|
         const dfl tf = df_mul(df_dotv<DIM>(hl, hu), inv);
         for (int q = 0; q < a.nq; ++q) __stcs(a.dK + q * C + c, df_to_double(df_mul(dfl{a.whi[q], a.wlo[q]}, tf)));

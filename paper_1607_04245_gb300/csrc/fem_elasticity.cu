@@ -61,13 +61,11 @@ __device__ __forceinline__ void el_element(const T (&n)[DIM][DIM], T det, const 
         for (int i = k + 1; i < DIM; ++i) Tm[k][i] = Tm[i][k] = sm * (H[k][i] + H[i][k]);
     }
 #pragma unroll
-    for (int k = 0; k < DIM; ++k) r[0][k] = T(0);
-#pragma unroll
     for (int b = 1; b <= DIM; ++b)
 #pragma unroll
         for (int k = 0; k < DIM; ++k) {
             r[b][k] = dotv<DIM>(Tm[k], n[b - 1]);
-            r[0][k] -= r[b][k];
+            r[0][k] = b == 1 ? from_zero(neg(r[b][k])) : r[0][k] - r[b][k];
         }
 }
 

@@ -133,16 +133,16 @@ __global__ void __launch_bounds__(kBlock) lap_geom_kernel(const __grid_constant_
             bad_det |= det_bad(det);
             det = det < T(0) ? -det : det;
             const T s = ks[i].value() * det;
-            T sum = zero<T>();
+            T sum;
 #pragma unroll
             for (int j = 0; j < DIM; ++j) {
                 T d = gm[j * DIM][i] * gv[0];
 #pragma unroll
                 for (int k = 1; k < DIM; ++k) d = fma(gm[j * DIM + k][i], gv[k], d);
                 r[j + 1][i] = s * d;
-                sum = sum + r[j + 1][i];
+                sum = j == 0 ? from_zero(r[j + 1][i]) : sum + r[j + 1][i];
             }
-            r[0][i] = -sum;
+            r[0][i] = neg(sum);
         }
 #pragma unroll
         for (int b = 0; b < NB; ++b) cells.store(out + b * C, r[b]);

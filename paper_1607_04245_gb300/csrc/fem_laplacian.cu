@@ -49,11 +49,11 @@ __device__ __forceinline__ void lap_apply(const T (&n)[DIM][DIM], T s, const T (
 #pragma unroll
         for (int i = 0; i < DIM; ++i) h[i] = fma(du, n[j][i], h[i]);
     }
-    T sum = zero<T>();
+    T sum;
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
         r[j + 1] = s * dotv<DIM>(n[j], h);
-        sum = sum + r[j + 1];
+        sum = j == 0 ? from_zero(r[j + 1]) : sum + r[j + 1];
     }
     r[0] = neg(sum);
 }
@@ -84,11 +84,11 @@ __device__ __forceinline__ void lap_adj_element(const T (&n)[DIM][DIM], T det, c
     if constexpr (std::is_same<T, f2>::value) one = f2_splat(1.0f);
     else one = T(1);
     const T y = quot_abs(one, det), s = kbar * y;
-    T sum = zero<T>();
+    T sum;
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
         r[j + 1] = s * dotv<DIM>(n[j], hl);
-        sum = sum + r[j + 1];
+        sum = j == 0 ? from_zero(r[j + 1]) : sum + r[j + 1];
     }
     r[0] = neg(sum);
     tf = dotv<DIM>(hl, hu) * y;

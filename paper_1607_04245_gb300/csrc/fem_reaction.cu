@@ -95,13 +95,13 @@ __device__ __forceinline__ void rd_element(const RdArgs &a, const T (&n)[DIM][DI
     constexpr bool ONE_RCP = std::is_same<T, double>::value && NEWTON;
     const T y = ONE_RCP ? quot_abs(T(1), det) : T(0);
     const T s = ONE_RCP ? kbar * y : quot_div<NEWTON>(kbar, det);
-    T sum = zero<T>();
+    T sum;
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
         r[j + 1] = s * dotv<DIM>(n[j], h);
-        sum = sum + r[j + 1];
+        sum = j == 0 ? from_zero(r[j + 1]) : sum + r[j + 1];
     }
-    r[0] = -sum;
+    r[0] = neg(sum);
     if constexpr (DRIFT) {
         T ha[DIM];
 #pragma unroll

@@ -65,3 +65,33 @@ def test_columns_bit_for_bit(dim, kind):
             same = xs.contiguous().view(torch.int64) == y.contiguous().view(torch.int64)
             assert bool((same | (xs.isnan() & y.isnan())).all())
     fem.fem_device_error()  # cells of no volume are reported, here as anywhere
+
+
+@pytest.mark.parametrize("C", [33, 75000])
+@pytest.mark.parametrize("constant", [False, True])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_first_row_is_minus_the_sum(dim, constant, C):
+    """r_0 = -(0 + r_1 + ... + r_d) bit for bit, the signs of zeros of a constant field included: its
+    first and last operation run on the integer pipes."""
+    n = workloads.meshes.smallest_square_for(C) if dim == 2 else workloads.smallest_cube_for(C)
+    mesh = workloads.first_cells(workloads.square_mesh(n) if dim == 2 else workloads.cube_mesh(n), C)
+    rng = np.random.default_rng(C)
+    rule, V = workloads.rule_for_dim(dim), mesh.n_verts
+    dev = lambda a: to_dev(a, torch.float64)
+    m, pw = (dev(mesh.coords), to_dev(mesh.conn, torch.int32)), (rule.points, rule.weights)
+    field = lambda *s: dev(np.full(s, 0.75) if constant else rng.uniform(-1, 1, s))
+    K, M = dev(rng.lognormal(0, 1, (rule.n_q, C))), dev(rng.lognormal(0, 1, (rule.n_q, C)))
+    geom = fem.fem_precompute_geometry(*m, prec="fp64")
+    bits = lambda t: t.contiguous().view(torch.int64)
+    for r in (fem.fem_integrate_laplacian(*m, field(V), K, *pw, prec="fp64"),
+              fem.fem_integrate_laplacian_fields(*m, field(3, V), K, *pw, prec="fp64")[1],
+              fem.fem_integrate_laplacian_geom(m[1], V, field(V), K, *pw, geom, prec="fp64")):
+        total = torch.zeros_like(r[0])
+        for j in range(dim):
+            total = total + r[j + 1]
+        assert torch.equal(bits(r[0]), bits(-total))
+    e = fem.fem_integrate_elasticity(*m, field(dim, V), K, M, *pw, prec="fp64").view(dim + 1, dim, C)
+    total = torch.zeros_like(e[0])
+    for j in range(dim):
+        total = total - e[j + 1]
+    assert torch.equal(bits(e[0]), bits(total))
