@@ -53,9 +53,9 @@ HEADLINE_KERNEL = ("lap_pair_kernel<3, FP32_MIXED, NQ=4> (two consecutive cells 
 FLUSH_BYTES = 512 << 20
 # float64 instructions per cell of the float64 3D Laplacian kernel, counted by ncu
 # (smsp__sass_thread_inst_executed_op_dfma/dadd/dmul_pred_on.sum over one launch on the
-# 1,572,864-tet workload, divided by the cells): DFMA 30, DADD 7 (the 9 coordinate differences are
-# taken by integer operations), DMUL 21
-FP64_INST_PER_CELL_LAP3D = {"dfma": 30, "dadd": 7, "dmul": 21}
+# 1,572,864-tet workload, divided by the cells): DFMA 30, DADD 5 (the 9 coordinate differences, a
+# sum's first term and a sign are integer operations), DMUL 21
+FP64_INST_PER_CELL_LAP3D = {"dfma": 30, "dadd": 5, "dmul": 21}
 # FP64 peak: 1.25 TFLOP/s nominal for GB300 = 0.625 T FMA instructions/s, i.e. 2 float64
 # instructions per clock per SM at 2070 MHz on 152 SMs
 FP64_NOMINAL_TFLOPS = 1.25

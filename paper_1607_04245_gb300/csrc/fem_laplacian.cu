@@ -264,10 +264,10 @@ __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ Lap
 //
 // A solve in element form applies the float64 residual hundreds of times to one mesh and
 // coefficient. What of it does not depend on u, the adjugate rows n_j and s = Kbar / |det J|, is
-// formed once per cell, [dim * dim + 1][C], and an application does the rest: 27 instead of 58
+// formed once per cell, [dim * dim + 1][C], and an application does the rest: 26 instead of 56
 // float64 operations a tet, the same ones in the same order as lap_kernel's, so the same bits.
 // 80 more bytes per tet: the float64 pipe stays what an application waits for (1,572,864 tets: an
-// iteration of the solve 255 us at first, 125).
+// iteration of the solve 255 us, 119 so; the residual in it 78).
 
 template <int DIM>
 __global__ void __launch_bounds__(kWarpCta) lap_factors_kernel(const __grid_constant__ LapArgs a) {
