@@ -278,7 +278,7 @@ fem_status fem_integrate_laplacian_transposed(int dim, int64_t n_cells, const vo
  * Value arrays are float64 for FEM_FP64 and FEM_FP64_DF (the residual then runs in the
  * double-float form) and float32 otherwise; dot products accumulate in float64 (float32 vectors: in float32 pairs) in a fixed order (reproducible on
  * one device). The iteration is CG in Chronopoulos and Gear's form.
- * The float32 forms, and FEM_FP64 in 3D up to 45,000 cells times components, with
+ * The float32 forms, and FEM_FP64 in 3D up to 30,000 cells times components, with
  * fem_pcg_work_bytes() of workspace: the operator's rows are assembled on the device at the start of the solve, from element matrices in prec's
  * geometry, and the whole loop runs in one kernel, which occupies the device until the solve
  * ends; other streams' kernels run before or after it. A smaller workspace is accepted down to

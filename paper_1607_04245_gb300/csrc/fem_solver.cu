@@ -911,17 +911,18 @@ struct Workspace {
 // iterations, 2 of 120 on 200,000 to 1,000,000; elasticity 3 of 32 on 100,000 and 200,000; also in 2D,
 // and against the double-float operator, whose entries are 5e-14 off): x then differs by 3e-9, no
 // further from the solution, but float64 results are held to 1e-9 of the element form's. So float64
-// takes it on 3D meshes of up to kAssembled64 cells times components (the residual norms of 20
-// solves of 60,000 tets agreed to 3e-6, of 16 of elasticity on 20,000 to 3e-10).
-constexpr int64_t kAssembled64 = 45000;
+// takes it on 3D meshes of up to kAssembled64 cells times components (the residual norms of 150
+// solves of 30,000 tets agreed to 2e-5, of 150 of 45,000 to 1e-2).
+constexpr int64_t kAssembled64 = 30000;
 
 static bool assembled_form(int physics, int dim, int64_t C, fem_precision prec) {
     return prec == FEM_FP32_MIXED || prec == FEM_FP32 ||
            (prec == FEM_FP64 && dim == 3 && C * (physics == 0 ? 1 : dim) <= kAssembled64);
 }
 
-// The assembled operator is provided for up to kMatrixMaxBytes of workspace; beyond that (3D:
-// some 600 M cells for the Laplacian, 70 M for elasticity in float64) the solve runs in element form.
+// The assembled operator, and the factors, are provided for up to kMatrixMaxBytes of workspace; beyond
+// that (3D float32: some 1,200 M cells for the Laplacian, 240 M for elasticity; factors 430 M) a solve
+// runs in element form, or applies the residual kernel.
 constexpr size_t kMatrixMaxBytes = size_t(32) << 30;
 
 // what a solve's workspace holds beside its vectors: the assembled operator, or (element form of
