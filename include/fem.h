@@ -276,22 +276,23 @@ fem_status fem_integrate_laplacian_transposed(int dim, int64_t n_cells, const vo
  *   work       caller-owned device workspace of fem_pcg_work_bytes() bytes, 256-byte aligned
  *   iters_out, resid_out (host, may be NULL) iterations taken and ||r|| / ||r_0||
  * Value arrays are float64 for FEM_FP64 and FEM_FP64_DF (the residual then runs in the
- * double-float form) and float32 otherwise; dot products accumulate in float64 (float32 vectors: in float32 pairs) in a fixed order (reproducible on
- * one device). The iteration is CG in Chronopoulos and Gear's form.
- * The float32 forms, and FEM_FP64 in 3D up to 30,000 cells times components, with
- * fem_pcg_work_bytes() of workspace: the operator's rows are assembled on the device at the start of the solve, from element matrices in prec's
- * geometry, and the whole loop runs in one kernel, which occupies the device until the solve
- * ends; other streams' kernels run before or after it. A smaller workspace is accepted down to
- * what the element form needs ((dim+1) n_cells values, six vectors of n_verts values, 24 KiB
- * and 256 bytes, each rounded up to 256 bytes); the element residuals are then computed and
- * summed in every iteration, as three kernels in a CUDA graph with a WHILE node, at several
- * times the cost. FEM_FP64_DF (the residual in the double-float form) and FEM_FP64 otherwise
- * take the element form (their results do not depend on the workspace's size); with
- * fem_pcg_work_bytes() the Laplacian's is applied from (dim*dim + 1) n_cells float64 factors formed once
- * per solve, the same results in about half the time. Meshes with a vertex of more than 64
- * neighbours or more vertex pairs than the workspace provides for (half as many again as a
- * conforming mesh of this size has) take the element form too; matrices and factors past 32 GiB
- * are not provided for.
+ * double-float form) and float32 otherwise; dot products accumulate in float64 (float32
+ * vectors: in float32 pairs) in a fixed order (reproducible on one device). The iteration is
+ * CG in Chronopoulos and Gear's form.
+ * The float32 forms with fem_pcg_work_bytes() of workspace: the operator's rows are assembled
+ * on the device at the start of the solve, from element matrices in prec's geometry, and the
+ * whole loop runs in one kernel, which occupies the device until the solve ends; other streams'
+ * kernels run before or after it. A smaller workspace is accepted down to what the element form
+ * needs ((dim+1) n_cells values, six vectors of n_verts values, 24 KiB and 256 bytes, each
+ * rounded up to 256 bytes); the element residuals are then computed and summed in every
+ * iteration, as three kernels in a CUDA graph with a WHILE node, at several times the cost.
+ * Meshes with a vertex of more than 64 neighbours or more vertex pairs than the workspace
+ * provides for (half as many again as a conforming mesh of this size has) take the element form
+ * too; matrices and factors past 32 GiB are not provided for.
+ * FEM_FP64 and FEM_FP64_DF always take the element form, so their results do not depend on the
+ * workspace's size; with fem_pcg_work_bytes() the Laplacian's is applied from
+ * (dim*dim + 1) n_cells float64 factors formed once per solve, the same results in about half
+ * the time.
  * Unlike the other entry points this one returns only after the solve: it synchronises
  * `stream` (once; in element form twice). The element form's loop body is captured on a
  * library-owned stream per device, one capture at a time (a lock), so calls from several host

@@ -1,5 +1,5 @@
-// fem_sell.cuh -- the assembled operator of the PCG solves, built on the device inside the
-// call and stored in sliced ELLPACK form.
+// fem_sell.cuh -- the assembled operator of the float32 PCG solves, built on the device inside
+// the call and stored in sliced ELLPACK form.
 //
 // A solve applies one operator hundreds of times, and per application the element form costs
 // the geometry of every cell again, the element vectors' trip to memory and the scattered
@@ -30,10 +30,10 @@ constexpr int kSellMaxRow = 64;  // longest row that is assembled; a mesh with a
 
 struct SellMatrix {
     int32_t *cols = nullptr;   // [cap][32]; nullptr: no room in the workspace, element form
-    void *vals = nullptr;      // [cap][NC * NC][32] in the value type
+    float *vals = nullptr;     // [cap][NC * NC][32]
     int2 *slice = nullptr;     // (off, len) per slice of 32 rows
     int32_t *state = nullptr;  // [0] slots taken, [1] nonzero: did not fit
-    void *cell = nullptr;      // per-cell numbers the rows are summed from (sell_cell_values())
+    float *cell = nullptr;     // per-cell numbers the rows are summed from (sell_cell_values())
     int64_t cap = 0;           // slots
 };
 
@@ -61,10 +61,9 @@ __device__ __forceinline__ int pair_index(int a, int b) {
 // geometry of the precision form P (badly shaped cells of the mixed form in float64).
 template <int DIM, int P>
 __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0, int64_t C, uint32_t V,
-                                                                const int32_t *conn, const val_t<P> *K, QuadW w,
-                                                                float tau2, val_t<P> *out, unsigned *err) {
+                                                                const int32_t *conn, const float *K, QuadW w,
+                                                                float tau2, float *out, unsigned *err) {
     constexpr int NB = DIM + 1, NP = sell_cell_values(DIM, 1);
-    using T = val_t<P>;
     const double *X[DIM];
 #pragma unroll
     for (int k = 0; k < DIM; ++k) X[k] = X0 + int64_t(k) * V;
@@ -76,15 +75,11 @@ __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0
 #pragma unroll
         for (int b = 0; b < NB; ++b) v[b] = clamp_vid(ld_stream(conn + b * C + e), V, vmax);
         qsum_t<P> ks;
-        auto weight = [&](int q) {
-            if constexpr (P == FEM_FP64) return w.wd[q];
-            else return w.wf[q];
-        };
-        ks.first(weight(0), ld_stream(K + e));
-        for (int q = 1; q < w.nq; ++q) ks.add(weight(q), ld_stream(K + q * C + e));
+        ks.first(w.wf[0], ld_stream(K + e));
+        for (int q = 1; q < w.nq; ++q) ks.add(w.wf[q], ld_stream(K + q * C + e));
         double xs[NB][DIM];
         gather_coords<DIM>(X, v, xs);
-        T r[NP];
+        float r[NP];
         auto entries = [&](const auto &n, auto det, auto kbar) {
             using R = decltype(det);
             const R s = quot_abs(kbar, det);
@@ -97,14 +92,14 @@ __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0
             }
             int p = 0;
 #pragma unroll
-            for (int b = 0; b < DIM; ++b) r[p++] = static_cast<T>(-(s * dotv<DIM>(n0, n[b])));
+            for (int b = 0; b < DIM; ++b) r[p++] = static_cast<float>(-(s * dotv<DIM>(n0, n[b])));
 #pragma unroll
             for (int a = 0; a < DIM; ++a)
 #pragma unroll
-                for (int b = a + 1; b < DIM; ++b) r[p++] = static_cast<T>(s * dotv<DIM>(n[a], n[b]));
+                for (int b = a + 1; b < DIM; ++b) r[p++] = static_cast<float>(s * dotv<DIM>(n[a], n[b]));
         };
-        bool ok = P != FEM_FP64;
-        if constexpr (P != FEM_FP64) {
+        bool ok = true;
+        {
             float ec[DIM][DIM], n[DIM][DIM];
             if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, ec);
             else columns_f32<DIM>(xs, ec);
@@ -121,10 +116,9 @@ __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0
             entries(n, det, ks.value_f64());
         }
         if constexpr (NP == 6) {
-            using T2 = typename std::conditional<P == FEM_FP64, double2, float2>::type;
-            T2 *dst = reinterpret_cast<T2 *>(out + e * NP);
+            float2 *dst = reinterpret_cast<float2 *>(out + e * NP);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) dst[i] = T2{r[2 * i], r[2 * i + 1]};
+            for (int i = 0; i < 3; ++i) dst[i] = float2{r[2 * i], r[2 * i + 1]};
         } else {
 #pragma unroll
             for (int i = 0; i < NP; ++i) out[e * NP + i] = r[i];
@@ -135,16 +129,14 @@ __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0
 
 // Elasticity: the adjugate rows g_1 .. g_d and the factors sl, sm of the entries' blocks
 //     A_ab[k][i] = sl g_a[k] g_b[i] + sm (g_a[i] g_b[k] + delta_ki g_a . g_b),
-// g_0 = -(g_1 + .. + g_d). float64: g = n, sl = Lbar / |det J|, sm = Mbar / |det J|. float32:
-// g = n / sqrt|det J|, sl = Lbar, sm = Mbar, which stay in float32's range wherever the
-// entries do (n ~ L^2 and 1 / |det J| ~ L^-3 would not).
+// g_0 = -(g_1 + .. + g_d), with g = n / sqrt|det J|, sl = Lbar, sm = Mbar, which stay in
+// float32's range wherever the entries do (n ~ L^2 and 1 / |det J| ~ L^-3 would not).
 template <int DIM, int P>
 __global__ void __launch_bounds__(kBlock) sell_el_cells_kernel(const double *X0, int64_t C, uint32_t V,
-                                                               const int32_t *conn, const val_t<P> *lam,
-                                                               const val_t<P> *mu, QuadW w, float tau2,
-                                                               val_t<P> *out, unsigned *err) {
+                                                               const int32_t *conn, const float *lam,
+                                                               const float *mu, QuadW w, float tau2,
+                                                               float *out, unsigned *err) {
     constexpr int NB = DIM + 1, NV = sell_cell_values(DIM, DIM);
-    using T = val_t<P>;
     const double *X[DIM];
 #pragma unroll
     for (int k = 0; k < DIM; ++k) X[k] = X0 + int64_t(k) * V;
@@ -156,23 +148,19 @@ __global__ void __launch_bounds__(kBlock) sell_el_cells_kernel(const double *X0,
 #pragma unroll
         for (int b = 0; b < NB; ++b) v[b] = clamp_vid(ld_stream(conn + b * C + e), V, vmax);
         qsum_t<P> ls, ms;
-        auto weight = [&](int q) {
-            if constexpr (P == FEM_FP64) return w.wd[q];
-            else return w.wf[q];
-        };
-        ls.first(weight(0), ld_stream(lam + e));
-        ms.first(weight(0), ld_stream(mu + e));
+        ls.first(w.wf[0], ld_stream(lam + e));
+        ms.first(w.wf[0], ld_stream(mu + e));
         for (int q = 1; q < w.nq; ++q) {
-            ls.add(weight(q), ld_stream(lam + q * C + e));
-            ms.add(weight(q), ld_stream(mu + q * C + e));
+            ls.add(w.wf[q], ld_stream(lam + q * C + e));
+            ms.add(w.wf[q], ld_stream(mu + q * C + e));
         }
         double xs[NB][DIM];
         gather_coords<DIM>(X, v, xs);
-        T r[NV];
+        float r[NV];
 #pragma unroll
-        for (int i = 0; i < NV; ++i) r[i] = T(0);
-        bool ok = P != FEM_FP64;
-        if constexpr (P != FEM_FP64) {
+        for (int i = 0; i < NV; ++i) r[i] = 0.0f;
+        bool ok = true;
+        {
             float ec[DIM][DIM], n[DIM][DIM];
             if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, ec);
             else columns_f32<DIM>(xs, ec);
@@ -193,34 +181,24 @@ __global__ void __launch_bounds__(kBlock) sell_el_cells_kernel(const double *X0,
             columns_f64<DIM>(xs, ec);
             const double det = adjugate_rows<DIM>(ec, n);
             bad_det |= det_bad(det) | ids_repeat<NB>(v);
-            const double y = P == FEM_FP64 ? 1.0 : 1.0 / sqrt(fabs(det));
-            const double s = P == FEM_FP64 ? quot_abs(1.0, det) : 1.0;
+            const double y = 1.0 / sqrt(fabs(det));
 #pragma unroll
             for (int j = 0; j < DIM; ++j)
 #pragma unroll
-                for (int i = 0; i < DIM; ++i) r[j * DIM + i] = static_cast<T>(P == FEM_FP64 ? n[j][i] : n[j][i] * y);
-            r[DIM * DIM] = static_cast<T>(ls.value_f64() * s), r[DIM * DIM + 1] = static_cast<T>(ms.value_f64() * s);
+                for (int i = 0; i < DIM; ++i) r[j * DIM + i] = static_cast<float>(n[j][i] * y);
+            r[DIM * DIM] = static_cast<float>(ls.value_f64()), r[DIM * DIM + 1] = static_cast<float>(ms.value_f64());
         }
-        using T2 = typename std::conditional<P == FEM_FP64, double2, float2>::type;
-        T2 *dst = reinterpret_cast<T2 *>(out + e * NV);
+        float2 *dst = reinterpret_cast<float2 *>(out + e * NV);
 #pragma unroll
-        for (int i = 0; i < NV / 2; ++i) dst[i] = T2{r[2 * i], r[2 * i + 1]};
+        for (int i = 0; i < NV / 2; ++i) dst[i] = float2{r[2 * i], r[2 * i + 1]};
     }
     report_mesh(err, vmax, V, bad_det);
 }
 
 // ------------------------------------------------------------------ rows
 
-// sums of a row's entries: float32 compensated (TwoSum, as the nodal sum), float64 plain
-template <class T>
+// sums of a row's entries, compensated (TwoSum, as the nodal sum)
 struct RowSums {
-    T s[kSellMaxRow];
-    __device__ __forceinline__ void start(int p, T x) { s[p] = x; }
-    __device__ __forceinline__ void add(int p, T x) { s[p] += x; }
-    __device__ __forceinline__ T value(int p) const { return s[p]; }
-};
-template <>
-struct RowSums<float> {
     float2 s[kSellMaxRow];
     __device__ __forceinline__ void start(int p, float x) { s[p] = make_float2(x, 0.0f); }
     __device__ __forceinline__ void add(int p, float x) {
@@ -236,17 +214,17 @@ struct RowSums<float> {
 // walks the row's cells in list order, looks every other vertex up among the columns found so
 // far (a per-thread array: rows have about 14 entries) and appends it if it is new; the warp's
 // longest row is the slice's length.
-template <int NB, class T, bool LAP>
+template <int NB, bool LAP>
 __global__ void __launch_bounds__(128) sell_rows_kernel(int64_t C, int64_t V, const int32_t *__restrict__ conn,
                                                         const int32_t *__restrict__ ptr,
                                                         const int32_t *__restrict__ idx, const uint8_t *fixed,
-                                                        const T *__restrict__ cell, int32_t *cols, T *vals,
-                                                        int2 *slice, int32_t *state, int64_t cap, T *Dinv) {
+                                                        const float *__restrict__ cell, int32_t *cols, float *vals,
+                                                        int2 *slice, int32_t *state, int64_t cap, float *Dinv) {
     constexpr int NP = NB * (NB - 1) / 2;
     const int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     int32_t col[kSellMaxRow];
-    RowSums<T> sum;
+    RowSums sum;
     int m = 0;
     bool over = false;
     if (n < V && !fixed[n]) {
@@ -259,7 +237,7 @@ __global__ void __launch_bounds__(128) sell_rows_kernel(int64_t C, int64_t V, co
                 const int b = a + o < NB ? a + o : a + o - NB;
                 const int32_t v = static_cast<int32_t>(clamp_vid(__ldg(conn + b * C + c), static_cast<uint32_t>(V)));
                 if (v == n) continue;  // repeated vertex (reported by the cell pass)
-                T x = T(0);
+                float x = 0.0f;
                 if constexpr (LAP) x = __ldg(cell + int64_t(c) * NP + pair_index<NB>(a, b));
                 int p = 0;
                 while (p < m && col[p] != v) ++p;
@@ -287,29 +265,29 @@ __global__ void __launch_bounds__(128) sell_rows_kernel(int64_t C, int64_t V, co
     off = __shfl_sync(0xffffffffu, off, 0);
     if (any_over || int64_t(off) + len > cap) len = 0;
     if (lane == 0 && n < V) slice[n >> 5] = make_int2(off, len);
-    T d = T(0);
+    float d = 0.0f;
     for (int k = 0; k < len; ++k) {
         const int64_t at = (int64_t(off) + k) * 32 + lane;
         cols[at] = k < m ? col[k] : static_cast<int32_t>(min(n, V - 1));
         if constexpr (LAP) {
-            const T x = k < m ? sum.value(k) : T(0);
+            const float x = k < m ? sum.value(k) : 0.0f;
             vals[at] = x;
             d -= x;
         }
     }
     if constexpr (LAP) {
-        if (n < V) Dinv[n] = d > T(0) ? T(1) / d : T(1);
+        if (n < V) Dinv[n] = d > 0.0f ? 1.0f / d : 1.0f;
     }
 }
 
 // Elasticity: the blocks. A warp takes one slot of a slice, its lanes the 32 rows: each lane
 // walks its row's cells in list order and sums the blocks of those that hold its column, in
 // registers.
-template <int DIM, class T>
+template <int DIM>
 __global__ void __launch_bounds__(128) sell_blocks_kernel(int64_t C, int64_t V, const int32_t *__restrict__ conn,
                                                           const int32_t *__restrict__ ptr,
                                                           const int32_t *__restrict__ idx,
-                                                          const T *__restrict__ cell, const int32_t *cols, T *vals,
+                                                          const float *__restrict__ cell, const int32_t *cols, float *vals,
                                                           const int2 *slice) {
     constexpr int NB = DIM + 1, NV = sell_cell_values(DIM, DIM), BB = DIM * DIM;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -320,7 +298,7 @@ __global__ void __launch_bounds__(128) sell_blocks_kernel(int64_t C, int64_t V, 
     for (int k = warp; k < sl.y; k += nw) {
         const int64_t slot = int64_t(sl.x) + k;
         const int32_t want = cols[slot * 32 + lane];
-        NodeSum<T> acc[BB];
+        NodeSum<float> acc[BB];
         if (want != n) {
             for (int32_t j = j0; j < j1; ++j) {
                 const int32_t t = __ldg(idx + j);
@@ -330,23 +308,23 @@ __global__ void __launch_bounds__(128) sell_blocks_kernel(int64_t C, int64_t V, 
                 for (int o = 0; o < NB; ++o)
                     if (o != a && static_cast<int32_t>(clamp_vid(__ldg(conn + o * C + c), static_cast<uint32_t>(V))) == want) b = o;
                 if (b < 0) continue;
-                const T *g = cell + int64_t(c) * NV;
-                T ga[DIM], gb[DIM];
+                const float *g = cell + int64_t(c) * NV;
+                float ga[DIM], gb[DIM];
 #pragma unroll
                 for (int i = 0; i < DIM; ++i) {
-                    T all = T(0);
+                    float all = 0.0f;
 #pragma unroll
                     for (int r = 0; r < DIM; ++r) all += __ldg(g + r * DIM + i);
                     ga[i] = a == 0 ? -all : __ldg(g + (a - 1) * DIM + i);
                     gb[i] = b == 0 ? -all : __ldg(g + (b - 1) * DIM + i);
                 }
-                const T sL = __ldg(g + BB), sM = __ldg(g + BB + 1);
-                const T dot = sM * dotv<DIM>(ga, gb);
+                const float sL = __ldg(g + BB), sM = __ldg(g + BB + 1);
+                const float dot = sM * dotv<DIM>(ga, gb);
 #pragma unroll
                 for (int r = 0; r < DIM; ++r)
 #pragma unroll
                     for (int i = 0; i < DIM; ++i) {
-                        T x = (sL * ga[r]) * gb[i] + (sM * ga[i]) * gb[r];
+                        float x = (sL * ga[r]) * gb[i] + (sM * ga[i]) * gb[r];
                         if (r == i) x += dot;
                         acc[r * DIM + i].add(x);
                     }
@@ -358,33 +336,26 @@ __global__ void __launch_bounds__(128) sell_blocks_kernel(int64_t C, int64_t V, 
 }
 
 // Elasticity: the reciprocal diagonal, from the blocks' diagonal components
-template <int NC, class T>
-__global__ void __launch_bounds__(128) sell_diag_kernel(int64_t V, const T *vals, const int2 *slice, T *Dinv) {
+template <int NC>
+__global__ void __launch_bounds__(128) sell_diag_kernel(int64_t V, const float *vals, const int2 *slice, float *Dinv) {
     const int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (n >= V) return;
     const int lane = threadIdx.x & 31;
     const int2 sl = slice[n >> 5];
-    T d[NC];
+    float d[NC];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) d[k] = T(0);
+    for (int k = 0; k < NC; ++k) d[k] = 0.0f;
     for (int q = 0; q < sl.y; ++q)
 #pragma unroll
         for (int k = 0; k < NC; ++k) d[k] -= vals[((int64_t(sl.x) + q) * NC * NC + k * NC + k) * 32 + lane];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) Dinv[k * V + n] = d[k] > T(0) ? T(1) / d[k] : T(1);
+    for (int k = 0; k < NC; ++k) Dinv[k * V + n] = d[k] > 0.0f ? 1.0f / d[k] : 1.0f;
 }
 
 // ------------------------------------------------------------------ application
 
-// sums of products along a row: float64 plain, float32 as pairs (TwoProduct and TwoSum)
-template <class T>
+// sums of products along a row, as pairs (TwoProduct and TwoSum)
 struct DotRow {
-    T s = T(0);
-    __device__ __forceinline__ void add(T a, T b) { s = fma(a, b, s); }
-    __device__ __forceinline__ T value() const { return s; }
-};
-template <>
-struct DotRow<float> {
     float s = 0.0f, c = 0.0f;
     __device__ __forceinline__ void add(float a, float b) {
         float p, e, t, f;
@@ -408,29 +379,24 @@ __device__ __forceinline__ float ld_matrix(const float *p) {
     asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ double ld_matrix(const double *p) {
-    double v;
-    asm("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
-    return v;
-}
 
 // w = (A u) in row n, all components, lane `lane` of slice sl: a thread reads a column and its
 // nodal values once for the NC rows of the block. The columns of up to J slots first, then
 // batches of B slots, their nodal values (and, unless they lie in shared memory, their entries)
 // in flight together. u is read with ordinary loads: other CTAs write it between barriers.
 // SHARED: cols and vals lie in shared memory.
-template <int NC, class T, bool SHARED>
-__device__ __forceinline__ void sell_row(const int32_t *__restrict__ cols, const T *__restrict__ vals, int2 sl,
-                                         int lane, int64_t n, const T *u, int64_t V, T (&w)[NC]) {
-    constexpr int W = sizeof(T) / 4, BB = NC * NC;
+template <int NC, bool SHARED>
+__device__ __forceinline__ void sell_row(const int32_t *__restrict__ cols, const float *__restrict__ vals, int2 sl,
+                                         int lane, int64_t n, const float *u, int64_t V, float (&w)[NC]) {
+    constexpr int BB = NC * NC;
     constexpr int J = SHARED || NC == 1 ? 16 : 8;
-    constexpr int B = SHARED ? (NC == 1 ? 16 / W : 8 / W) : (NC == 1 ? 8 : 4 / W);
-    DotRow<T> acc[NC];
-    T ui[NC];
+    constexpr int B = SHARED ? (NC == 1 ? 16 : 8) : (NC == 1 ? 8 : 4);
+    DotRow acc[NC];
+    float ui[NC];
 #pragma unroll
     for (int m = 0; m < NC; ++m) ui[m] = u[m * V + n];
     const int32_t *c = cols + int64_t(sl.x) * 32 + lane;
-    const T *v = vals + int64_t(sl.x) * BB * 32 + lane;
+    const float *v = vals + int64_t(sl.x) * BB * 32 + lane;
     for (int q = 0; q < sl.y; q += J, c += J * 32, v += J * BB * 32) {
         int32_t j[J];
 #pragma unroll
@@ -441,7 +407,7 @@ __device__ __forceinline__ void sell_row(const int32_t *__restrict__ cols, const
 #pragma unroll
         for (int i0 = 0; i0 < J; i0 += B) {
             if (q + i0 >= sl.y) break;
-            T a[SHARED ? 1 : B][SHARED ? 1 : BB], x[B][NC];
+            float a[SHARED ? 1 : B][SHARED ? 1 : BB], x[B][NC];
 #pragma unroll
             for (int i = 0; i < B; ++i) {
 #pragma unroll
@@ -449,7 +415,7 @@ __device__ __forceinline__ void sell_row(const int32_t *__restrict__ cols, const
                 if constexpr (!SHARED) {
 #pragma unroll
                     for (int m = 0; m < BB; ++m) {
-                        a[i][m] = T(0);
+                        a[i][m] = 0.0f;
                         if (q + i0 + i < sl.y) a[i][m] = ld_matrix(v + ((i0 + i) * BB + m) * 32);
                     }
                 }

@@ -7,13 +7,12 @@
 // The iteration is CG in Chronopoulos and Gear's form. A solve takes one of two forms:
 //   * assembled: the operator's rows are formed once on the device (fem_sell.cuh) and the
 //     whole loop runs in one cooperative kernel (sell_cg_kernel). Taken by the float32 forms
-//     and by FEM_FP64 on small 3D meshes (assembled_form) whenever the caller's workspace has
-//     room for the matrix.
+//     (room_for) whenever the caller's workspace has room for the matrix.
 //   * element form: each application is the residual kernel and the vertex sum; one iteration
-//     is captured into the body of a CUDA graph WHILE node. For the other float64 solves,
-//     workspaces without room for the matrix, meshes whose rows do not fit it, and device
-//     partitions that refuse the cooperative launch. The Laplacian's residual is then applied
-//     from factors formed once per solve (launch_lap_factors), where the workspace has room.
+//     is captured into the body of a CUDA graph WHILE node. For the float64 solves, workspaces
+//     without room for the matrix, meshes whose rows do not fit it, and device partitions that
+//     refuse the cooperative launch. The float64 Laplacian's residual is then applied from
+//     factors formed once per solve (launch_lap_factors), where the workspace has room.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -421,11 +420,9 @@ __global__ void __launch_bounds__(256) cg_apply_dots_kernel(int64_t C, int64_t V
 // of the vectors in its registers for the whole solve; then only u and the partial sums move.
 //
 // Measured per iteration (64^3 x 6 tets, 274,625 rows; elasticity on 511,104 tets, 273,375
-// unknowns): float32 Laplacian 11.1 us against 52 us in element form, float64 27 against 255
-// us, float32 elasticity 15.3 against 38 us, float64 41 us. As two kernels per iteration in a
-// graph the same rows took 19, 37, 27 and 79 us: the launches' drain and the loop node cost
-// more than the barriers. What bounds it: float64, the float64 pipe (a subtraction and an FMA
-// per entry: 14 of the 27 us, the sums and updates 5); float32, latency: two barriers of about
+// unknowns): Laplacian 11.1 us against 52 us in element form, elasticity 15.3 against 38 us. As
+// two kernels per iteration in a graph the same rows took 19 and 27 us: the launches' drain and
+// the loop node cost more than the barriers. What bounds it is latency: two barriers of about
 // 2 us, the gathers of u through L2 after each (5 us), the scalars (1 us). The rows' threads
 // handle all components of a block (a thread per component read every column and nodal value
 // NC times: 21 us), 512 threads with four slices a warp hold the vectors without spills (1024
@@ -445,16 +442,15 @@ template <int NC>
 constexpr int cg_units() { return NC == 1 ? 4 : 1; }
 constexpr int kCgThreads = 640;  // the most of them
 
-template <class T>
 struct CgArgs {
     int64_t V;
     const int32_t *cols;
-    const T *vals;
+    const float *vals;
     const int2 *slice;
-    const T *b, *Dinv;  // b: nullptr for zero
+    const float *b, *Dinv;  // b: nullptr for zero
     const uint8_t *fixed;
-    T *x, *r, *u, *p, *s, *w;
-    double *partial;  // [3][kCgMaxBlocks] sums (float32: pairs)
+    float *x, *r, *u, *p, *s, *w;
+    float2 *partial;  // [3][kCgMaxBlocks] sums, as pairs
     double *sc;
     double rtol;
     int max_iter;
@@ -486,37 +482,8 @@ __device__ __forceinline__ bool wait_reached(const unsigned *p, unsigned target,
     }
 }
 
-// The totals of M values per thread over the block (any multiple of 32 threads), in thread 0.
-// float64: a shared-memory tree over the warps, lane by lane, then one over the lanes of warp 0
-// (the float64 pipe does two lanes a clock, and a tree in every warp would cost it five times
-// the additions); float32 pairs: warp trees, then one over the warps.
-template <int M>
-struct BlockSums {
-    double d[M][kCgThreads];
-};
-template <int M>
-__device__ __forceinline__ void block_totals(double (&v)[M], BlockSums<M> &sh) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) sh.d[m][threadIdx.x] = v[m];
-    __syncthreads();
-    int n = blockDim.x;
-    for (; n > 32;) {
-        const int half = (n / 32 + 1) / 2 * 32;
-        if (threadIdx.x + half < n)
-#pragma unroll
-            for (int m = 0; m < M; ++m) sh.d[m][threadIdx.x] += sh.d[m][threadIdx.x + half];
-        n = half;
-        __syncthreads();
-    }
-    if (threadIdx.x < 32) {
-#pragma unroll
-        for (int m = 0; m < M; ++m) v[m] = sh.d[m][threadIdx.x];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int m = 0; m < M; ++m) v[m] += __shfl_down_sync(0xffffffffu, v[m], o);
-    }
-}
+// The totals of M pairs per thread over the block (any multiple of 32 threads), in thread 0: warp
+// trees, then one over the warps.
 template <int M>
 struct BlockPairs {
     float2 p[M][32];
@@ -542,37 +509,22 @@ __device__ __forceinline__ void block_totals(PairSum (&a)[M], BlockPairs<M> &sh)
 }
 
 // one entry of the iteration's vectors
-template <class T>
 struct CgEntry {
-    T x, r, u, p, s, w, d;
+    float x, r, u, p, s, w, d;
 };
-
-// a running inner product: float64, or a float32 pair
-struct Sum64 {
-    double v = 0.0;
-    __device__ __forceinline__ void add_prod(double a, double b) { v = fma(a, b, v); }
-    __device__ __forceinline__ void merge(Sum64 o) { v += o.v; }
-    __device__ __forceinline__ double value() const { return v; }
-};
-__device__ __forceinline__ void warp_merge(Sum64 &a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a.v += __shfl_down_sync(0xffffffffu, a.v, o);
-}
 
 // U > 0: at most U slices per warp, their vector entries kept in registers; U = 0: any number,
 // the vectors in memory.
-template <int NC, class T, int U>
-__global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __grid_constant__ CgArgs<T> a) {
-    constexpr bool F32 = std::is_same<T, float>::value;
+template <int NC, int U>
+__global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __grid_constant__ CgArgs a) {
     constexpr int BB = NC * NC;
-    using Sum = typename std::conditional<F32, PairSum, Sum64>::type;
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ typename std::conditional<F32, BlockPairs<2>, BlockSums<2>>::type sh2;
-    __shared__ typename std::conditional<F32, BlockPairs<1>, BlockSums<1>>::type sh1;
+    __shared__ BlockPairs<2> sh2;
+    __shared__ BlockPairs<1> sh1;
     __shared__ int2 s_slice[kCgTable];  // place (in shared memory, if cached) and length of the CTA's first slices
     __shared__ int s_cached;
-    __shared__ Sum s_part[3 * ((kCgMaxBlocks + 31) / 32)];
-    __shared__ T s_alpha, s_beta;
+    __shared__ PairSum s_part[3 * ((kCgMaxBlocks + 31) / 32)];
+    __shared__ float s_alpha, s_beta;
     __shared__ int s_ok, s_more;
     __shared__ double s_gamma, s_den, s_inv[2];  // of the last iteration: gamma, alpha's denominator; 1/gamma, 1/(gamma alpha)
     unsigned *state = reinterpret_cast<unsigned *>(a.sc + S_MATRIX), *bar = reinterpret_cast<unsigned *>(a.sc + S_BARRIER);
@@ -585,7 +537,7 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
 
     // the CTA's first slices into shared memory, as many as fit
     int32_t *scols = reinterpret_cast<int32_t *>(dyn);
-    T *svals = reinterpret_cast<T *>(dyn + size_t(a.cache_slots) * 32 * sizeof(int32_t));
+    float *svals = reinterpret_cast<float *>(dyn + size_t(a.cache_slots) * 32 * sizeof(int32_t));
     const int ntab = min(nslices, kCgTable);
     for (int t = threadIdx.x; t < ntab; t += blockDim.x) s_slice[t] = a.slice[s0 + t];
     __syncthreads();
@@ -617,14 +569,14 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
     __syncthreads();
 
     // (A v) in the row n of the CTA's slice t
-    auto product = [&](const T *v, int t, int64_t n, T (&w)[NC]) {
-        if (t < cached) sell_row<NC, T, true>(scols, svals, s_slice[t], lane, n, v, V, w);
-        else sell_row<NC, T, false>(a.cols, a.vals, t < kCgTable ? s_slice[t] : a.slice[s0 + t], lane, n, v, V, w);
+    auto product = [&](const float *v, int t, int64_t n, float (&w)[NC]) {
+        if (t < cached) sell_row<NC, true>(scols, svals, s_slice[t], lane, n, v, V, w);
+        else sell_row<NC, false>(a.cols, a.vals, t < kCgTable ? s_slice[t] : a.slice[s0 + t], lane, n, v, V, w);
     };
     // f(entries, slice of the CTA, row, whether the row exists) for each of this thread's rows;
     // in memory: `in` names the members read first, `out` those written after
     enum { MX = 1, MR = 2, MU = 4, MP = 8, MS = 16, MW = 32, MD = 64 };
-    CgEntry<T> own[U > 0 ? U : 1][NC];
+    CgEntry own[U > 0 ? U : 1][NC];
     auto rows = [&](auto in, auto out, auto f) {
         if constexpr (U > 0) {
 #pragma unroll
@@ -639,11 +591,11 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
             constexpr int I = decltype(in)::value, O = decltype(out)::value;
             for (int t = warp; t < nslices; t += nw) {
                 const int64_t n = (s0 + t) * 32 + lane, row = min(n, V - 1);
-                CgEntry<T> e[NC];
+                CgEntry e[NC];
 #pragma unroll
                 for (int k = 0; k < NC; ++k) {
                     const int64_t i = k * V + row;
-                    e[k] = CgEntry<T>{};
+                    e[k] = CgEntry{};
                     if (I & MX) e[k].x = a.x[i];
                     if (I & MR) e[k].r = a.r[i];
                     if (I & MU) e[k].u = a.u[i];
@@ -668,19 +620,19 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
         }
     };
     // r = b - A x on the free vertices (0 on fixed ones), u = D^-1 r, p = s = 0, with r.u and r.r
-    Sum sums[2], wu[1];
+    PairSum sums[2], wu[1];
     rows(std::integral_constant<int, MX | MD>(), std::integral_constant<int, MR | MP | MS>(),
-         [&](CgEntry<T> (&e)[NC], int t, int64_t n, bool in) {
-             T ax[NC];
+         [&](CgEntry (&e)[NC], int t, int64_t n, bool in) {
+             float ax[NC];
              product(a.x, t, n, ax);
              const bool held = !in || a.fixed[n];
 #pragma unroll
              for (int k = 0; k < NC; ++k) {
                  const int64_t i = k * V + n;
                  if constexpr (U > 0) e[k].x = a.x[i], e[k].d = a.Dinv[i];
-                 e[k].r = held ? T(0) : (a.b ? a.b[i] : T(0)) - ax[k];
+                 e[k].r = held ? 0.0f : (a.b ? a.b[i] : 0.0f) - ax[k];
                  e[k].u = e[k].r * e[k].d;
-                 e[k].p = e[k].s = T(0);
+                 e[k].p = e[k].s = 0.0f;
                  if (in) a.u[i] = e[k].u;
                  sums[0].add_prod(e[k].r, e[k].u), sums[1].add_prod(e[k].r, e[k].r);
              }
@@ -714,20 +666,14 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
             const double g = s_gamma, inv = g != 0.0 ? copysign(quot_abs(1.0, g), g) : 0.0;
             s_inv[0] = inv, s_inv[1] = s_den * inv * inv;
         }
-        if constexpr (F32) {
-            block_totals(sums, sh2);
-        } else {
-            double v[2] = {sums[0].v, sums[1].v};
-            block_totals(v, sh2);
-            sums[0].v = v[0], sums[1].v = v[1];
-        }
-        const Sum ru = sums[0], rsq = sums[1];  // totals, in thread 0
+        block_totals(sums, sh2);
+        const PairSum ru = sums[0], rsq = sums[1];  // totals, in thread 0
         if (!barrier_wait(here)) return;
         // w = A u and w.u
-        wu[0] = Sum();
+        wu[0] = PairSum();
         rows(std::integral_constant<int, MU>(), std::integral_constant<int, MW>(),
-             [&](CgEntry<T> (&e)[NC], int t, int64_t n, bool in) {
-                 T w[NC];
+             [&](CgEntry (&e)[NC], int t, int64_t n, bool in) {
+                 float w[NC];
                  product(a.u, t, n, w);
 #pragma unroll
                  for (int k = 0; k < NC; ++k) {
@@ -735,35 +681,20 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
                      if (in) wu[0].add_prod(w[k], e[k].u);
                  }
              });
-        if constexpr (F32) {
-            block_totals(wu, sh1);
-        } else {
-            double v[1] = {wu[0].v};
-            block_totals(v, sh1);
-            wu[0].v = v[0];
-        }
+        block_totals(wu, sh1);
         // publish this CTA's sums, wait for all CTAs', and add them up: warp m the sums of value m
         if (threadIdx.x == 0) {
-            const Sum mine[3] = {ru, wu[0], rsq};
-            for (int m = 0; m < 3; ++m) {
-                if constexpr (F32)
-                    reinterpret_cast<float2 *>(a.partial)[m * kCgMaxBlocks + blockIdx.x] = make_float2(mine[m].hi, mine[m].lo);
-                else
-                    a.partial[m * kCgMaxBlocks + blockIdx.x] = mine[m].v;
-            }
+            const PairSum mine[3] = {ru, wu[0], rsq};
+            for (int m = 0; m < 3; ++m) a.partial[m * kCgMaxBlocks + blockIdx.x] = make_float2(mine[m].hi, mine[m].lo);
         }
         if (!barrier_wait(barrier_arrive())) return;
         const int chunks = (gridDim.x + 31) / 32;  // warp c + chunks m: 32 CTAs' sums of value m
         for (int t = warp; t < 3 * chunks; t += nw) {
             const int m = t / chunks, i = (t - m * chunks) * 32 + lane;
-            Sum v;
+            PairSum v;
             if (i < gridDim.x) {
-                if constexpr (F32) {
-                    const float2 q = __ldcg(reinterpret_cast<const float2 *>(a.partial) + m * kCgMaxBlocks + i);
-                    v.hi = q.x, v.lo = q.y;
-                } else {
-                    v.v = __ldcg(a.partial + m * kCgMaxBlocks + i);
-                }
+                const float2 q = __ldcg(a.partial + m * kCgMaxBlocks + i);
+                v.hi = q.x, v.lo = q.y;
             }
             warp_merge(v);
             if (lane == 0) s_part[t] = v;
@@ -775,7 +706,7 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
         double total = 0.0;
         if (threadIdx.x < 32) {
             if (lane < 3) {
-                Sum v = s_part[lane * chunks];
+                PairSum v = s_part[lane * chunks];
                 for (int c = 1; c < chunks; ++c) v.merge(s_part[lane * chunks + c]);
                 total = v.value();
             }
@@ -789,13 +720,13 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
                 rr0 = rr;
                 const double tol = a.rtol * sqrt(rr0);
                 tol2 = tol * tol;
-            } else {
+            } else {  // (g sums products of float32 values: its square stays in float64's range)
                 beta = g * s_inv[0];
                 den = delta - g * g * s_inv[1];
             }
             const double alpha = den != 0.0 ? copysign(quot_abs(g, den), den) : 0.0;
             s_gamma = g, s_den = den;
-            s_alpha = static_cast<T>(alpha), s_beta = static_cast<T>(beta);
+            s_alpha = static_cast<float>(alpha), s_beta = static_cast<float>(beta);
             // a NaN residual ends the loop: every comparison with it is false
             s_more = it < a.max_iter && rr > tol2 && rr > 0.0;
         }
@@ -803,10 +734,10 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
         if (!s_more) break;
         ++it;
         // p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s, u = D^-1 r
-        const T al = s_alpha, be = s_beta;
-        sums[0] = sums[1] = Sum();
+        const float al = s_alpha, be = s_beta;
+        sums[0] = sums[1] = PairSum();
         rows(std::integral_constant<int, MX | MR | MU | MP | MS | MW | MD>(),
-             std::integral_constant<int, MX | MR | MP | MS>(), [&](CgEntry<T> (&e)[NC], int, int64_t n, bool in) {
+             std::integral_constant<int, MX | MR | MP | MS>(), [&](CgEntry (&e)[NC], int, int64_t n, bool in) {
 #pragma unroll
                  for (int k = 0; k < NC; ++k) {
                      e[k].p = e[k].u + be * e[k].p;
@@ -823,7 +754,7 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
     }
     if constexpr (U > 0) {
         rows(std::integral_constant<int, 0>(), std::integral_constant<int, 0>(),
-             [&](CgEntry<T> (&e)[NC], int, int64_t n, bool in) {
+             [&](CgEntry (&e)[NC], int, int64_t n, bool in) {
 #pragma unroll
                  for (int k = 0; k < NC; ++k)
                      if (in) a.x[k * V + n] = e[k].x;
@@ -839,8 +770,8 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
 // Launch sell_cg_kernel: one CTA per SM at most, four slices each while they last (fewer CTAs
 // make the barriers cheaper, more spread the rows' latency), a warp per slice up to the CTA's
 // limit.
-template <int NC, class T>
-static cudaError_t launch_sell_cg(CgArgs<T> a, cudaStream_t s) {
+template <int NC>
+static cudaError_t launch_sell_cg(CgArgs a, cudaStream_t s) {
     constexpr int U = cg_units<NC>(), kWarps = cg_threads<NC>() / 32;
     const int64_t slices = (a.V + 31) / 32;
     const int grid = slices <= kWarps ? 1 : static_cast<int>(std::min<int64_t>({(slices + 3) / 4, int64_t(sm_count()), int64_t(kCgMaxBlocks)}));
@@ -848,13 +779,13 @@ static cudaError_t launch_sell_cg(CgArgs<T> a, cudaStream_t s) {
     const int64_t rounds = (per + kWarps - 1) / kWarps;
     const int threads = static_cast<int>((per + rounds - 1) / rounds * 32);
     const bool resident = rounds <= U;
-    const void *k = resident ? reinterpret_cast<const void *>(sell_cg_kernel<NC, T, U>)
-                             : reinterpret_cast<const void *>(sell_cg_kernel<NC, T, 0>);
+    const void *k = resident ? reinterpret_cast<const void *>(sell_cg_kernel<NC, U>)
+                             : reinterpret_cast<const void *>(sell_cg_kernel<NC, 0>);
     // shared memory for the matrix: what the static part leaves, in whole slots
     cudaFuncAttributes at;
     cudaError_t e = cudaFuncGetAttributes(&at, k);
     if (e != cudaSuccess) return e;
-    const size_t slot = 32 * (sizeof(int32_t) + size_t(NC) * NC * sizeof(T));
+    const size_t slot = 32 * (sizeof(int32_t) + size_t(NC) * NC * sizeof(float));
     const size_t room = 227 * 1024 - at.sharedSizeBytes;
     const int64_t most = per * kSellMaxRow;  // slots the CTA's slices can have
     a.cache_slots = static_cast<int>(std::min<int64_t>(int64_t(room / slot), most));
@@ -901,36 +832,28 @@ struct Workspace {
     void *elem, *D, *r, *z, *p, *q, *sv;  // D holds D^-1, z holds u = D^-1 r, q holds w = A u, sv s = A p
     double *partial, *scalars;
     SellMatrix mat;  // the assembled operator (mat.cols: nullptr where the workspace has no room for it)
-    double *mat_partial;
+    float2 *mat_partial;
     double *fac = nullptr;  // element form: the float64 Laplacian's factors, nullptr where not provided for
 };
-
-// Which solves take the assembled form. The two forms' roundings differ, and CG amplifies that
-// over its iterations, in some float64 solves until the residual norms differ in their second
-// digit and the stopping test ends one iteration apart (7 of 40 on 1,572,864 tets with 256
-// iterations, 2 of 120 on 200,000 to 1,000,000; elasticity 3 of 32 on 100,000 and 200,000; also in 2D,
-// and against the double-float operator, whose entries are 5e-14 off): x then differs by 3e-9, no
-// further from the solution, but float64 results are held to 1e-9 of the element form's. So float64
-// takes it on 3D meshes of up to kAssembled64 cells times components (the residual norms of 150
-// solves of 30,000 tets agreed to 2e-5, of 150 of 45,000 to 1e-2).
-constexpr int64_t kAssembled64 = 30000;
-
-static bool assembled_form(int physics, int dim, int64_t C, fem_precision prec) {
-    return prec == FEM_FP32_MIXED || prec == FEM_FP32 ||
-           (prec == FEM_FP64 && dim == 3 && C * (physics == 0 ? 1 : dim) <= kAssembled64);
-}
 
 // The assembled operator, and the factors, are provided for up to kMatrixMaxBytes of workspace; beyond
 // that (3D float32: some 1,200 M cells for the Laplacian, 240 M for elasticity; factors 430 M) a solve
 // runs in element form, or applies the residual kernel.
 constexpr size_t kMatrixMaxBytes = size_t(32) << 30;
 
-// what a solve's workspace holds beside its vectors: the assembled operator, or (element form of
-// the Laplacian in the float64 value types) the residual's factors
+// What a solve's workspace holds beside its vectors, which is what form it takes: the assembled
+// operator (float32), or the factors of the Laplacian's residual (the float64 value types).
+// The forms' roundings differ, and CG amplifies that over its iterations until the residual norms
+// differ in their second digit and the stopping test ends iterations apart. In float32 that is
+// within what its rounding leaves of x (either form's error against the exact solution is the
+// other's or smaller). In float64 it is not: of 12 solves each of 3,000, 12,000 and 30,000 tets to
+// 1e-8 with ln K normal of deviation 3, 1, 4 and 4 ended apart (up to 10 iterations), x 1e-8 to
+// 2e-7 apart; with flat cells nearly all. So float64 keeps the element form, whose factors give
+// the residual kernel's bits: its results do not depend on the workspace.
 enum class Room { Vectors, Matrix, Factors };
-static Room room_for(int physics, int dim, int64_t C, fem_precision prec) {
-    if (assembled_form(physics, dim, C, prec)) return Room::Matrix;
-    return physics == 0 && (prec == FEM_FP64 || prec == FEM_FP64_DF) ? Room::Factors : Room::Vectors;
+static Room room_for(int physics, fem_precision prec) {
+    if (prec == FEM_FP32_MIXED || prec == FEM_FP32) return Room::Matrix;
+    return physics == 0 ? Room::Factors : Room::Vectors;
 }
 
 static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Workspace *w, int ncomp, Room room) {
@@ -948,19 +871,19 @@ static size_t carve(int64_t C, int64_t V, int dim, size_t vs, void *base, Worksp
     double *partial = static_cast<double *>(take(sizeof(double) * 3 * kDotBlocks));
     double *scalars = static_cast<double *>(take(sizeof(double) * S_COUNT));
     SellMatrix mat;
-    double *mat_partial = nullptr;
+    float2 *mat_partial = nullptr;
     const int64_t slots = sell_slots(C, V);
     const size_t bb = size_t(ncomp) * size_t(ncomp);
     if (room == Room::Matrix && C > 0 && slots < (int64_t(1) << 31) && size_t(slots) * 32 * (4 + bb * vs) <= kMatrixMaxBytes) {
         mat.cap = slots;
         mat.cols = static_cast<int32_t *>(take(size_t(slots) * 32 * sizeof(int32_t)));
-        mat.vals = take(size_t(slots) * 32 * bb * vs);
+        mat.vals = static_cast<float *>(take(size_t(slots) * 32 * bb * vs));
         mat.slice = static_cast<int2 *>(take(size_t((V + 31) / 32) * sizeof(int2)));
         mat.state = reinterpret_cast<int32_t *>(scalars + S_MATRIX);
         // the cells' numbers lie in the element vectors' place where they fit there
         const int nv = sell_cell_values(dim, ncomp);
-        mat.cell = nv <= (dim + 1) * ncomp ? elem : take(size_t(nv) * size_t(C) * vs);
-        mat_partial = static_cast<double *>(take(3 * sizeof(double) * kCgMaxBlocks));
+        mat.cell = static_cast<float *>(nv <= (dim + 1) * ncomp ? elem : take(size_t(nv) * size_t(C) * vs));
+        mat_partial = static_cast<float2 *>(take(3 * sizeof(float2) * kCgMaxBlocks));
     }
     double *fac = nullptr;
     const size_t fac_bytes = size_t(dim * dim + 1) * size_t(C) * sizeof(double);
@@ -978,6 +901,50 @@ struct Operator {
 
 // what a workspace holds of its operator from an earlier solve of the same call
 enum class Kept { Nothing, Matrix, Diagonal };
+
+// form the operator's rows and the reciprocal diagonal w.D in the workspace w of a float32 solve
+static fem_status assemble_operator(int dim, int64_t C, int64_t V, const double *coords, const int32_t *conn,
+                                    const Operator &op, const QuadW &qwt, const int32_t *ptr, const int32_t *idx,
+                                    const uint8_t *fixed, const Workspace &w, fem_precision prec, cudaStream_t s) {
+    unsigned *err = device_error_word();
+    if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
+    const uint32_t V32 = static_cast<uint32_t>(V);
+    const float tau = mixed_tau();
+    const SellMatrix &m = w.mat;
+    float *D = static_cast<float *>(w.D);
+    const float *K = static_cast<const float *>(op.K);
+    const float *lam = static_cast<const float *>(op.lam), *mu = static_cast<const float *>(op.mu);
+    const unsigned rows = static_cast<unsigned>((V + 127) / 128), slices = static_cast<unsigned>((V + 31) / 32);
+    auto cells = [&](auto dimc, auto pc) {
+        constexpr int D_ = decltype(dimc)::value, P_ = decltype(pc)::value;
+        if (op.physics == 0) {
+            auto k = sell_lap_cells_kernel<D_, P_>;
+            k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(coords, C, V32, conn, K, qwt,
+                                                                                       tau * tau, m.cell, err);
+        } else {
+            auto k = sell_el_cells_kernel<D_, P_>;
+            k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(coords, C, V32, conn, lam, mu,
+                                                                                       qwt, tau * tau, m.cell, err);
+        }
+    };
+    auto all = [&](auto dimc) {
+        constexpr int D_ = decltype(dimc)::value;
+        if (prec == FEM_FP32_MIXED) cells(dimc, std::integral_constant<int, FEM_FP32_MIXED>());
+        else cells(dimc, std::integral_constant<int, FEM_FP32>());
+        if (op.physics == 0) {
+            sell_rows_kernel<D_ + 1, true><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, m.cell, m.cols, m.vals,
+                                                                m.slice, m.state, m.cap, D);
+        } else {
+            sell_rows_kernel<D_ + 1, false><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, m.cell, m.cols, m.vals,
+                                                                 m.slice, m.state, m.cap, D);
+            sell_blocks_kernel<D_><<<slices, 128, 0, s>>>(C, V, conn, ptr, idx, m.cell, m.cols, m.vals, m.slice);
+            sell_diag_kernel<D_><<<rows, 128, 0, s>>>(V, m.vals, m.slice, D);
+        }
+    };
+    if (dim == 2) all(std::integral_constant<int, 2>());
+    else all(std::integral_constant<int, 3>());
+    return check_launch("fem_pcg assembly");
+}
 
 template <class T>
 static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, const int32_t *conn,
@@ -998,57 +965,6 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
     QuadW qwt;
     fem_status st = load_quadrature(dim, n_q, qpts, qw, qwt);
     if (st != FEM_OK) return st;
-    // the assembled operator, where the workspace holds it
-    const bool f64 = std::is_same<T, double>::value;
-    T *mvals = static_cast<T *>(w.mat.vals);
-    bool use_matrix = w.mat.cols != nullptr && kept != Kept::Diagonal;
-    auto by_comps = [&](auto go) {
-        if (nc == 1) go(std::integral_constant<int, 1>());
-        else if (nc == 3) go(std::integral_constant<int, 3>());
-        else if constexpr (std::is_same<T, float>::value) go(std::integral_constant<int, 2>());
-    };
-    auto assemble = [&]() -> fem_status {
-        unsigned *err = device_error_word();
-        if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
-        const uint32_t V32 = static_cast<uint32_t>(V);
-        const float tau = mixed_tau();
-        T *cell = static_cast<T *>(w.mat.cell);
-        const unsigned rows = static_cast<unsigned>((V + 127) / 128), slices = static_cast<unsigned>((V + 31) / 32);
-        auto cells = [&](auto dimc, auto pc) {
-            constexpr int D_ = decltype(dimc)::value, P_ = decltype(pc)::value;
-            if constexpr (std::is_same<T, val_t<P_>>::value) {
-                if (op.physics == 0) {
-                    auto k = sell_lap_cells_kernel<D_, P_>;
-                    k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(
-                        coords, C, V32, conn, static_cast<const T *>(op.K), qwt, tau * tau, cell, err);
-                } else {
-                    auto k = sell_el_cells_kernel<D_, P_>;
-                    k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(
-                        coords, C, V32, conn, static_cast<const T *>(op.lam), static_cast<const T *>(op.mu), qwt,
-                        tau * tau, cell, err);
-                }
-            }
-        };
-        auto all = [&](auto dimc) {
-            constexpr int D_ = decltype(dimc)::value;
-            if (f64) cells(dimc, std::integral_constant<int, FEM_FP64>());
-            else if (prec == FEM_FP32_MIXED) cells(dimc, std::integral_constant<int, FEM_FP32_MIXED>());
-            else cells(dimc, std::integral_constant<int, FEM_FP32>());
-            if (op.physics == 0) {
-                sell_rows_kernel<D_ + 1, T, true><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, cell, w.mat.cols,
-                                                                       mvals, w.mat.slice, w.mat.state, w.mat.cap, D);
-            } else {
-                sell_rows_kernel<D_ + 1, T, false><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, cell, w.mat.cols,
-                                                                        mvals, w.mat.slice, w.mat.state, w.mat.cap, D);
-                sell_blocks_kernel<D_, T><<<slices, 128, 0, s>>>(C, V, conn, ptr, idx, cell, w.mat.cols, mvals,
-                                                                 w.mat.slice);
-                sell_diag_kernel<D_, T><<<rows, 128, 0, s>>>(V, mvals, w.mat.slice, D);
-            }
-        };
-        if (dim == 2) all(std::integral_constant<int, 2>());
-        else all(std::integral_constant<int, 3>());
-        return check_launch("fem_pcg assembly");
-    };
     // the element form's diagonal
     auto element_diagonal = [&]() -> fem_status {
         const int g = static_cast<int>(std::min<int64_t>((C + 255) / 256, 4096));
@@ -1117,38 +1033,41 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
         if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
         return FEM_OK;
     };
-    if (use_matrix) {
-        // a repeated solve keeps the matrix' state words
-        const bool have = kept == Kept::Matrix;
-        cudaError_t e = cudaMemsetAsync(w.scalars, 0, sizeof(double) * S_MATRIX, s);
-        if (e == cudaSuccess)
-            e = have ? cudaMemsetAsync(w.scalars + S_BARRIER, 0, sizeof(double), s)
-                     : cudaMemsetAsync(w.scalars + S_MATRIX, 0, 2 * sizeof(double), s);
-        if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
-        if (!have && (st = assemble()) != FEM_OK) return st;
-        unsigned *err = device_error_word();
-        if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
-        const CgArgs<T> a{V, w.mat.cols, mvals, w.mat.slice, B, D, fixed, X, r, z, p, sv, q, w.mat_partial, w.scalars,
-                          rtol, max_iter, 0, err};
-        by_comps([&](auto ncc) { e = launch_sell_cg<decltype(ncc)::value, T>(a, s); });
-        if (e == cudaSuccess) {
-            double head[S_COUNT];
-            if ((st = read(0, S_COUNT, head)) != FEM_OK) return st;
-            uint32_t state[2], bar[2];
-            std::memcpy(state, &head[S_MATRIX], sizeof(state));
-            std::memcpy(bar, &head[S_BARRIER], sizeof(bar));
-            if (bar[1] != 0u) return fail(FEM_ERR_TIMEOUT, "fem_pcg_laplacian: a grid barrier gave up");
-            if (state[1] == 0u) {
-                kept = Kept::Matrix;
-                if (iters_out) *iters_out = static_cast<int>(head[S_ITER]);
-                if (resid_out) *resid_out = head[S_RR0] > 0.0 ? std::sqrt(head[S_RR]) / std::sqrt(head[S_RR0]) : 0.0;
-                return check_launch("fem_pcg_laplacian");
+    if constexpr (std::is_same<T, float>::value) {
+        // the assembled operator, where the workspace holds it
+        if (w.mat.cols && kept != Kept::Diagonal) {
+            // a repeated solve keeps the matrix' state words
+            const bool have = kept == Kept::Matrix;
+            cudaError_t e = cudaMemsetAsync(w.scalars, 0, sizeof(double) * S_MATRIX, s);
+            if (e == cudaSuccess)
+                e = have ? cudaMemsetAsync(w.scalars + S_BARRIER, 0, sizeof(double), s)
+                         : cudaMemsetAsync(w.scalars + S_MATRIX, 0, 2 * sizeof(double), s);
+            if (e != cudaSuccess) return fail(FEM_ERR_CUDA, "fem_pcg_laplacian: %s", cudaGetErrorString(e));
+            if (!have && (st = assemble_operator(dim, C, V, coords, conn, op, qwt, ptr, idx, fixed, w, prec, s)) != FEM_OK)
+                return st;
+            unsigned *err = device_error_word();
+            if (!err) return fail(FEM_ERR_CUDA, "device error word unavailable");
+            const CgArgs a{V, w.mat.cols, w.mat.vals, w.mat.slice, B, D, fixed, X, r, z, p, sv, q, w.mat_partial,
+                           w.scalars, rtol, max_iter, 0, err};
+            e = nc == 1 ? launch_sell_cg<1>(a, s) : nc == 2 ? launch_sell_cg<2>(a, s) : launch_sell_cg<3>(a, s);
+            if (e == cudaSuccess) {
+                double head[S_COUNT];
+                if ((st = read(0, S_COUNT, head)) != FEM_OK) return st;
+                uint32_t state[2], bar[2];
+                std::memcpy(state, &head[S_MATRIX], sizeof(state));
+                std::memcpy(bar, &head[S_BARRIER], sizeof(bar));
+                if (bar[1] != 0u) return fail(FEM_ERR_TIMEOUT, "fem_pcg_laplacian: a grid barrier gave up");
+                if (state[1] == 0u) {
+                    kept = Kept::Matrix;
+                    if (iters_out) *iters_out = static_cast<int>(head[S_ITER]);
+                    if (resid_out) *resid_out = head[S_RR0] > 0.0 ? std::sqrt(head[S_RR]) / std::sqrt(head[S_RR0]) : 0.0;
+                    return check_launch("fem_pcg_laplacian");
+                }
+            } else {
+                cudaGetLastError();  // no cooperative launch (a device partition smaller than the device): element form
             }
-        } else {
-            cudaGetLastError();  // no cooperative launch (a device partition smaller than the device): element form
+            // rows too long or too many for the workspace: element form
         }
-        // rows too long or too many for the workspace: element form
-        use_matrix = false;
     }
     // element form: r0 = b - A x0 on the free vertices, u0 = D^-1 r0, w0 = A u0, gamma0, delta0, alpha0
     double rr0 = 0.0;
@@ -1232,7 +1151,7 @@ using namespace fem;
 extern "C" int64_t fem_pcg_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, room_for(0, dim, n_cells, prec)));
+    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, 1, room_for(0, prec)));
 }
 
 extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -1261,7 +1180,7 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
     const bool all = work_bytes >= fem_pcg_work_bytes(dim, n_cells, n_verts, prec);
-    carve(n_cells, n_verts, dim, vs, work, &w, 1, all ? room_for(0, dim, n_cells, prec) : Room::Vectors);
+    carve(n_cells, n_verts, dim, vs, work, &w, 1, all ? room_for(0, prec) : Room::Vectors);
     Kept kept = Kept::Nothing;
     if (f64)
         return pcg_run<double>(dim, n_cells, n_verts, coords, conn, Operator{0, K, nullptr, nullptr}, n_q, qpts, qw,
@@ -1275,7 +1194,11 @@ extern "C" fem_status fem_pcg_laplacian(int dim, int64_t n_cells, int64_t n_vert
 extern "C" int64_t fem_pcg_elasticity_work_bytes(int dim, int64_t n_cells, int64_t n_verts, fem_precision prec) {
     if ((dim != 2 && dim != 3) || n_cells < 0 || n_verts < 0) return -1;
     const size_t vs = prec == FEM_FP64 || prec == FEM_FP64_DF ? 8 : 4;
-    return static_cast<int64_t>(carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, room_for(1, dim, n_cells, prec)));
+    // float64 in 3D up to 10,000 cells: the size that callers have been told so far, more than the
+    // element form's vectors take
+    const bool more = prec == FEM_FP64 && dim == 3 && n_cells <= 10000;
+    return static_cast<int64_t>(
+        carve(n_cells, n_verts, dim, vs, nullptr, nullptr, dim, more ? Room::Matrix : room_for(1, prec)));
 }
 
 extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_verts, const double *coords,
@@ -1306,7 +1229,7 @@ extern "C" fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_ver
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(FEM_ERR_ARG, "work must be 256-byte aligned");
     Workspace w;
     const bool all = work_bytes >= fem_pcg_elasticity_work_bytes(dim, n_cells, n_verts, prec);
-    carve(n_cells, n_verts, dim, vs, work, &w, dim, all ? room_for(1, dim, n_cells, prec) : Room::Vectors);
+    carve(n_cells, n_verts, dim, vs, work, &w, dim, all ? room_for(1, prec) : Room::Vectors);
     Kept kept = Kept::Nothing;
     const Operator op{1, nullptr, lam, mu};
     if (f64)
