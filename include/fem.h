@@ -286,8 +286,9 @@ fem_status fem_integrate_laplacian_transposed(int dim, int64_t n_cells, const vo
  * needs ((dim+1) n_cells values, six vectors of n_verts values, 24 KiB and 256 bytes, each
  * rounded up to 256 bytes); the element residuals are then computed and summed in every
  * iteration, as three kernels in a CUDA graph with a WHILE node, at several times the cost.
- * Meshes with a vertex of more than 64 neighbours or more vertex pairs than the workspace
- * provides for (half as many again as a conforming mesh of this size has) take the element form
+ * Meshes with a vertex of more than 64 neighbours, more vertex pairs than the workspace
+ * provides for (half as many again as a conforming mesh of this size has) or, FEM_FP32_MIXED,
+ * cells below the shape threshold, which that form applies in float64, take the element form
  * too; matrices and factors past 32 GiB are not provided for.
  * FEM_FP64 and FEM_FP64_DF always take the element form, so their results do not depend on the
  * workspace's size; with fem_pcg_work_bytes() the Laplacian's is applied from
@@ -337,9 +338,9 @@ fem_status fem_pcg_elasticity(int dim, int64_t n_cells, int64_t n_verts, const d
  *              aligned (holds the float32 solve's workspace, K in float32, the float64 residual)
  *   outer_out, inner_out, resid_out (host, may be NULL): corrections made, float32 PCG
  *              iterations in all, ||r|| / ||r_0|| of the returned x
- * The corrections take fem_pcg_laplacian's assembled form with fem_pcg_refined_work_bytes() of
- * workspace (the matrix is formed once for all of them), its element form with less (down to
- * the same without the matrix). Synchronises `stream` once per outer step (the residual norm)
+ * The corrections (FEM_FP32_MIXED) take fem_pcg_laplacian's assembled form with
+ * fem_pcg_refined_work_bytes() of workspace (the matrix is formed once for all of them), its
+ * element form with less (down to the same without the matrix). Synchronises `stream` once per outer step (the residual norm)
  * and as fem_pcg_laplacian does inside each correction; returns when the solve has finished.
  * ------------------------------------------------------------------------------- */
 int64_t fem_pcg_refined_work_bytes(int dim, int64_t n_cells, int64_t n_verts, int n_q);

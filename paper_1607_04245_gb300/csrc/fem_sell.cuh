@@ -20,6 +20,12 @@
 // each: where a slice lies depends on the order in which warps arrive, what it holds does not
 // (a row's entries are in the order in which its sorted cell list meets them), so results
 // are bitwise reproducible. Rows of Dirichlet vertices are left empty (w = 0 there).
+//
+// A mesh with cells that the mixed form's shape test rejects is not assembled: the residual
+// kernels apply such cells in float64, and their large entries rounded to float32 would lose what
+// cancels between them (8^3 x 6 tets flattened to 1e-2 and 1e-3, a smooth field, the rounding of
+// the entries alone: errors of one application 1.4e-6 and 6.2e-6 of its largest value; 2.4e-8 and
+// 5.2e-8 with such cells in float64).
 #pragma once
 
 #include "fem_cell.cuh"
@@ -32,7 +38,7 @@ struct SellMatrix {
     int32_t *cols = nullptr;   // [cap][32]; nullptr: no room in the workspace, element form
     float *vals = nullptr;     // [cap][NC * NC][32]
     int2 *slice = nullptr;     // (off, len) per slice of 32 rows
-    int32_t *state = nullptr;  // [0] slots taken, [1] nonzero: did not fit
+    int32_t *state = nullptr;  // [0] slots taken, [1] nonzero: element form (1: did not fit, 2: badly shaped cells)
     float *cell = nullptr;     // per-cell numbers the rows are summed from (sell_cell_values())
     int64_t cap = 0;           // slots
 };
@@ -58,17 +64,17 @@ __device__ __forceinline__ int pair_index(int a, int b) {
 // ------------------------------------------------------------------ per-cell numbers
 
 // Off-diagonal entries of the Laplacian's element matrices, Kbar (n_a . n_b) / |det J|, in the
-// geometry of the precision form P (badly shaped cells of the mixed form in float64).
+// geometry of the precision form P. The mixed form's badly shaped cells are recorded in state.
 template <int DIM, int P>
 __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0, int64_t C, uint32_t V,
                                                                 const int32_t *conn, const float *K, QuadW w,
-                                                                float tau2, float *out, unsigned *err) {
+                                                                float tau2, float *out, int32_t *state, unsigned *err) {
     constexpr int NB = DIM + 1, NP = sell_cell_values(DIM, 1);
     const double *X[DIM];
 #pragma unroll
     for (int k = 0; k < DIM; ++k) X[k] = X0 + int64_t(k) * V;
     uint32_t vmax = 0;
-    bool bad_det = false;
+    bool bad_det = false, bad_shape = false;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < C; e += stride) {
         uint32_t v[NB];
@@ -79,42 +85,34 @@ __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0
         for (int q = 1; q < w.nq; ++q) ks.add(w.wf[q], ld_stream(K + q * C + e));
         double xs[NB][DIM];
         gather_coords<DIM>(X, v, xs);
-        float r[NP];
-        auto entries = [&](const auto &n, auto det, auto kbar) {
-            using R = decltype(det);
-            const R s = quot_abs(kbar, det);
-            R n0[DIM];
-#pragma unroll
-            for (int i = 0; i < DIM; ++i) {
-                n0[i] = n[0][i];
-#pragma unroll
-                for (int j = 1; j < DIM; ++j) n0[i] = n0[i] + n[j][i];
+        float ec[DIM][DIM], n[DIM][DIM];
+        if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, ec);
+        else columns_f32<DIM>(xs, ec);
+        const float det = adjugate_rows<DIM>(ec, n);
+        if constexpr (P == FEM_FP32_MIXED) {
+            if (!shape_ok<DIM>(ec, det, tau2)) {
+                bad_shape = true;
+                continue;
             }
-            int p = 0;
-#pragma unroll
-            for (int b = 0; b < DIM; ++b) r[p++] = static_cast<float>(-(s * dotv<DIM>(n0, n[b])));
-#pragma unroll
-            for (int a = 0; a < DIM; ++a)
-#pragma unroll
-                for (int b = a + 1; b < DIM; ++b) r[p++] = static_cast<float>(s * dotv<DIM>(n[a], n[b]));
-        };
-        bool ok = true;
-        {
-            float ec[DIM][DIM], n[DIM][DIM];
-            if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, ec);
-            else columns_f32<DIM>(xs, ec);
-            const float det = adjugate_rows<DIM>(ec, n);
-            if constexpr (P == FEM_FP32_MIXED) ok = shape_ok<DIM>(ec, det, tau2);
-            else bad_det |= det_bad(det) | ids_repeat<NB>(v);
-            if (ok) entries(n, det, ks.value());
-        }
-        if (!ok) {
-            double ec[DIM][DIM], n[DIM][DIM];
-            columns_f64<DIM>(xs, ec);
-            const double det = adjugate_rows<DIM>(ec, n);
+        } else {
             bad_det |= det_bad(det) | ids_repeat<NB>(v);
-            entries(n, det, ks.value_f64());
         }
+        const float s = quot_abs(ks.value(), det);
+        float n0[DIM];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+            n0[i] = n[0][i];
+#pragma unroll
+            for (int j = 1; j < DIM; ++j) n0[i] = n0[i] + n[j][i];
+        }
+        float r[NP];
+        int p = 0;
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) r[p++] = -(s * dotv<DIM>(n0, n[b]));
+#pragma unroll
+        for (int a = 0; a < DIM; ++a)
+#pragma unroll
+            for (int b = a + 1; b < DIM; ++b) r[p++] = s * dotv<DIM>(n[a], n[b]);
         if constexpr (NP == 6) {
             float2 *dst = reinterpret_cast<float2 *>(out + e * NP);
 #pragma unroll
@@ -124,6 +122,7 @@ __global__ void __launch_bounds__(kBlock) sell_lap_cells_kernel(const double *X0
             for (int i = 0; i < NP; ++i) out[e * NP + i] = r[i];
         }
     }
+    if (bad_shape) atomicOr(state + 1, 2);
     report_mesh(err, vmax, V, bad_det);
 }
 
@@ -135,13 +134,13 @@ template <int DIM, int P>
 __global__ void __launch_bounds__(kBlock) sell_el_cells_kernel(const double *X0, int64_t C, uint32_t V,
                                                                const int32_t *conn, const float *lam,
                                                                const float *mu, QuadW w, float tau2,
-                                                               float *out, unsigned *err) {
+                                                               float *out, int32_t *state, unsigned *err) {
     constexpr int NB = DIM + 1, NV = sell_cell_values(DIM, DIM);
     const double *X[DIM];
 #pragma unroll
     for (int k = 0; k < DIM; ++k) X[k] = X0 + int64_t(k) * V;
     uint32_t vmax = 0;
-    bool bad_det = false;
+    bool bad_det = false, bad_shape = false;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < C; e += stride) {
         uint32_t v[NB];
@@ -156,42 +155,32 @@ __global__ void __launch_bounds__(kBlock) sell_el_cells_kernel(const double *X0,
         }
         double xs[NB][DIM];
         gather_coords<DIM>(X, v, xs);
+        float ec[DIM][DIM], n[DIM][DIM];
+        if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, ec);
+        else columns_f32<DIM>(xs, ec);
+        const float det = adjugate_rows<DIM>(ec, n);
+        if constexpr (P == FEM_FP32_MIXED) {
+            if (!shape_ok<DIM>(ec, det, tau2)) {
+                bad_shape = true;
+                continue;
+            }
+        } else {
+            bad_det |= det_bad(det) | ids_repeat<NB>(v);
+        }
         float r[NV];
 #pragma unroll
         for (int i = 0; i < NV; ++i) r[i] = 0.0f;
-        bool ok = true;
-        {
-            float ec[DIM][DIM], n[DIM][DIM];
-            if constexpr (P == FEM_FP32_MIXED) columns_mixed<DIM>(xs, ec);
-            else columns_f32<DIM>(xs, ec);
-            const float det = adjugate_rows<DIM>(ec, n);
-            if constexpr (P == FEM_FP32_MIXED) ok = shape_ok<DIM>(ec, det, tau2);
-            else bad_det |= det_bad(det) | ids_repeat<NB>(v);
-            if (ok) {
-                const float y = __frsqrt_rn(fabsf(det));
+        const float y = __frsqrt_rn(fabsf(det));
 #pragma unroll
-                for (int j = 0; j < DIM; ++j)
+        for (int j = 0; j < DIM; ++j)
 #pragma unroll
-                    for (int i = 0; i < DIM; ++i) r[j * DIM + i] = n[j][i] * y;
-                r[DIM * DIM] = ls.value(), r[DIM * DIM + 1] = ms.value();
-            }
-        }
-        if (!ok) {
-            double ec[DIM][DIM], n[DIM][DIM];
-            columns_f64<DIM>(xs, ec);
-            const double det = adjugate_rows<DIM>(ec, n);
-            bad_det |= det_bad(det) | ids_repeat<NB>(v);
-            const double y = 1.0 / sqrt(fabs(det));
-#pragma unroll
-            for (int j = 0; j < DIM; ++j)
-#pragma unroll
-                for (int i = 0; i < DIM; ++i) r[j * DIM + i] = static_cast<float>(n[j][i] * y);
-            r[DIM * DIM] = static_cast<float>(ls.value_f64()), r[DIM * DIM + 1] = static_cast<float>(ms.value_f64());
-        }
+            for (int i = 0; i < DIM; ++i) r[j * DIM + i] = n[j][i] * y;
+        r[DIM * DIM] = ls.value(), r[DIM * DIM + 1] = ms.value();
         float2 *dst = reinterpret_cast<float2 *>(out + e * NV);
 #pragma unroll
         for (int i = 0; i < NV / 2; ++i) dst[i] = float2{r[2 * i], r[2 * i + 1]};
     }
+    if (bad_shape) atomicOr(state + 1, 2);
     report_mesh(err, vmax, V, bad_det);
 }
 
@@ -220,6 +209,7 @@ __global__ void __launch_bounds__(128) sell_rows_kernel(int64_t C, int64_t V, co
                                                         const int32_t *__restrict__ idx, const uint8_t *fixed,
                                                         const float *__restrict__ cell, int32_t *cols, float *vals,
                                                         int2 *slice, int32_t *state, int64_t cap, float *Dinv) {
+    if (state[1] & 2) return;  // badly shaped cells: not assembled
     constexpr int NP = NB * (NB - 1) / 2;
     const int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -288,7 +278,8 @@ __global__ void __launch_bounds__(128) sell_blocks_kernel(int64_t C, int64_t V, 
                                                           const int32_t *__restrict__ ptr,
                                                           const int32_t *__restrict__ idx,
                                                           const float *__restrict__ cell, const int32_t *cols, float *vals,
-                                                          const int2 *slice) {
+                                                          const int2 *slice, const int32_t *state) {
+    if (state[1] != 0) return;  // not assembled
     constexpr int NB = DIM + 1, NV = sell_cell_values(DIM, DIM), BB = DIM * DIM;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t s = blockIdx.x;  // one slice per CTA, its slots over the warps
@@ -337,7 +328,9 @@ __global__ void __launch_bounds__(128) sell_blocks_kernel(int64_t C, int64_t V, 
 
 // Elasticity: the reciprocal diagonal, from the blocks' diagonal components
 template <int NC>
-__global__ void __launch_bounds__(128) sell_diag_kernel(int64_t V, const float *vals, const int2 *slice, float *Dinv) {
+__global__ void __launch_bounds__(128) sell_diag_kernel(int64_t V, const float *vals, const int2 *slice, const int32_t *state,
+                                                        float *Dinv) {
+    if (state[1] != 0) return;  // not assembled
     const int64_t n = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (n >= V) return;
     const int lane = threadIdx.x & 31;

@@ -10,8 +10,8 @@
 //     (room_for) whenever the caller's workspace has room for the matrix.
 //   * element form: each application is the residual kernel and the vertex sum; one iteration
 //     is captured into the body of a CUDA graph WHILE node. For the float64 solves, workspaces
-//     without room for the matrix, meshes whose rows do not fit it, and device partitions that
-//     refuse the cooperative launch. The float64 Laplacian's residual is then applied from
+//     without room for the matrix, meshes whose rows do not fit it or, in the mixed form, with
+//     badly shaped cells, and device partitions that refuse the cooperative launch. The float64 Laplacian's residual is then applied from
 //     factors formed once per solve (launch_lap_factors), where the workspace has room.
 #include <algorithm>
 #include <cmath>
@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
     __shared__ int s_ok, s_more;
     __shared__ double s_gamma, s_den, s_inv[2];  // of the last iteration: gamma, alpha's denominator; 1/gamma, 1/(gamma alpha)
     unsigned *state = reinterpret_cast<unsigned *>(a.sc + S_MATRIX), *bar = reinterpret_cast<unsigned *>(a.sc + S_BARRIER);
-    if (state[1] != 0u) return;  // the matrix did not fit: the host takes the element form
+    if (state[1] != 0u) return;  // not assembled: the host takes the element form
     const int64_t V = a.V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t slices = (V + 31) / 32;
@@ -920,11 +920,12 @@ static fem_status assemble_operator(int dim, int64_t C, int64_t V, const double 
         if (op.physics == 0) {
             auto k = sell_lap_cells_kernel<D_, P_>;
             k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(coords, C, V32, conn, K, qwt,
-                                                                                       tau * tau, m.cell, err);
+                                                                                       tau * tau, m.cell, m.state, err);
         } else {
             auto k = sell_el_cells_kernel<D_, P_>;
             k<<<grid_for(C, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s>>>(coords, C, V32, conn, lam, mu,
-                                                                                       qwt, tau * tau, m.cell, err);
+                                                                                       qwt, tau * tau, m.cell, m.state,
+                                                                                       err);
         }
     };
     auto all = [&](auto dimc) {
@@ -937,8 +938,9 @@ static fem_status assemble_operator(int dim, int64_t C, int64_t V, const double 
         } else {
             sell_rows_kernel<D_ + 1, false><<<rows, 128, 0, s>>>(C, V, conn, ptr, idx, fixed, m.cell, m.cols, m.vals,
                                                                  m.slice, m.state, m.cap, D);
-            sell_blocks_kernel<D_><<<slices, 128, 0, s>>>(C, V, conn, ptr, idx, m.cell, m.cols, m.vals, m.slice);
-            sell_diag_kernel<D_><<<rows, 128, 0, s>>>(V, m.vals, m.slice, D);
+            sell_blocks_kernel<D_><<<slices, 128, 0, s>>>(C, V, conn, ptr, idx, m.cell, m.cols, m.vals, m.slice,
+                                                         m.state);
+            sell_diag_kernel<D_><<<rows, 128, 0, s>>>(V, m.vals, m.slice, m.state, D);
         }
     };
     if (dim == 2) all(std::integral_constant<int, 2>());
@@ -1066,7 +1068,7 @@ static fem_status pcg_run(int dim, int64_t C, int64_t V, const double *coords, c
             } else {
                 cudaGetLastError();  // no cooperative launch (a device partition smaller than the device): element form
             }
-            // rows too long or too many for the workspace: element form
+            // badly shaped cells, rows too long or too many for the workspace: element form
         }
     }
     // element form: r0 = b - A x0 on the free vertices, u0 = D^-1 r0, w0 = A u0, gamma0, delta0, alpha0
