@@ -410,6 +410,34 @@ def fem_integrate_reaction_diffusion(coords, conn, u, a, qpts, qw, c=None, a_spa
     return out
 
 
+def _up256(n: int) -> int:
+    return (n + 255) // 256 * 256
+
+
+def _pcg_least_bytes(dim: int, C: int, V: int, n_comp: int, value_bytes: int) -> int:
+    """The smallest workspace that a PCG solve accepts (fem_pcg_laplacian in include/fem.h)."""
+    return (_up256((dim + 1) * n_comp * C * value_bytes) + 6 * _up256(n_comp * V * value_bytes) + _up256(24 * 1024)
+            + 256)
+
+
+def _refined_least_bytes(dim: int, C: int, V: int, n_q: int, n_comp: int) -> int:
+    """The same for a refined solve: the float32 solve's, the coefficients, residual and correction
+    in float32, the element vectors and two nodal vectors in float64, the sums."""
+    n_coef = 1 if n_comp == 1 else 2
+    return (_pcg_least_bytes(dim, C, V, n_comp, 4) + n_coef * _up256(4 * n_q * C) + 2 * _up256(4 * n_comp * V)
+            + _up256(8 * (dim + 1) * n_comp * C) + 2 * _up256(8 * n_comp * V) + _up256(8 * 1024) + 256)
+
+
+def _pcg_work(need: int, least: int, dev) -> torch.Tensor:
+    """A solve's workspace: all it can use, or, where the device has no room for that, the least it accepts."""
+    try:
+        return torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
+    except torch.OutOfMemoryError:
+        if least >= need:
+            raise
+    return torch.empty(max(least, 1), dtype=torch.uint8, device=dev)
+
+
 def fem_pcg_laplacian(coords, conn, K, qpts, qw, node_ptr, node_idx, fixed, x, b=None, max_iter=1000, rtol=1e-8,
                       work=None, prec="fp64", stream=None):
     """Solve the assembled Laplacian system on the free vertices (Dirichlet values in x).
@@ -419,9 +447,9 @@ def fem_pcg_laplacian(coords, conn, K, qpts, qw, node_ptr, node_idx, fixed, x, b
     dim, V, C = _mesh_sizes(coords, conn)
     nq = int(np.asarray(qw).shape[0]) if not isinstance(qw, torch.Tensor) else int(qw.shape[0])
     dev = coords.device
-    need = int(lib().fem_pcg_work_bytes(dim, C, V, p))
     if work is None:
-        work = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
+        need = int(lib().fem_pcg_work_bytes(dim, C, V, p))
+        work = _pcg_work(need, _pcg_least_bytes(dim, C, V, 1, dt.itemsize), dev)
     qp, w = _HostTable(qpts, (nq, dim), "qpts"), _HostTable(qw, (nq,), "qw")
     iters, resid = ctypes.c_int(0), ctypes.c_double(0.0)
     st = lib().fem_pcg_laplacian(
@@ -444,9 +472,9 @@ def fem_pcg_elasticity(coords, conn, lam, mu, qpts, qw, node_ptr, node_idx, fixe
     dim, V, C = _mesh_sizes(coords, conn)
     nq = int(np.asarray(qw).shape[0]) if not isinstance(qw, torch.Tensor) else int(qw.shape[0])
     dev = coords.device
-    need = int(lib().fem_pcg_elasticity_work_bytes(dim, C, V, p))
     if work is None:
-        work = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
+        need = int(lib().fem_pcg_elasticity_work_bytes(dim, C, V, p))
+        work = _pcg_work(need, _pcg_least_bytes(dim, C, V, dim, dt.itemsize), dev)
     qp, w = _HostTable(qpts, (nq, dim), "qpts"), _HostTable(qw, (nq,), "qw")
     iters, resid = ctypes.c_int(0), ctypes.c_double(0.0)
     st = lib().fem_pcg_elasticity(
@@ -474,7 +502,7 @@ def fem_pcg_laplacian_refined(coords, conn, K, qpts, qw, node_ptr, node_idx, fix
     if need < 0:
         raise ValueError("bad sizes")
     if work is None:
-        work = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
+        work = _pcg_work(need, _refined_least_bytes(dim, C, V, nq, 1), dev)
     qp, w = _HostTable(qpts, (nq, dim), "qpts"), _HostTable(qw, (nq,), "qw")
     outer, inner, resid = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_double(0.0)
     f64 = torch.float64
@@ -501,7 +529,7 @@ def fem_pcg_elasticity_refined(coords, conn, lam, mu, qpts, qw, node_ptr, node_i
     if need < 0:
         raise ValueError("bad sizes")
     if work is None:
-        work = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
+        work = _pcg_work(need, _refined_least_bytes(dim, C, V, nq, dim), dev)
     qp, w = _HostTable(qpts, (nq, dim), "qpts"), _HostTable(qw, (nq,), "qw")
     outer, inner, resid = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_double(0.0)
     f64 = torch.float64
