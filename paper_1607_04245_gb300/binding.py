@@ -10,13 +10,15 @@ fails, a RuntimeError is raised.
 The integration, adjoint and assembly functions first offer their arguments to the native
 marshalling module (csrc/fem_marshal.cpp), which makes the call if every argument is exactly
 what the entry point takes, at about a fifth of the host time, and returns None if not: then
-the code here converts what can be converted, or raises the error that names the argument.
+the code here converts what can be converted, or raises the error that names the argument. The
+code here also makes every call where that module cannot be used (native()).
 """
 
 from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from typing import Optional, Tuple, Union
 
 import numpy as np
@@ -107,16 +109,34 @@ def lib():
     return _lib
 
 
+class _Declines:
+    """In place of the marshalling module: leaves every call to the Python path."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def native():
-    """The native marshalling module, bound to the loaded libfem (raises if it has not been built)."""
+    """The native marshalling module, bound to the loaded libfem. Where it is not built, or built
+    against another torch or interpreter than the running one, every call takes the Python path
+    (the same C calls at some 20 us more of host time each), with one warning."""
     global _native
     if _native is None:
         L = lib()
         try:
             from . import _marshal
+            from .build import marshal_stamp
+
+            running, built = marshal_stamp(), getattr(_marshal, "built_for", "an unknown torch")
+            why = "" if built == running else f"built for {built}, running {running}"
         except ImportError as e:
-            raise RuntimeError("the marshalling module is not built: run __graft_entry__.build() "
-                               f"or python -m paper_1607_04245_gb300.build ({e})") from e
+            why = str(e)
+        if why:
+            warnings.warn("the native marshalling module is unavailable, calls are marshalled in Python: run "
+                          f"__graft_entry__.build() or python -m paper_1607_04245_gb300.build ({why})",
+                          RuntimeWarning, stacklevel=3)
+            _native = _Declines()
+            return _native
         names = ("fem_integrate_laplacian", "fem_integrate_laplacian_fields", "fem_integrate_elasticity",
                  "fem_integrate_reaction_diffusion", "fem_integrate_pointwise", "fem_integrate_laplacian_geom",
                  "fem_adjoint_laplacian", "fem_build_node2cell", "fem_gather_nodes", "fem_node2cell_work_size")

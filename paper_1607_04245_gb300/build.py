@@ -46,6 +46,22 @@ def _deps_mtime() -> float:
 MARSHAL = os.path.join(PKG, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 
+def marshal_stamp() -> str:
+    """What the marshalling module is compiled against (its inlined accessors read torch's own
+    structures): recorded in the module, compared before it is kept or used."""
+    import torch
+
+    return (f"torch {torch.__version__} abi {int(torch._C._GLIBCXX_USE_CXX11_ABI)} "
+            f"python {sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
+def _marshal_is_current() -> bool:
+    if not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < _deps_mtime():
+        return False
+    with open(MARSHAL, "rb") as f:
+        return marshal_stamp().encode() + b"\0" in f.read()
+
+
 def _build_marshal() -> None:
     """fem_marshal.cpp against this interpreter and the installed torch."""
     import torch
@@ -55,7 +71,8 @@ def _build_marshal() -> None:
     cuda_inc = [d for d in (os.path.join(cuda, "include"), "/usr/local/cuda/include") if os.path.isdir(d)]
     tmp = MARSHAL + ".tmp"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", sysconfig.get_path("include"),
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DFEM_MARSHAL_BUILT_FOR="{marshal_stamp()}"', "-I", sysconfig.get_path("include"),
            "-I", os.path.join(t, "include"), "-I", os.path.join(t, "include", "torch", "csrc", "api", "include")]
     cmd += [x for d in cuda_inc for x in ("-I", d)]
     cmd += [os.path.join(CSRC, "fem_marshal.cpp"), "-o", tmp, "-L", os.path.join(t, "lib"), "-ltorch_python",
@@ -67,8 +84,9 @@ def _build_marshal() -> None:
 
 
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
-    done = all(os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime() for f in (OUT, MARSHAL))
-    if not force and not verbose_ptxas and done:
+    if not force and not verbose_ptxas and os.path.exists(OUT) and os.path.getmtime(OUT) >= _deps_mtime():
+        if not _marshal_is_current():
+            _build_marshal()
         return OUT
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
@@ -87,7 +105,6 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
         marshal = ex.submit(_build_marshal)
         results = list(ex.map(compile_one, SOURCES))
-        marshal.result()
     if verbose_ptxas:
         for _, log in results:
             sys.stderr.write(log)
@@ -97,6 +114,7 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stderr}")
     os.replace(tmp, OUT)
+    marshal.result()  # a failure is raised with the library in place, which works without the module
     return OUT
 
 

@@ -480,4 +480,10 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", "native argument marsha
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&module); }
+// built_for: the torch and interpreter this was compiled against (build.marshal_stamp()); the
+// binding uses the module only where they are the running ones
+PyMODINIT_FUNC PyInit__marshal() {
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", FEM_MARSHAL_BUILT_FOR) != 0) Py_CLEAR(m);
+    return m;
+}
