@@ -140,7 +140,7 @@ def native():
         names = ("fem_integrate_laplacian", "fem_integrate_laplacian_fields", "fem_integrate_elasticity",
                  "fem_integrate_reaction_diffusion", "fem_integrate_pointwise", "fem_integrate_laplacian_geom",
                  "fem_adjoint_laplacian", "fem_build_node2cell", "fem_gather_nodes", "fem_node2cell_work_size")
-        _marshal.init(_check, {n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in names})
+        _marshal.init(_check, torch.cuda.Stream, {n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in names})
         _native = _marshal
     return _native
 

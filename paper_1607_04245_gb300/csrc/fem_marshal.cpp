@@ -48,6 +48,7 @@ struct Functions {
     decltype(&fem_node2cell_work_size) node2cell_work_size;
 } fn;
 PyObject *check = nullptr;  // binding._check(name, status): raises
+PyObject *stream_type = nullptr;  // torch.cuda.Stream
 
 // ------------------------------------------------------------------ arguments
 
@@ -119,7 +120,12 @@ at::ScalarType value_type(fem_precision p) { return p == FEM_FP64 || p == FEM_FP
 
 fem_stream stream(PyObject *o) {
     if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-    PyObject *n = PyLong_CheckExact(o) ? Py_NewRef(o) : PyObject_GetAttrString(o, "cuda_stream");
+    const bool number = PyLong_CheckExact(o);
+    if (!number && PyObject_IsInstance(o, stream_type) != 1) {
+        PyErr_Clear();
+        throw NotPlain();
+    }
+    PyObject *n = number ? Py_NewRef(o) : PyObject_GetAttrString(o, "cuda_stream");
     if (!n) {
         PyErr_Clear();
         throw NotPlain();
@@ -446,10 +452,10 @@ bool address(PyObject *d, const char *name, F &f) {
     return true;
 }
 
-// init(check, {name: address})
+// init(check, torch.cuda.Stream, {name: address})
 PyObject *init(PyObject *, PyObject *args) {
-    PyObject *c, *d;
-    if (!PyArg_ParseTuple(args, "OO!", &c, &PyDict_Type, &d)) return nullptr;
+    PyObject *c, *t, *d;
+    if (!PyArg_ParseTuple(args, "OO!O!", &c, &PyType_Type, &t, &PyDict_Type, &d)) return nullptr;
     if (!address(d, "fem_integrate_laplacian", fn.integrate_laplacian) ||
         !address(d, "fem_integrate_laplacian_fields", fn.integrate_laplacian_fields) ||
         !address(d, "fem_integrate_elasticity", fn.integrate_elasticity) ||
@@ -461,6 +467,7 @@ PyObject *init(PyObject *, PyObject *args) {
         !address(d, "fem_node2cell_work_size", fn.node2cell_work_size))
         return nullptr;
     Py_XSETREF(check, Py_NewRef(c));
+    Py_XSETREF(stream_type, Py_NewRef(t));
     Py_RETURN_NONE;
 }
 

@@ -81,3 +81,21 @@ def test_the_python_path_gives_the_same(fresh):
     with pytest.warns(RuntimeWarning):
         got = residual(c, d, "mixed")
     assert torch.equal(got, ref)
+
+
+@pytest.mark.gpu
+def test_what_is_no_stream_is_refused():
+    """An object that is no torch stream is refused as the Python path refuses it, whatever its attributes."""
+    import workloads
+    from gpu_util import device_arrays, residual
+
+    case = workloads.laplacian_cube_case(6 * 5 ** 3)
+    c, d = device_arrays(case, "mixed")
+    other = types.SimpleNamespace(cuda_stream=torch.cuda.current_stream().cuda_stream)
+    with pytest.raises(TypeError):
+        residual(c, d, "mixed", stream=other)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    r = residual(c, d, "mixed", stream=s)
+    s.synchronize()
+    assert torch.equal(r, residual(c, d, "mixed", stream=torch.cuda.current_stream().cuda_stream))
