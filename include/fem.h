@@ -645,9 +645,11 @@ fem_status fem_probe(int kind, int64_t n_threads, int iters, void *out, fem_stre
  * ------------------------------------------------------------------------------- */
 fem_status fem_device_error(fem_stream stream);
 
-/* fem_selftest_wait -- launches one CTA that waits, with a bounded wait and a budget of budget_ns (0 .. 10 s), for a barrier phase that never
- * completes, so that the next fem_device_error() returns FEM_ERR_TIMEOUT. For tests of
- * the timeout path; it faults nothing and leaves the context usable. */
+/* fem_selftest_wait -- launches one CTA that waits, with the bounded wait of the solves' loop
+ * kernel and a budget of budget_ns (0 .. 10 s), for a counter that stays one short of its
+ * target, so that the next fem_device_error() returns FEM_ERR_TIMEOUT (only if the wait also
+ * returned at once for targets that were reached). For tests of the timeout path; it faults
+ * nothing and leaves the context usable. */
 fem_status fem_selftest_wait(int64_t budget_ns, fem_stream stream);
 
 /* fem_selftest_quotient -- the float64 kernels' division num / |det J| on the device, for

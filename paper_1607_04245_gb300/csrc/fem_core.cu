@@ -231,15 +231,22 @@ __global__ void __launch_bounds__(256) probe_kernel(int iters, void *out) {
     }
 }
 
-// Self-test of the bounded wait: one thread initialises an mbarrier that expects two
-// arrivals, arrives once, and waits for a phase that can never complete.
-__global__ void selftest_wait_kernel(uint64_t budget_ns, unsigned *err) {
-    __shared__ uint64_t bar;
+// Self-test of the bounded wait, on counters of its own: targets that have been reached (also past
+// the wrap of the count) return at once and set nothing; one that stays one ahead runs out of its
+// budget, sets the flag and records the timeout. Only if all of that holds is the timeout passed on
+// to the device error word.
+constexpr int kSelftests = 64;  // calls that may overlap
+static __device__ unsigned g_fem_selftest[kSelftests][3];  // counter, gave up, error bits
+
+__global__ void selftest_wait_kernel(uint64_t budget_ns, int slot, unsigned *err) {
     if (threadIdx.x != 0) return;
-    mbar_init(&bar, 2);
-    fence_barrier_init();
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&bar)) : "memory");
-    if (!mbar_wait_bounded(&bar, 0, budget_ns)) record_device_error(err, FEM_DEVERR_TIMEOUT);
+    unsigned *count = g_fem_selftest[slot], *gave_up = count + 1, *bits = count + 2;
+    atomicExch(count, 5u), atomicExch(gave_up, 0u), atomicExch(bits, 0u);
+    bool ok = wait_reached(count, 5u, budget_ns, gave_up, bits) && wait_reached(count, 0xfffffffau, budget_ns, gave_up, bits);
+    ok = ok && atomicAdd(gave_up, 0u) == 0u && atomicAdd(bits, 0u) == 0u;
+    ok = ok && !wait_reached(count, 6u, budget_ns, gave_up, bits);
+    ok = ok && atomicAdd(gave_up, 0u) == 1u && atomicAdd(bits, 0u) == FEM_DEVERR_TIMEOUT;
+    if (ok) record_device_error(err, FEM_DEVERR_TIMEOUT);
 }
 
 // The float64 kernels' quotient num / |den| (a Newton-Raphson reciprocal, fem_cell.cuh)
@@ -294,7 +301,8 @@ extern "C" fem_status fem_selftest_wait(int64_t budget_ns, fem_stream stream) {
         return fail(FEM_ERR_ARG, "budget_ns must lie in [0, 10 s]");
     unsigned *w = device_error_word();
     if (!w) return fail(FEM_ERR_CUDA, "fem_selftest_wait: device error word unavailable");
-    selftest_wait_kernel<<<1, 32, 0, stream>>>(static_cast<uint64_t>(budget_ns), w);
+    static std::atomic<unsigned> calls{0};
+    selftest_wait_kernel<<<1, 32, 0, stream>>>(static_cast<uint64_t>(budget_ns), static_cast<int>(calls++ % kSelftests), w);
     return check_launch("fem_selftest_wait");
 }
 

@@ -20,6 +20,7 @@
 
 #include "fem_cell.cuh"
 #include "fem_sell.cuh"
+#include "fem_wait.cuh"
 
 namespace fem {
 
@@ -458,29 +459,9 @@ struct CgArgs {
     unsigned *err;
 };
 
-// A bounded wait of one thread until the barrier's counter *p has reached `target`; what the
-// other CTAs wrote before they arrived is visible afterwards. CTAs that wait for one another
-// are resident together (cooperative launch), so the wait ends unless a CTA is lost; after
-// kCgWaitNs it records a timeout and returns false, as the other CTAs' then do.
+// The budget of a wait at the grid's barrier. CTAs that wait for one another are resident
+// together (cooperative launch), so a wait ends unless a CTA is lost.
 constexpr uint64_t kCgWaitNs = 4000000000ull;
-__device__ __forceinline__ bool wait_reached(const unsigned *p, unsigned target, unsigned *gave_up, unsigned *err) {
-    uint64_t t0 = 0, t = 0;
-    unsigned spins = 0;
-    for (;;) {
-        unsigned seen;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(p) : "memory");
-        if (static_cast<int>(seen - target) >= 0) return true;
-        if ((++spins & 255u) == 0u) {
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            if (t0 == 0) t0 = t;
-            if (t - t0 > kCgWaitNs) {
-                atomicExch(gave_up, 1u);
-                record_device_error(err, FEM_DEVERR_TIMEOUT);
-                return false;
-            }
-        }
-    }
-}
 
 // The totals of M pairs per thread over the block (any multiple of 32 threads), in thread 0: warp
 // trees, then one over the warps.
@@ -652,7 +633,7 @@ __global__ void __launch_bounds__(cg_threads<NC>(), 1) sell_cg_kernel(const __gr
     };
     auto barrier_wait = [&](unsigned target) -> bool {
         if (threadIdx.x == 0) {
-            s_ok = wait_reached(bar, target, bar + 1, a.err);
+            s_ok = wait_reached(bar, target, kCgWaitNs, bar + 1, a.err);
         }
         __syncthreads();
         return s_ok != 0;

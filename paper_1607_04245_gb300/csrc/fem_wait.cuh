@@ -1,6 +1,4 @@
-// fem_wait.cuh -- a bounded wait on an mbarrier in shared memory, for the self-test of the
-// timeout path (fem_selftest_wait): a wait that runs out of its %globaltimer budget returns
-// false instead of spinning on.
+// fem_wait.cuh -- the bounded wait of the solves' loop kernel at its grid barrier.
 #pragma once
 
 #include <stdint.h>
@@ -9,44 +7,27 @@
 
 namespace fem {
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-
-// make the barrier initialisation visible to the bulk-copy (async) proxy
-__device__ __forceinline__ void fence_barrier_init() {
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ uint64_t global_timer_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Wait for the phase with the given parity to complete; false when the budget ran out.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint64_t budget_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
-    while (!mbar_try_wait(bar, parity))
-        if (global_timer_ns() - t0 > budget_ns) return false;
-    return true;
+// One thread waits until the counter *p has reached `target` (modulo 2^32); what other CTAs wrote
+// before they raised it is visible afterwards. After budget_ns (%globaltimer, looked at every 256
+// reads) it sets *gave_up, records a timeout in *err and returns false.
+__device__ __forceinline__ bool wait_reached(const unsigned *p, unsigned target, uint64_t budget_ns, unsigned *gave_up,
+                                             unsigned *err) {
+    uint64_t t0 = 0, t = 0;
+    unsigned spins = 0;
+    for (;;) {
+        unsigned seen;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(p) : "memory");
+        if (static_cast<int>(seen - target) >= 0) return true;
+        if ((++spins & 255u) == 0u) {
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            if (t - t0 > budget_ns) {
+                atomicExch(gave_up, 1u);
+                record_device_error(err, FEM_DEVERR_TIMEOUT);
+                return false;
+            }
+        }
+    }
 }
 
 }  // namespace fem
