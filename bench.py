@@ -19,7 +19,7 @@ ranks.
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--rows all|none|PREFIX,...] [--no-cpu-baseline]
 
-Rank 0 prints one JSON line. With N > 1 (torchrun), every rank integrates its own
+Rank 0 prints one JSON line, its rows in short, and every row whole on stderr. With N > 1 (torchrun), every rank integrates its own
 copy of the workload (independent problems, no data-path collective): weak scaling.
 """
 
@@ -1462,9 +1462,42 @@ def run_ours(args):
             "clocks": clocks, "rows": rows,
             "served_p99_ms": rows.get("serving", {}).get("poisson", {}).get("p99_ms"),
             "device_status": device_status}
-    print(json.dumps(line))
+    print_line(line)
     barrier(dist, ws)
     return 0
+
+
+# The JSON line is kept below this: a line of 34 KB (every row with all it measured) was cut by
+# what read it, and its value lost.
+LINE_LIMIT = 8000
+ROW_KEYS = {"ms": ("ms_per_launch", "ms_per_step", "ms_per_solve", "best_ms", "ms"),
+            "frac": ("hbm_frac_of_measured",), "err": ("rel_maxnorm_err_vs_oracle",),
+            "iters": ("iterations", "inner_iterations"), "p50_ms": ("p50_ms",), "p99_ms": ("p99_ms",),
+            "req_per_s": ("req_per_s",), "error": ("error",)}
+
+
+def row_summary(row):
+    """A row's time, rate and error to four digits; rows of several measurements one by one."""
+    out = {}
+    for short, names in ROW_KEYS.items():
+        v = next((row[n] for n in names if row.get(n) is not None), None)
+        if v is not None:
+            out[short] = float(f"{v:.4g}") if isinstance(v, float) else (v[:80] if isinstance(v, str) else v)
+    if "poisson" in row:
+        out = row_summary(row["poisson"])
+    elif not out:
+        out = {k: row_summary(v).get("ms") for k, v in row.items() if isinstance(v, dict)}
+    return out
+
+
+def print_line(line):
+    """The one JSON line, rows in short; the whole rows go to stderr, one line each."""
+    for name, row in line["rows"].items():
+        print(f"bench: row {name} {json.dumps(row)}", file=sys.stderr)
+    text = json.dumps(dict(line, rows={name: row_summary(row) for name, row in line["rows"].items()}))
+    if len(text) > LINE_LIMIT:
+        text = json.dumps(dict(line, rows="see stderr"))
+    print(text)
 
 
 def main(argv=None):
