@@ -813,51 +813,47 @@ __global__ void __launch_bounds__(kBlock, 3) lap_rec_kernel(const __grid_constan
     report_mesh(a.err, vmax, a.V, false);
 }
 
-// host_rows: the cell-indexed rows lie in page-locked host memory and are reached across the
-// host link
+// host4: float64 rows in page-locked host memory, reached across the host link and 16-byte aligned
 template <int DIM, int P, bool ADJ>
-static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_t s, bool host_rows) {
+static fem_status launch_lap(const LapArgs &a, bool pairs, bool host4, cudaStream_t s) {
     constexpr const char *kName = ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian";
     // the quadrature size of the workloads' rules (3 points in 2D, 4 in 3D) is compiled in
     const bool native_nq = a.w.nq == DIM + 1;
     if constexpr (P == FEM_FP64) {
+        if constexpr (!ADJ) {
+            if (host4) {
+                // four cells per thread: few wide accesses for the link
+                const int64_t n = (a.C + 3) / 4;
+                if (native_nq) {
+                    auto k = lap_kernel<DIM, P, 4, DIM + 1, ADJ>;
+                    launch_overlapped(k, grid_for(n, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
+                } else {
+                    auto k = lap_kernel<DIM, P, 4, 0, ADJ>;
+                    launch_overlapped(k, grid_for(n, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
+                }
+                return check_launch(kName);
+            }
+        }
         // one cell per thread, 3D 1,572,864 / 200,000 tets: residual 212 -> 191.5 / 40.6 -> 27.2 us,
         // adjoint 301 -> 273 / 60.7 -> 42.6, against a persistent kernel that staged 1024-cell
         // chunks with bulk copies (its last round of chunks left SMs idle: 5.05 chunks a CTA)
-        if (!(host_rows && vec)) {
-            if (native_nq) {
-                auto k = lap_kernel<DIM, P, 1, DIM + 1, ADJ>;
-                launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
-            } else {
-                auto k = lap_kernel<DIM, P, 1, 0, ADJ>;
-                launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
-            }
-            return check_launch(kName);
+        if (native_nq) {
+            auto k = lap_kernel<DIM, P, 1, DIM + 1, ADJ>;
+            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+        } else {
+            auto k = lap_kernel<DIM, P, 1, 0, ADJ>;
+            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
         }
-    } else {
+    } else if (pairs) {
         // the pair kernel; its plain 8-byte loads also serve host rows: from host buffers 0.309
         // against 0.331 ms per step with lap_kernel
-        if (pairs) {
-            if (native_nq) launch_pair<DIM, P, DIM + 1, ADJ, false>(a, s);
-            else launch_pair<DIM, P, 0, ADJ, false>(a, s);
-            return check_launch(kName);
-        }
+        if (native_nq) launch_pair<DIM, P, DIM + 1, ADJ, false>(a, s);
+        else launch_pair<DIM, P, 0, ADJ, false>(a, s);
+    } else if (a.C % 2 != 0 && native_nq) {
         // an odd cell count (every second row starts between 8-byte words): the same pairs from
         // cells 32 apart, single-value accesses (999,999 tets: 23.8 -> 17.0 us, the adjoint 45.7
         // -> 36.7, against one cell per thread; an even count takes 14.8: twice the row accesses)
-        if (a.C % 2 != 0 && native_nq) {
-            launch_pair<DIM, P, DIM + 1, ADJ, true>(a, s);
-            return check_launch(kName);
-        }
-    }
-    if (vec && native_nq) {
-        auto k = lap_kernel<DIM, P, 4, DIM + 1, ADJ>;
-        int grid = grid_for((a.C + 3) / 4, kBlock, reinterpret_cast<const void *>(k));
-        launch_overlapped(k, grid, kBlock, 0, s, a);
-    } else if (vec) {
-        auto k = lap_kernel<DIM, P, 4, 0, ADJ>;
-        int grid = grid_for((a.C + 3) / 4, kBlock, reinterpret_cast<const void *>(k));
-        launch_overlapped(k, grid, kBlock, 0, s, a);
+        launch_pair<DIM, P, DIM + 1, ADJ, true>(a, s);
     } else if (native_nq) {
         // float32 rows misaligned by their base pointers: two cells per thread, 32 apart (10^6
         // tets: 23.4 -> 17.8 us against one cell with the run-time rule, bitwise the same results)
@@ -872,25 +868,24 @@ static fem_status launch_lap(const LapArgs &a, bool vec, bool pairs, cudaStream_
     return check_launch(kName);
 }
 
-// vec: every cell-indexed row 16-byte aligned (C % 4 == 0); the pair kernel needs 8 bytes
+// the pair kernel needs 8-byte aligned rows; host4: see launch_lap
 template <bool ADJ>
-static fem_status dispatch_lap(int dim, fem_precision prec, const LapArgs &args, bool vec, cudaStream_t s,
-                               bool host_rows = false) {
+static fem_status dispatch_lap(int dim, fem_precision prec, const LapArgs &args, cudaStream_t s, bool host4 = false) {
     LapArgs a = args;
     if (!(a.err = device_error_word())) return fail(FEM_ERR_CUDA, "device error word unavailable");
     const bool pairs = a.C % 2 == 0 && aligned8(a.conn) && aligned8(a.K) && aligned8(a.out) &&
                        (!ADJ || (aligned8(a.lam) && aligned8(a.dK)));
     if (dim == 2) {
         switch (prec) {
-            case FEM_FP64: return launch_lap<2, FEM_FP64, ADJ>(a, vec, pairs, s, host_rows);
-            case FEM_FP32_MIXED: return launch_lap<2, FEM_FP32_MIXED, ADJ>(a, vec, pairs, s, host_rows);
-            case FEM_FP32: return launch_lap<2, FEM_FP32, ADJ>(a, vec, pairs, s, host_rows);
+            case FEM_FP64: return launch_lap<2, FEM_FP64, ADJ>(a, pairs, host4, s);
+            case FEM_FP32_MIXED: return launch_lap<2, FEM_FP32_MIXED, ADJ>(a, pairs, host4, s);
+            case FEM_FP32: return launch_lap<2, FEM_FP32, ADJ>(a, pairs, host4, s);
         }
     } else {
         switch (prec) {
-            case FEM_FP64: return launch_lap<3, FEM_FP64, ADJ>(a, vec, pairs, s, host_rows);
-            case FEM_FP32_MIXED: return launch_lap<3, FEM_FP32_MIXED, ADJ>(a, vec, pairs, s, host_rows);
-            case FEM_FP32: return launch_lap<3, FEM_FP32, ADJ>(a, vec, pairs, s, host_rows);
+            case FEM_FP64: return launch_lap<3, FEM_FP64, ADJ>(a, pairs, host4, s);
+            case FEM_FP32_MIXED: return launch_lap<3, FEM_FP32_MIXED, ADJ>(a, pairs, host4, s);
+            case FEM_FP32: return launch_lap<3, FEM_FP32, ADJ>(a, pairs, host4, s);
         }
     }
     return fail(FEM_ERR_ARG, "unknown precision %d", static_cast<int>(prec));
@@ -947,8 +942,7 @@ extern "C" fem_status fem_integrate_laplacian(int dim, int64_t n_cells, int64_t 
     if (n_cells == 0) return FEM_OK;
     if (!u || !K || !elem_out) return fail(FEM_ERR_ARG, "u, K or elem_out is NULL");
     a.out = elem_out;
-    const bool vec = n_cells % 4 == 0 && aligned16(conn) && aligned16(K) && aligned16(elem_out);
-    return dispatch_lap<false>(dim, prec, a, vec, stream);
+    return dispatch_lap<false>(dim, prec, a, stream);
 }
 
 extern "C" fem_status fem_integrate_laplacian_fields(int dim, int64_t n_cells, int64_t n_verts,
@@ -990,8 +984,8 @@ fem_status integrate_laplacian_plain(int dim, int64_t n_cells, int64_t n_verts, 
     fem_status st = fill_args(a, dim, n_cells, n_verts, coords, conn, u, K, n_q, qpts, qw, prec);
     if (st != FEM_OK || n_cells == 0) return st;
     a.out = elem_out;
-    const bool vec = n_cells % 4 == 0 && aligned16(conn) && aligned16(K) && aligned16(elem_out);
-    return dispatch_lap<false>(dim, prec, a, vec, stream, true);
+    const bool host4 = n_cells % 4 == 0 && aligned16(conn) && aligned16(K) && aligned16(elem_out);
+    return dispatch_lap<false>(dim, prec, a, stream, host4);
 }
 
 fem_status launch_gather(int dim, int n_comp, int64_t C, int64_t V, const void *elem, const int32_t *node_ptr,
@@ -1024,9 +1018,7 @@ extern "C" fem_status fem_adjoint_laplacian(int dim, int64_t n_cells, int64_t n_
         a.lam = lambda;
         a.out = scratch;
         a.dK = dK;
-        const bool vec = n_cells % 4 == 0 && aligned16(conn) && aligned16(K) && aligned16(lambda) &&
-                         aligned16(dK) && aligned16(scratch);
-        if ((st = dispatch_lap<true>(dim, prec, a, vec, stream)) != FEM_OK) return st;
+        if ((st = dispatch_lap<true>(dim, prec, a, stream)) != FEM_OK) return st;
     }
     return launch_gather(dim, 1, n_cells, n_verts, scratch, node_ptr, node_idx, du, prec, stream);
 }
