@@ -163,8 +163,7 @@ __device__ __forceinline__ void lap_cell(const double (&xs)[DIM + 1][DIM],
 // Direct kernel: one thread owns CPT consecutive cells (or, STR, 32 apart) and reads the
 // cell-indexed rows with (vector) loads from global memory. The float64 form's kernel, with one
 // cell per thread; in the float32 forms, used where the pair kernel does not apply (rows
-// misaligned by their base pointers, odd counts with other rules); and, with four cells, for
-// float64 rows in page-locked host memory.
+// misaligned by their base pointers, odd counts with other rules).
 template <int DIM, int P, int CPT, int NQ, bool ADJ, bool STR = false>
 __global__ void __launch_bounds__(kBlock) lap_kernel(const __grid_constant__ LapArgs a) {
     pdl_wait();  // overlapped launch: the previous kernel's writes are visible from here
@@ -813,36 +812,27 @@ __global__ void __launch_bounds__(kBlock, 3) lap_rec_kernel(const __grid_constan
     report_mesh(a.err, vmax, a.V, false);
 }
 
-// host4: float64 rows in page-locked host memory, reached across the host link and 16-byte aligned
+// host_rows: the cell-indexed rows lie in page-locked host memory and are reached across the
+// host link
 template <int DIM, int P, bool ADJ>
-static fem_status launch_lap(const LapArgs &a, bool pairs, bool host4, cudaStream_t s) {
+static fem_status launch_lap(const LapArgs &a, bool pairs, bool host_rows, cudaStream_t s) {
     constexpr const char *kName = ADJ ? "fem_adjoint_laplacian" : "fem_integrate_laplacian";
     // the quadrature size of the workloads' rules (3 points in 2D, 4 in 3D) is compiled in
     const bool native_nq = a.w.nq == DIM + 1;
     if constexpr (P == FEM_FP64) {
-        if constexpr (!ADJ) {
-            if (host4) {
-                // four cells per thread: few wide accesses for the link
-                const int64_t n = (a.C + 3) / 4;
-                if (native_nq) {
-                    auto k = lap_kernel<DIM, P, 4, DIM + 1, ADJ>;
-                    launch_overlapped(k, grid_for(n, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
-                } else {
-                    auto k = lap_kernel<DIM, P, 4, 0, ADJ>;
-                    launch_overlapped(k, grid_for(n, kBlock, reinterpret_cast<const void *>(k)), kBlock, 0, s, a);
-                }
-                return check_launch(kName);
-            }
-        }
         // one cell per thread, 3D 1,572,864 / 200,000 tets: residual 212 -> 191.5 / 40.6 -> 27.2 us,
         // adjoint 301 -> 273 / 60.7 -> 42.6, against a persistent kernel that staged 1024-cell
-        // chunks with bulk copies (its last round of chunks left SMs idle: 5.05 chunks a CTA)
+        // chunks with bulk copies (its last round of chunks left SMs idle: 5.05 chunks a CTA).
+        // Rows in page-locked host memory in CTAs of two warps: 1,000,000 / 999,999 / 50,001 tets 306 /
+        // 346 / 35.0 us (one warp 306 / 356 / 35.5; four cells per thread, aligned rows only, 435)
+        const unsigned cta = host_rows ? 2 * kWarpCta : kWarpCta;
+        const unsigned grid = static_cast<unsigned>((a.C + cta - 1) / cta);
         if (native_nq) {
             auto k = lap_kernel<DIM, P, 1, DIM + 1, ADJ>;
-            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+            launch_overlapped(k, grid, cta, 0, s, a);
         } else {
             auto k = lap_kernel<DIM, P, 1, 0, ADJ>;
-            launch_overlapped(k, warp_ctas(a.C), kWarpCta, 0, s, a);
+            launch_overlapped(k, grid, cta, 0, s, a);
         }
     } else if (pairs) {
         // the pair kernel; its plain 8-byte loads also serve host rows: from host buffers 0.309
@@ -868,24 +858,25 @@ static fem_status launch_lap(const LapArgs &a, bool pairs, bool host4, cudaStrea
     return check_launch(kName);
 }
 
-// the pair kernel needs 8-byte aligned rows; host4: see launch_lap
+// the pair kernel needs 8-byte aligned rows
 template <bool ADJ>
-static fem_status dispatch_lap(int dim, fem_precision prec, const LapArgs &args, cudaStream_t s, bool host4 = false) {
+static fem_status dispatch_lap(int dim, fem_precision prec, const LapArgs &args, cudaStream_t s,
+                               bool host_rows = false) {
     LapArgs a = args;
     if (!(a.err = device_error_word())) return fail(FEM_ERR_CUDA, "device error word unavailable");
     const bool pairs = a.C % 2 == 0 && aligned8(a.conn) && aligned8(a.K) && aligned8(a.out) &&
                        (!ADJ || (aligned8(a.lam) && aligned8(a.dK)));
     if (dim == 2) {
         switch (prec) {
-            case FEM_FP64: return launch_lap<2, FEM_FP64, ADJ>(a, pairs, host4, s);
-            case FEM_FP32_MIXED: return launch_lap<2, FEM_FP32_MIXED, ADJ>(a, pairs, host4, s);
-            case FEM_FP32: return launch_lap<2, FEM_FP32, ADJ>(a, pairs, host4, s);
+            case FEM_FP64: return launch_lap<2, FEM_FP64, ADJ>(a, pairs, host_rows, s);
+            case FEM_FP32_MIXED: return launch_lap<2, FEM_FP32_MIXED, ADJ>(a, pairs, host_rows, s);
+            case FEM_FP32: return launch_lap<2, FEM_FP32, ADJ>(a, pairs, host_rows, s);
         }
     } else {
         switch (prec) {
-            case FEM_FP64: return launch_lap<3, FEM_FP64, ADJ>(a, pairs, host4, s);
-            case FEM_FP32_MIXED: return launch_lap<3, FEM_FP32_MIXED, ADJ>(a, pairs, host4, s);
-            case FEM_FP32: return launch_lap<3, FEM_FP32, ADJ>(a, pairs, host4, s);
+            case FEM_FP64: return launch_lap<3, FEM_FP64, ADJ>(a, pairs, host_rows, s);
+            case FEM_FP32_MIXED: return launch_lap<3, FEM_FP32_MIXED, ADJ>(a, pairs, host_rows, s);
+            case FEM_FP32: return launch_lap<3, FEM_FP32, ADJ>(a, pairs, host_rows, s);
         }
     }
     return fail(FEM_ERR_ARG, "unknown precision %d", static_cast<int>(prec));
@@ -984,8 +975,7 @@ fem_status integrate_laplacian_plain(int dim, int64_t n_cells, int64_t n_verts, 
     fem_status st = fill_args(a, dim, n_cells, n_verts, coords, conn, u, K, n_q, qpts, qw, prec);
     if (st != FEM_OK || n_cells == 0) return st;
     a.out = elem_out;
-    const bool host4 = n_cells % 4 == 0 && aligned16(conn) && aligned16(K) && aligned16(elem_out);
-    return dispatch_lap<false>(dim, prec, a, stream, host4);
+    return dispatch_lap<false>(dim, prec, a, stream, true);
 }
 
 fem_status launch_gather(int dim, int n_comp, int64_t C, int64_t V, const void *elem, const int32_t *node_ptr,
