@@ -205,7 +205,9 @@ __global__ void __launch_bounds__(kBlock) fill_kernel(const int32_t *conn, int64
 // instructions per warp and 82 % of the issue slots (lists of 1,000,000 tets 51.9 -> 44.9 us,
 // 200,000: 20.1 -> 19.1; 2D, with 6 entries, would lose 0.5 %). Other lists of up to kSortShared
 // entries go to shared memory, where an entry's place is the number of smaller ones (all entries of
-// a list are distinct). Longer ones: insertion sort in place by one lane.
+// a list are distinct). Longer ones are sorted in place by the eight lanes with bitonic merges (lists
+// of meshes of hubs, us, by insertion sort of one lane -> so: 5000 of 129 entries 861 -> 159, 2000 of
+// 400 4708 -> 236, 500 of 1000 19,510 -> 353; by a thread per vertex they took 677, 3500, 19,490).
 constexpr int kSortShared = 128;
 
 // 32 values over 8 lanes, four to a lane, into ascending order (entry 4 lane + i in x[i]): bitonic
@@ -264,15 +266,25 @@ __global__ void __launch_bounds__(kBlock) sort_segments_kernel(const int32_t *pt
                 idx[b + r] = x;
             }
             __syncwarp(mask);
-        } else if (lane == 0) {
-            for (int32_t i = b + 1; i < b + m; ++i) {
-                const int32_t x = idx[i];
-                int32_t j = i - 1;
-                while (j >= b && idx[j] > x) {
-                    idx[j + 1] = idx[j];
-                    --j;
+        } else {
+            // in place, by the same merges as sort32's; entries past the end count as the largest,
+            // and no exchange reaches them
+            int32_t *p = idx + b;
+            const uint32_t len = static_cast<uint32_t>(m);
+            auto step = [&](uint32_t d, uint32_t mirror) {
+                for (uint32_t q = lane;; q += G) {
+                    const uint32_t i = 2 * (q & ~(d - 1)) + (q & (d - 1)), j = mirror ? i ^ mirror : i + d;
+                    if (i >= len) break;
+                    if (j < len) {
+                        const int32_t x = p[i], y = p[j];
+                        if (x > y) p[i] = y, p[j] = x;
+                    }
                 }
-                idx[j + 1] = x;
+                __syncwarp(mask);
+            };
+            for (uint64_t k = 2; k / 2 < len; k *= 2) {
+                step(static_cast<uint32_t>(k / 2), static_cast<uint32_t>(k - 1));
+                for (uint32_t d = static_cast<uint32_t>(k / 4); d > 0; d /= 2) step(d, 0u);
             }
         }
     }
