@@ -285,7 +285,8 @@ fem_status fem_integrate_laplacian_transposed(int dim, int64_t n_cells, const vo
  * kernels run before or after it. A smaller workspace is accepted down to what the element form
  * needs ((dim+1) n_cells values, six vectors of n_verts values, 24 KiB and 256 bytes, each
  * rounded up to 256 bytes); the element residuals are then computed and summed in every
- * iteration, as three kernels in a CUDA graph with a WHILE node, at several times the cost.
+ * iteration, as three kernels in a CUDA graph with a WHILE node, at several times the cost. The
+ * two forms' x differ by what float32 rounding leaves of it, and their iteration counts may too.
  * Meshes with a vertex of more than 64 neighbours, more vertex pairs than the workspace
  * provides for (half as many again as a conforming mesh of this size has) or, FEM_FP32_MIXED,
  * cells below the shape threshold, which that form applies in float64, take the element form

@@ -234,11 +234,10 @@ __device__ __forceinline__ bool rd_cell(const RdArgs &a, const double *const (&X
 // Grid-stride over groups of CPT consecutive cells. A_P1: the coefficient field is nodal;
 // DRIFT (P1 only): the grad a term. CPT = 4 with NQ > 0 (the quadrature size fixed at
 // compile time) reads the connectivity, reaction and P0 coefficient rows and writes the
-// element vectors with 16-byte vector accesses; CPT = 1, NQ = 0 is the general form
-// (any n_q, unaligned rows, ragged sizes). Staging the rows through shared memory with the
-// bulk-copy loop of the Laplacian kernel was slower here (37.2 against 33.7 us on the
-// 1,572,864-tet workload): at that kernel's 2 CTAs per SM the register cap spills this
-// element's state.
+// element vectors with 16-byte vector accesses (STR: cells 32 apart, any size and alignment);
+// CPT = 1, NQ = 0 is the general form (any n_q) and float64's. Staging the rows through shared
+// memory with bulk copies was slower here (37.2 against 33.7 us on the 1,572,864-tet workload):
+// at 2 CTAs per SM the register cap spilled this element's state.
 // 3D float32 forms take two cells per thread at 80 registers (3 CTAs of 256 threads per SM):
 // 31.2 us on the 1,572,864-tet workload with reaction and drift, against 33.0 us with four
 // cells at 128 registers (2 CTAs); 64 registers spill, and 2 CTAs of two cells run 39 us.
